@@ -180,7 +180,6 @@ __global__ void __launch_bounds__(WPB * 32, 1) rhs_adjoint1d_kernel(const Adjoin
     const T alpha = p.alpha_ptr ? T(*p.alpha_ptr) : T(__longlong_as_double((long long)p.ctl->amax[p.slot_in][0]));
     const T sc = T(p.scale);
     const T gm1 = T(p.gamma - 1.0), eps = T(p.eps), CT = T(p.CT), dxT = T(p.dx);
-    const T kt = keep_all_factor(CT);
     const T *U = static_cast<const T *>(p.U);
     const T *V = static_cast<const T *>(p.v);
     T *out = static_cast<T *>(p.out);
@@ -244,8 +243,16 @@ __global__ void __launch_bounds__(WPB * 32, 1) rhs_adjoint1d_kernel(const Adjoin
                 qm[k][t] = sm;
             }
             if (!p.masks) {  // recorded masks make the cutoff unnecessary
-                word |= cutoff_bits(qp[k][1], qp[k][2], qp[k][3], qp[k][4], qp[k][5], eps, CT, kt) << (3 * k);
-                word |= cutoff_bits(qm[k][5], qm[k][4], qm[k][3], qm[k][2], qm[k][1], eps, CT, kt) << (3 * (3 + k));
+                if constexpr (sizeof(T) == 8) {
+                    const Cut64 cut = cut64(eps, CT, p.kt);
+                    word |= cutoff_bits(qp[k][1], qp[k][2], qp[k][3], qp[k][4], qp[k][5], cut) << (3 * k);
+                    word |= cutoff_bits(qm[k][5], qm[k][4], qm[k][3], qm[k][2], qm[k][1], cut) << (3 * (3 + k));
+                } else {
+                    const float kt = p.f_kt;
+                    word |= cutoff_bits(qp[k][1], qp[k][2], qp[k][3], qp[k][4], qp[k][5], eps, CT, kt) << (3 * k);
+                    word |= cutoff_bits(qm[k][5], qm[k][4], qm[k][3], qm[k][2], qm[k][1], eps, CT, kt)
+                            << (3 * (3 + k));
+                }
             }
         }
         const unsigned wl = __shfl_up_sync(0xffffffffu, word, 1);
@@ -385,7 +392,7 @@ cudaError_t launch_rhs_adjoint1d(const Adjoint1D &p, cudaStream_t st) {
     const int nw = warps_per_cta(ntiles, true);
     int grid = (ntiles + nw - 1) / nw;
     if (grid > num_sms() * 4 * (WPB / nw)) grid = num_sms() * 4 * (WPB / nw);
-    rhs_adjoint1d_kernel<T><<<grid, nw * 32, 0, st>>>(p);
+    rhs_adjoint1d_kernel<T><<<grid, nw * 32, 0, st>>>(with_kt(p));
     return cudaGetLastError();
 }
 

@@ -17,5 +17,7 @@ struct Adjoint1D {
     int slot_in;               // alpha of U (frozen) ...
     const double *alpha_ptr;   // ... or, if not null, read from here
     double scale;              // out += scale (dL/dU)^T v
+    double kt;                 // keep_all_factor(CT), set by the launcher
+    float f_kt;
 };
 }  // namespace t7

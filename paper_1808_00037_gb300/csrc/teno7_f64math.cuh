@@ -1,0 +1,196 @@
+// teno7_f64math.cuh -- the parts of the FP64 path that need not run on the FP64
+// pipe.
+//
+// GB300 issues one FP64 warp instruction per SM every 19 cycles (measured: add,
+// multiply, FMA and compare alike, whatever the active lanes; 64 cycles from a
+// single warp), while the FP32 and integer pipes take 2 to 4 per cycle.  So an
+// FP64 instruction is worth some 40 integer or FP32 ones, and every decision
+// that FP32 can take with a proven error bound is taken there, the FP64
+// evaluation remaining for the windows the bound leaves open.  The decided
+// bits are the FP64 evaluation's own.
+//
+// Host-compilable (T7_HD), so that the functions can be checked without a GPU.
+#pragma once
+#include <math.h>
+#include <stdint.h>
+#include <string.h>
+
+#ifdef __CUDACC__
+#define T7_HD __host__ __device__ __forceinline__
+#else
+#define T7_HD inline
+#endif
+
+namespace t7 {
+
+T7_HD uint64_t f64_bits(double x) {
+#ifdef __CUDA_ARCH__
+    return (uint64_t)__double_as_longlong(x);
+#else
+    uint64_t b;
+    memcpy(&b, &x, 8);
+    return b;
+#endif
+}
+T7_HD double f64_of(uint64_t b) {
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)b);
+#else
+    double x;
+    memcpy(&x, &b, 8);
+    return x;
+#endif
+}
+T7_HD float f32_of(uint32_t b) {
+#ifdef __CUDA_ARCH__
+    return __uint_as_float(b);
+#else
+    float x;
+    memcpy(&x, &b, 4);
+    return x;
+#endif
+}
+T7_HD float f32_rcp(float x) {  // approximate reciprocal, within 2 ulp
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    return 1.0f / x;
+#endif
+}
+
+// --------------------------------------------------------------------------
+// Shortcut of the cutoff test.  If tau < kt (beta_min + eps), every
+// g_k = 1 + tau / (beta_k + eps) lies in [1, 1 + kt), so
+// chi_k = g_k^6 / sum_j g_j^6 >= 1 / (3 (1 + kt)^6).  With
+// 1 + kt = 0.9 (3 C_T)^(-1/6) that bound is C_T / 0.9^6 = 1.88 C_T: every
+// stencil is kept, and the divisions and powers need not be evaluated.  The
+// 10% margin in g (1.9x in chi) is far above the rounding of either
+// precision, so the bits are exactly the ones the full evaluation gives.
+// kt = 0 (the shortcut never applies) when C_T >= 1/3.  Host functions: the
+// launchers evaluate kt once (in the kernels an FP64 pow per thread cost more
+// than the whole scalar stage at 200 cells).
+// --------------------------------------------------------------------------
+inline double keep_all_factor(double CT) {
+    return (CT > 0.0 && CT < 1.0 / 3.0) ? 0.9 * pow(3.0 * CT, -1.0 / 6.0) - 1.0 : 0.0;
+}
+inline float keep_all_factor(float CT) {
+    return (CT > 0.f && CT < 1.f / 3.f) ? 0.9f * powf(3.f * CT, -1.f / 6.f) - 1.f : 0.f;
+}
+
+// Parameters of the FP64 cutoff test: epsilon, C_T and kt, and their FP32 forms
+// (4 epsilon; C_T, or 0 where FP32 cannot hold it and only kept windows are
+// decided there).
+struct Cut64 {
+    double eps, CT, kt;
+    float e4, ktf, ctf;
+};
+T7_HD Cut64 cut64(double eps, double CT, double kt) {
+    Cut64 K;
+    K.eps = eps;
+    K.CT = CT;
+    K.kt = kt;
+    K.e4 = (float)(4.0 * eps);
+    K.ktf = (float)kt;
+    K.ctf = CT > 1e-30 ? (float)CT : 0.f;
+    return K;
+}
+
+// Five-point smoothness measure and cutoff bits (d0 | d1<<1 | d2<<2) of one
+// window w0..w4 = f_{i-2} .. f_{i+2} in upwind order, in FP64 (Eqs.
+// smooth_expl, tau5, TENO1 with C = 1 and q = 6, norm, seclect).
+T7_HD unsigned cutoff_bits_f64(double w0, double w1, double w2, double w3, double w4, double eps, double CT,
+                               double kt) {
+    // Eq. smooth_expl
+    double s0a = w0 - 4.0 * w1 + 3.0 * w2;
+    double s0b = w0 - 2.0 * w1 + w2;
+    double s2a = 3.0 * w2 - 4.0 * w3 + w4;
+    double s2b = w2 - 2.0 * w3 + w4;
+    double b0 = 0.25 * (s0a * s0a) + (13.0 / 12.0) * (s0b * s0b);
+    double b2 = 0.25 * (s2a * s2a) + (13.0 / 12.0) * (s2b * s2b);
+    // Eq. tau5, Eq. TENO1 with C = 1, q = 6 (squared, squared again, times square)
+    double tau = fabs(b0 - b2);
+    // every stencil kept (see keep_all_factor); beta_min >= 0, so tau < kt eps
+    // already suffices and beta_1 is not needed
+    if (tau < kt * eps) return 7u;
+    double s1a = w1 - w3;
+    double s1b = w1 - 2.0 * w2 + w3;
+    double b1 = 0.25 * (s1a * s1a) + (13.0 / 12.0) * (s1b * s1b);
+    if (tau < kt * (fmin(fmin(b0, b1), b2) + eps)) return 7u;
+    double g0 = 1.0 + tau / (b0 + eps);
+    double g1 = 1.0 + tau / (b1 + eps);
+    double g2 = 1.0 + tau / (b2 + eps);
+    double q0 = g0 * g0, q1 = g1 * g1, q2 = g2 * g2;
+    double y0 = (q0 * q0) * q0, y1 = (q1 * q1) * q1, y2 = (q2 * q2) * q2;
+    // Eqs. norm, seclect: delta = 0 iff chi < C_T
+    double S = (y0 + y1) + y2;
+    unsigned d0 = (y0 / S < CT) ? 0u : 1u;
+    unsigned d1 = (y1 / S < CT) ? 0u : 1u;
+    unsigned d2 = (y2 / S < CT) ? 0u : 1u;
+    return d0 | (d1 << 1) | (d2 << 2);
+}
+
+// x = h + l + r with h the leading 24 bits of x (truncated), l the next 23 and
+// |r| < 2^-46 |x|, by integer operations on x's bits and two FP32 operations.
+// |x| < 2^-126 gives 0; a magnitude of 2^126 and more, infinities and NaN give
+// an infinite h.
+T7_HD void split_f32(double x, float &h, float &l) {
+    const uint64_t b = f64_bits(x);
+    const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
+    const uint32_t a = hi & 0x7fffffffu, sign = hi & 0x80000000u;
+    const uint32_t t = a - 0x38000000u;  // exponent rebiased
+    uint32_t f = (t << 3) | (lo >> 29);
+    if (t - 0x00100000u >= 0x0fc00000u) f = a < 0x38100000u ? 0u : 0x7f800000u;
+    h = f32_of(f | sign);
+    const float m = f32_of(0x4b000000u | ((lo >> 6) & 0x7fffffu)) - 8388608.f;  // bits 28..6 as an integer
+    l = m * (f32_of((f & 0x7f800000u) | sign) * 1.4210854715202004e-14f);       // times 2^(e-46)
+}
+
+// The same bits as cutoff_bits_f64, decided in FP32 where its error bound
+// allows it.  The window enters through its four first differences, each
+// d_t = (h_{t+1} - h_t) + (l_{t+1} - l_t) within 2^-23 |d_t| + 2^-44 max|w|; the
+// measures are linear in them, so each beta (times 4: s^2 + 13/3 r^2) is known
+// within 2.2e-6 of itself plus A = 2^-60 max|w|^2 (1e-36 covers underflow).
+//   kept     tau + 1e-5 (beta_0 + beta_2) + A < kt (0.9999 (beta_min + eps) - A)
+//            implies tau < kt (beta_min + eps): all bits set (keep_all_factor).
+//   decided  where tau > 0.01 (beta_0 + beta_2) and A is below 1e-5 of the
+//            smallest beta + eps, g_k is known within 2.5e-4 and chi_k / C_T
+//            within 1%: the FP32 comparison holds unless chi_k is within 3% of
+//            C_T.
+// Everything else, and what FP32 cannot hold, goes to the FP64 evaluation.
+T7_HD unsigned cutoff_bits(double w0, double w1, double w2, double w3, double w4, const Cut64 &K) {
+    float h0, h1, h2, h3, h4, l0, l1, l2, l3, l4;
+    split_f32(w0, h0, l0);
+    split_f32(w1, h1, l1);
+    split_f32(w2, h2, l2);
+    split_f32(w3, h3, l3);
+    split_f32(w4, h4, l4);
+    const float d1 = (h1 - h0) + (l1 - l0), d2 = (h2 - h1) + (l2 - l1);
+    const float d3 = (h3 - h2) + (l3 - l2), d4 = (h4 - h3) + (l4 - l3);
+    const float c = 13.f / 3.f;
+    const float s0a = fmaf(3.f, d2, -d1), s0b = d2 - d1, s2a = fmaf(-3.f, d3, d4), s2b = d4 - d3;
+    const float s1a = d2 + d3, s1b = d3 - d2;
+    const float b0 = fmaf(c * s0b, s0b, s0a * s0a), b1 = fmaf(c * s1b, s1b, s1a * s1a);
+    const float b2 = fmaf(c * s2b, s2b, s2a * s2a);
+    const float W = fmaxf(fmaxf(fmaxf(fabsf(h0), fabsf(h1)), fmaxf(fabsf(h2), fabsf(h3))), fabsf(h4));
+    const float A = fmaf(W * W, 8.673617379884035e-19f, 1e-36f);
+    const float sum = b0 + b2, tau = fabsf(b0 - b2), bm = fminf(fminf(b0, b1), b2) + K.e4;
+    if (fmaf(1e-5f, sum, tau) + A < K.ktf * fmaf(0.9999f, bm, -A)) return 7u;
+    if (K.ctf > 0.f && tau > 0.01f * sum && A < 1e-5f * bm) {
+        const float g0 = fmaf(tau, f32_rcp(b0 + K.e4), 1.f), g1 = fmaf(tau, f32_rcp(b1 + K.e4), 1.f);
+        const float g2 = fmaf(tau, f32_rcp(b2 + K.e4), 1.f);
+        const float gm = fmaxf(fmaxf(g0, g1), g2), rg = f32_rcp(gm);
+        float x0 = g0 * rg, x1 = g1 * rg, x2 = g2 * rg;
+        x0 *= x0;
+        x1 *= x1;
+        x2 *= x2;
+        const float y0 = x0 * x0 * x0, y1 = x1 * x1 * x1, y2 = x2 * x2 * x2;
+        const float thr = K.ctf * ((y0 + y1) + y2), band = 0.03f * thr;
+        if (gm < 1e37f && fabsf(y0 - thr) > band && fabsf(y1 - thr) > band && fabsf(y2 - thr) > band)
+            return (y0 < thr ? 0u : 1u) | ((y1 < thr ? 0u : 1u) << 1) | ((y2 < thr ? 0u : 1u) << 2);
+    }
+    return cutoff_bits_f64(w0, w1, w2, w3, w4, K.eps, K.CT, K.kt);
+}
+
+}  // namespace t7

@@ -60,6 +60,8 @@ struct Stage1D {
     int halo;
     const double *alpha_in;  // nullable: alpha of Us from this device value instead of the control block
     int alpha_mode;          // t7_alpha_mode: 1 = one alpha per characteristic field (1D Euler)
+    double kt;               // keep_all_factor(CT), set by the launchers (here and below)
+    float f_kt;
 };
 
 // Ghost cells per side of a slab (the stencil reach of the scheme, Eq. app:
@@ -103,6 +105,8 @@ struct Stage2D {
     int halo;
     const double *alpha_in;  // nullable: [2] alpha_x, alpha_y of Us instead of the control block's
     double *alpha_rec;       // nullable: receives [2] alpha_x, alpha_y of the output (RK mode)
+    double kt;
+    float f_kt;
 };
 
 struct Alpha2D {
@@ -149,6 +153,8 @@ struct Batch1D {
     int *steps_out;            // device, per tube
     double *t_out;             // device, per tube
     DevCtl *ctl;               // error word
+    double kt;
+    float f_kt;
 };
 
 cudaError_t launch_batch1d_f64(const Batch1D &p, cudaStream_t s);
@@ -185,6 +191,8 @@ struct Recon {
     int n, sign;
     double eps, CT;
     DevCtl *ctl;
+    double kt;
+    float f_kt;
 };
 
 cudaError_t launch_stage1d_f64(const Stage1D &p, cudaStream_t s);

@@ -44,6 +44,7 @@
 
 #include <mutex>
 
+#include "teno7_f64math.cuh"
 #include "teno7_internal.h"
 
 namespace t7 {
@@ -74,95 +75,59 @@ __device__ __forceinline__ int pack_delta(unsigned dm, unsigned d0, unsigned dp)
                  ((dp >> 2) & 1u));
 }
 
-// Table co2, coefficients on f_{i-3} .. f_{i+3}; each FP64 entry is the nearest
-// double to the printed rational (FP32: that double rounded to float).
+// Table co2, coefficients on f_{i-3} .. f_{i+3} (rows of seven), and Table co1,
+// the TENO5 rows on f_{i-2} .. f_{i+2} (rows of five); each FP64 entry is the
+// nearest double to the printed rational (FP32: that double rounded to float).
+// In device memory: the lanes that copy them to shared memory read different
+// entries.
+// clang-format off
+#define T7_TABLE_CO2(T) \
+    T(-1.0/140.0), T(5.0/84.0), T(-101.0/420.0), T(319.0/420.0), T(107.0/210.0), T(-19.0/210.0), T(1.0/105.0), \
+    T(0), T(1.0/60.0), T(-2.0/15.0), T(37.0/60.0), T(37.0/60.0), T(-2.0/15.0), T(1.0/60.0), \
+    T(-1.0/60.0), T(7.0/60.0), T(-23.0/60.0), T(19.0/20.0), T(11.0/30.0), T(-1.0/30.0), T(0), \
+    T(0), T(0), T(-1.0/20.0), T(9.0/20.0), T(47.0/60.0), T(-13.0/60.0), T(1.0/30.0), \
+    T(0), T(1.0/30.0), T(-13.0/60.0), T(47.0/60.0), T(9.0/20.0), T(-1.0/20.0), T(0), \
+    T(-1.0/20.0), T(17.0/60.0), T(-43.0/60.0), T(77.0/60.0), T(1.0/5.0), T(0), T(0), \
+    T(0), T(0), T(0), T(1.0/4.0), T(13.0/12.0), T(-5.0/12.0), T(1.0/12.0), \
+    T(0), T(0), T(-1.0/12.0), T(7.0/12.0), T(7.0/12.0), T(-1.0/12.0), T(0), \
+    T(0), T(1.0/12.0), T(-5.0/12.0), T(13.0/12.0), T(1.0/4.0), T(0), T(0), \
+    T(-1.0/4.0), T(13.0/12.0), T(-23.0/12.0), T(25.0/12.0), T(0), T(0), T(0), \
+    T(0), T(0), T(0), T(1.0/3.0), T(5.0/6.0), T(-1.0/6.0), T(0), \
+    T(0), T(0), T(-1.0/6.0), T(5.0/6.0), T(1.0/3.0), T(0), T(0), \
+    T(0), T(1.0/3.0), T(-7.0/6.0), T(11.0/6.0), T(0), T(0), T(0)
+#define T7_TABLE_CO1(T) \
+    T(1.0/30.0), T(-13.0/60.0), T(47.0/60.0), T(9.0/20.0), T(-1.0/20.0), \
+    T(0), T(-1.0/9.0), T(2.0/3.0), T(1.0/2.0), T(-1.0/18.0), \
+    T(1.0/21.0), T(-13.0/42.0), T(41.0/42.0), T(2.0/7.0), T(0), \
+    T(0), T(0), T(1.0/3.0), T(5.0/6.0), T(-1.0/6.0), \
+    T(0), T(-1.0/6.0), T(5.0/6.0), T(1.0/3.0), T(0), \
+    T(1.0/3.0), T(-7.0/6.0), T(11.0/6.0), T(0), T(0), \
+    T(1.0/12.0), T(-7.0/24.0), T(17.0/24.0), T(5.0/8.0), T(-1.0/8.0)
+// clang-format on
+static __device__ const double CO2_F64[91] = {T7_TABLE_CO2(double)};
+static __device__ const float CO2_F32[91] = {T7_TABLE_CO2(float)};
+static __device__ const double CO1_F64[35] = {T7_TABLE_CO1(double)};
+static __device__ const float CO1_F32[35] = {T7_TABLE_CO1(float)};
+
 template <typename T>
 __device__ __forceinline__ T coef(int idx) {
-    switch (idx) {
-        // clang-format off
-        case 0: return T(-1.0/140.0); case 1: return T(5.0/84.0); case 2: return T(-101.0/420.0); case 3: return T(319.0/420.0);
-        case 4: return T(107.0/210.0); case 5: return T(-19.0/210.0); case 6: return T(1.0/105.0);
-        case 7: return T(0); case 8: return T(1.0/60.0); case 9: return T(-2.0/15.0); case 10: return T(37.0/60.0);
-        case 11: return T(37.0/60.0); case 12: return T(-2.0/15.0); case 13: return T(1.0/60.0);
-        case 14: return T(-1.0/60.0); case 15: return T(7.0/60.0); case 16: return T(-23.0/60.0); case 17: return T(19.0/20.0);
-        case 18: return T(11.0/30.0); case 19: return T(-1.0/30.0); case 20: return T(0);
-        case 21: return T(0); case 22: return T(0); case 23: return T(-1.0/20.0); case 24: return T(9.0/20.0);
-        case 25: return T(47.0/60.0); case 26: return T(-13.0/60.0); case 27: return T(1.0/30.0);
-        case 28: return T(0); case 29: return T(1.0/30.0); case 30: return T(-13.0/60.0); case 31: return T(47.0/60.0);
-        case 32: return T(9.0/20.0); case 33: return T(-1.0/20.0); case 34: return T(0);
-        case 35: return T(-1.0/20.0); case 36: return T(17.0/60.0); case 37: return T(-43.0/60.0); case 38: return T(77.0/60.0);
-        case 39: return T(1.0/5.0); case 40: return T(0); case 41: return T(0);
-        case 42: return T(0); case 43: return T(0); case 44: return T(0); case 45: return T(1.0/4.0);
-        case 46: return T(13.0/12.0); case 47: return T(-5.0/12.0); case 48: return T(1.0/12.0);
-        case 49: return T(0); case 50: return T(0); case 51: return T(-1.0/12.0); case 52: return T(7.0/12.0);
-        case 53: return T(7.0/12.0); case 54: return T(-1.0/12.0); case 55: return T(0);
-        case 56: return T(0); case 57: return T(1.0/12.0); case 58: return T(-5.0/12.0); case 59: return T(13.0/12.0);
-        case 60: return T(1.0/4.0); case 61: return T(0); case 62: return T(0);
-        case 63: return T(-1.0/4.0); case 64: return T(13.0/12.0); case 65: return T(-23.0/12.0); case 66: return T(25.0/12.0);
-        case 67: return T(0); case 68: return T(0); case 69: return T(0);
-        case 70: return T(0); case 71: return T(0); case 72: return T(0); case 73: return T(1.0/3.0);
-        case 74: return T(5.0/6.0); case 75: return T(-1.0/6.0); case 76: return T(0);
-        case 77: return T(0); case 78: return T(0); case 79: return T(-1.0/6.0); case 80: return T(5.0/6.0);
-        case 81: return T(1.0/3.0); case 82: return T(0); case 83: return T(0);
-        case 84: return T(0); case 85: return T(1.0/3.0); case 86: return T(-7.0/6.0); case 87: return T(11.0/6.0);
-        case 88: return T(0); case 89: return T(0); case 90: return T(0);
-        default: return T(0);
-        // clang-format on
+    if constexpr (sizeof(T) == 8) {
+        return CO2_F64[idx];
+    } else {
+        return CO2_F32[idx];
     }
 }
 
-// --------------------------------------------------------------------------
-// Shortcut of the cutoff test.  If tau < kt (beta_min + eps), every
-// g_k = 1 + tau / (beta_k + eps) lies in [1, 1 + kt), so
-// chi_k = g_k^6 / sum_j g_j^6 >= 1 / (3 (1 + kt)^6).  With
-// 1 + kt = 0.9 (3 C_T)^(-1/6) that bound is C_T / 0.9^6 = 1.88 C_T: every
-// stencil is kept, and the divisions and powers need not be evaluated.  The
-// 10% margin in g (1.9x in chi) is far above the rounding of either
-// precision, so the bits are exactly the ones the full evaluation gives.
-// kt = 0 (the shortcut never applies) when C_T >= 1/3.
-// --------------------------------------------------------------------------
-__device__ __forceinline__ double keep_all_factor(double CT) {
-    return (CT > 0.0 && CT < 1.0 / 3.0) ? 0.9 * pow(3.0 * CT, -1.0 / 6.0) - 1.0 : 0.0;
-}
-__device__ __forceinline__ float keep_all_factor(float CT) {
+// keep_all_factor of the FP32 1D tiles, evaluated in the kernel: with kt taken
+// from the launch parameters instead, the compiler if-converts the cutoff's slow
+// path and the 16.8M-cell stage executes 29% more instructions (1.06 -> 1.34 ms
+// per step); the powf costs a launch about a microsecond.
+__device__ __forceinline__ float keep_all_factor_device(float CT) {
     return (CT > 0.f && CT < 1.f / 3.f) ? 0.9f * powf(3.f * CT, -1.f / 6.f) - 1.f : 0.f;
 }
 
-// --------------------------------------------------------------------------
-// Five-point smoothness measure and cutoff bits (d0 | d1<<1 | d2<<2) of one
-// window w0..w4 = f_{i-2} .. f_{i+2} in upwind order; kt from keep_all_factor.
-// --------------------------------------------------------------------------
-__device__ __forceinline__ unsigned cutoff_bits(double w0, double w1, double w2, double w3, double w4, double eps,
-                                                double CT, double kt) {
-    // Eq. smooth_expl
-    double s0a = w0 - 4.0 * w1 + 3.0 * w2;
-    double s0b = w0 - 2.0 * w1 + w2;
-    double s2a = 3.0 * w2 - 4.0 * w3 + w4;
-    double s2b = w2 - 2.0 * w3 + w4;
-    double b0 = 0.25 * (s0a * s0a) + (13.0 / 12.0) * (s0b * s0b);
-    double b2 = 0.25 * (s2a * s2a) + (13.0 / 12.0) * (s2b * s2b);
-    // Eq. tau5, Eq. TENO1 with C = 1, q = 6 (squared, squared again, times square)
-    double tau = fabs(b0 - b2);
-    // every stencil kept (see keep_all_factor); beta_min >= 0, so tau < kt eps
-    // already suffices and beta_1 is not needed
-    if (tau < kt * eps) return 7u;
-    double s1a = w1 - w3;
-    double s1b = w1 - 2.0 * w2 + w3;
-    double b1 = 0.25 * (s1a * s1a) + (13.0 / 12.0) * (s1b * s1b);
-    if (tau < kt * (fmin(fmin(b0, b1), b2) + eps)) return 7u;
-    double g0 = 1.0 + tau / (b0 + eps);
-    double g1 = 1.0 + tau / (b1 + eps);
-    double g2 = 1.0 + tau / (b2 + eps);
-    double q0 = g0 * g0, q1 = g1 * g1, q2 = g2 * g2;
-    double y0 = (q0 * q0) * q0, y1 = (q1 * q1) * q1, y2 = (q2 * q2) * q2;
-    // Eqs. norm, seclect: delta = 0 iff chi < C_T
-    double S = (y0 + y1) + y2;
-    unsigned d0 = (y0 / S < CT) ? 0u : 1u;
-    unsigned d1 = (y1 / S < CT) ? 0u : 1u;
-    unsigned d2 = (y2 / S < CT) ? 0u : 1u;
-    return d0 | (d1 << 1) | (d2 << 2);
-}
-
+// Cutoff bits of one FP32 window (the FP64 form: cutoff_bits in
+// teno7_f64math.cuh); kt from keep_all_factor.
 __device__ __forceinline__ unsigned cutoff_bits(float w0, float w1, float w2, float w3, float w4, float eps,
                                                 float CT, float kt) {
     float s0a = fmaf(3.f, w2, fmaf(-4.f, w1, w0));
@@ -361,21 +326,12 @@ enum { SCH_TENO7EXT = 0, SCH_TENO5 = 1 };
 constexpr unsigned SEL5 = 0x01632457u;
 __device__ __forceinline__ int sel5(unsigned code) { return (int)((SEL5 >> (4 * (code & 7u))) & 15u); }
 
-// Table co1 coefficients, row-major [7][5]; FP64 entries are the nearest
-// doubles to the printed rationals.
 template <typename T>
 __device__ __forceinline__ T coef5(int idx) {
-    switch (idx) {
-        // clang-format off
-        case 0: return T(1.0/30.0); case 1: return T(-13.0/60.0); case 2: return T(47.0/60.0); case 3: return T(9.0/20.0); case 4: return T(-1.0/20.0);
-        case 5: return T(0); case 6: return T(-1.0/9.0); case 7: return T(2.0/3.0); case 8: return T(1.0/2.0); case 9: return T(-1.0/18.0);
-        case 10: return T(1.0/21.0); case 11: return T(-13.0/42.0); case 12: return T(41.0/42.0); case 13: return T(2.0/7.0); case 14: return T(0);
-        case 15: return T(0); case 16: return T(0); case 17: return T(1.0/3.0); case 18: return T(5.0/6.0); case 19: return T(-1.0/6.0);
-        case 20: return T(0); case 21: return T(-1.0/6.0); case 22: return T(5.0/6.0); case 23: return T(1.0/3.0); case 24: return T(0);
-        case 25: return T(1.0/3.0); case 26: return T(-7.0/6.0); case 27: return T(11.0/6.0); case 28: return T(0); case 29: return T(0);
-        case 30: return T(1.0/12.0); case 31: return T(-7.0/24.0); case 32: return T(17.0/24.0); case 33: return T(5.0/8.0); case 34: return T(-1.0/8.0);
-        default: return T(0);
-        // clang-format on
+    if constexpr (sizeof(T) == 8) {
+        return CO1_F64[idx];
+    } else {
+        return CO1_F32[idx];
     }
 }
 
@@ -467,7 +423,7 @@ struct TileArgs {
     int bc_lo, bc_hi;
     double dx;
     float f_dx;
-    T alpha, dtT, gamma, gm1, a, eps, CT;
+    T alpha, dtT, gamma, gm1, a, eps, CT, kt;
     T alf[3];        // per-field alphas (1D Euler, the per-field alpha mode)
     double dtD;      // FP64 step (mixed precision: FP64 state, FP32 reconstruction)
     int rhs_mode, stage;
@@ -503,7 +459,7 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
     const size_t cs = A.cs;
     const int ntiles = min((n + WT - 1) / WT, tile_end);  // tiles tile0, tile0 + tstride, ... below it
     const T alpha = A.alpha, dtT = A.dtT, gamma = A.gamma, gm1 = A.gm1, a = A.a, eps = A.eps, CT = A.CT;
-    const T kt = keep_all_factor(CT);
+    const Cut64 cut = cut64(eps, CT, A.kt);
     DevCtl *ctl = A.ctl;
     T wsmax = T(0);
     for (int tile = tile0; tile < ntiles; tile += tstride) {
@@ -645,8 +601,8 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
                     qm[k][t] = sm;
                 }
             }
-            const unsigned bp = cutoff_bits(qp[k][1], qp[k][2], qp[k][3], qp[k][4], qp[k][5], eps, CT, kt);
-            const unsigned bm = cutoff_bits(qm[k][5], qm[k][4], qm[k][3], qm[k][2], qm[k][1], eps, CT, kt);
+            const unsigned bp = cutoff_bits(qp[k][1], qp[k][2], qp[k][3], qp[k][4], qp[k][5], cut);
+            const unsigned bm = cutoff_bits(qm[k][5], qm[k][4], qm[k][3], qm[k][2], qm[k][1], cut);
             word |= bp << (3 * k);
             word |= bm << (3 * (M + k));
         }
@@ -835,6 +791,7 @@ __global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 ? 2 : 1)) stage1d_ke
     A.a = pick<T>(p.a, p.f_a);
     A.eps = pick<T>(p.eps, p.f_eps);
     A.CT = pick<T>(p.CT, p.f_CT);
+    A.kt = pick<T>(p.kt, p.f_kt);
     A.rhs_mode = p.rhs_mode;
     A.stage = p.stage;
     A.ebase = 0;
@@ -1168,7 +1125,7 @@ __device__ __forceinline__ float tiles1d_f32(const TileArgs<float> &A, float (*s
     // (TENO5's epsilon of 1e-40 is below FLT_MIN: raise it to FLT_MIN so that
     // beta + eps is never flushed to zero by the approximate reciprocal)
     const float eps4 = SCH == SCH_TENO5 ? fmaxf(4.f * A.eps, 1.17549435e-38f) : 4.f * A.eps, CT = A.CT;
-    const float kt = keep_all_factor(CT);
+    const float kt = keep_all_factor_device(CT);
     const float idx = 1.f / A.f_dx;
     const S *Us = reinterpret_cast<const S *>(A.Us);
     const S *U0 = reinterpret_cast<const S *>(A.U0);
@@ -1587,7 +1544,7 @@ __device__ __forceinline__ float tiles1d_f32_fp(const TileArgs<float> &A, float2
     const int lane = threadIdx.x & 31;
     const float alpha = A.alpha, dtT = A.dtT, gamma = A.gamma, gm1 = A.gm1, a = A.a;
     const float eps4 = SCH == SCH_TENO5 ? fmaxf(4.f * A.eps, 1.17549435e-38f) : 4.f * A.eps, CT = A.CT;
-    const float kt = keep_all_factor(CT);
+    const float kt = keep_all_factor_device(CT);
     const float idx = 1.f / A.f_dx;
     const float *Us = A.Us;
     const float *U0 = A.U0;
@@ -2158,7 +2115,6 @@ __global__ void __launch_bounds__(NT) recon_kernel(const Recon p) {
     const int s = blockIdx.x * TILE;
     const T *v = static_cast<const T *>(p.v);
     const T eps = T(p.eps), CT = T(p.CT);
-    const T kt = keep_all_factor(CT);
     for (int q = tid; q < 91; q += NT) s_coef[q] = coef<T>(q);
     for (int c = tid; c < NCELL; c += NT) {
         int l = s - HALO + c + 4;  // index into v (cell -4 is v[0])
@@ -2168,10 +2124,12 @@ __global__ void __launch_bounds__(NT) recon_kernel(const Recon p) {
     __syncthreads();
     const int j = s - 2 + tid;
     unsigned bits;
-    if (p.sign > 0)
-        bits = cutoff_bits(s_v[tid + 1], s_v[tid + 2], s_v[tid + 3], s_v[tid + 4], s_v[tid + 5], eps, CT, kt);
+    const T *w = s_v + (p.sign > 0 ? tid + 1 : tid + 6);
+    const int dir = p.sign > 0 ? 1 : -1;
+    if constexpr (sizeof(T) == 8)
+        bits = cutoff_bits(w[0], w[dir], w[2 * dir], w[3 * dir], w[4 * dir], cut64(eps, CT, p.kt));
     else
-        bits = cutoff_bits(s_v[tid + 6], s_v[tid + 5], s_v[tid + 4], s_v[tid + 3], s_v[tid + 2], eps, CT, kt);
+        bits = cutoff_bits(w[0], w[dir], w[2 * dir], w[3 * dir], w[4 * dir], eps, CT, p.f_kt);
     s_bits[tid] = bits;
     if (p.d3 && j >= -2 && j <= n) p.d3[j + 2] = (uint8_t)bits;
     __syncthreads();
@@ -2204,6 +2162,14 @@ __global__ void __launch_bounds__(NT) recon_kernel(const Recon p) {
 }
 
 // ---------------------------------------------------------------- launchers --
+// p with the factor of the cutoff shortcut of its C_T
+template <typename P>
+inline P with_kt(P p) {
+    p.kt = keep_all_factor(p.CT);
+    p.f_kt = keep_all_factor((float)p.CT);
+    return p;
+}
+
 inline int num_sms() {
     static int sms = 0;
     if (!sms) {
@@ -2281,7 +2247,8 @@ inline int stage_grid(Stage1DKernel k, int nctas, int threads, int waves) {
 
 // FP32 paired-split stage kernels; S = float (FP32 state) or double (mixed).
 template <typename S>
-cudaError_t launch_stage1d_paired(const Stage1D &p, cudaStream_t st) {
+cudaError_t launch_stage1d_paired(const Stage1D &p_, cudaStream_t st) {
+    const Stage1D p = with_kt(p_);
     const int ntiles = stage_tiles(p);
     if (ntiles < 1) return cudaErrorInvalidValue;
     const int nw = warps_per_cta(ntiles, false);
@@ -2342,10 +2309,11 @@ cudaError_t launch_stage1d_paired(const Stage1D &p, cudaStream_t st) {
 }
 
 template <typename T>
-cudaError_t launch_stage1d(const Stage1D &p, cudaStream_t st) {
+cudaError_t launch_stage1d(const Stage1D &p_, cudaStream_t st) {
     if constexpr (sizeof(T) == 4) {
-        return launch_stage1d_paired<float>(p, st);
+        return launch_stage1d_paired<float>(p_, st);
     } else {
+        const Stage1D p = with_kt(p_);
         const int ntiles = stage_tiles(p);
         if (ntiles < 1) return cudaErrorInvalidValue;
         const int nw = warps_per_cta(ntiles, true);
@@ -2399,7 +2367,7 @@ cudaError_t launch_alpha1d(const Alpha1D &p, cudaStream_t st) {
 template <typename T>
 cudaError_t launch_recon(const Recon &p, cudaStream_t st) {
     const int grid = (p.n + TILE - 1) / TILE;
-    recon_kernel<T><<<grid, NT, 0, st>>>(p);
+    recon_kernel<T><<<grid, NT, 0, st>>>(with_kt(p));
     return cudaGetLastError();
 }
 
@@ -2497,6 +2465,7 @@ __global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 ? 2 : 1)) batch1d_ke
         A.a = T(0);
         A.eps = T((dx * dx) * dx);
         A.CT = T(p.CT);
+        A.kt = pick<T>(p.kt, p.f_kt);
         A.rhs_mode = 0;
         A.ebase = (int)off;
         A.halo = 0;
@@ -2616,7 +2585,7 @@ cudaError_t launch_batch1d(const Batch1D &p, cudaStream_t st) {
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch1d_kernel<T>, WPB * 32, 0);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
-    batch1d_kernel<T><<<num_sms() * per_sm, WPB * 32, 0, st>>>(p);
+    batch1d_kernel<T><<<num_sms() * per_sm, WPB * 32, 0, st>>>(with_kt(p));
     return cudaGetLastError();
 }
 

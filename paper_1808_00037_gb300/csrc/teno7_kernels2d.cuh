@@ -50,7 +50,7 @@ __device__ __forceinline__ constexpr int rot(int c) {
 // gp(c, t) / gm(c, t): physical component c of the split fluxes of local cell
 // t; local cell t = 0 .. 7 is cell j-3+t of face j+1/2.
 template <typename T, int DIR, typename PR, typename GP, typename GM>
-__device__ __forceinline__ void face2d_bits(Face2D<T> &F, PR pr, GP gp, GM gm, T gm1, T eps, T CT, T kt) {
+__device__ __forceinline__ void face2d_bits(Face2D<T> &F, PR pr, GP gp, GM gm, T gm1, const Cut64 &cut) {
     const T unl = pr(0, 3), unr = pr(0, 4), utl = pr(1, 3), utr = pr(1, 4);
     const T Hl = pr(2, 3), Hr = pr(2, 4), sl = pr(3, 3), sr = pr(3, 4);
     F.un = (sl * unl + sr * unr) / (sl + sr);
@@ -86,8 +86,8 @@ __device__ __forceinline__ void face2d_bits(Face2D<T> &F, PR pr, GP gp, GM gm, T
             F.qp[k][t] = sp;
             F.qm[k][t] = sm;
         }
-        const unsigned bp = cutoff_bits(F.qp[k][1], F.qp[k][2], F.qp[k][3], F.qp[k][4], F.qp[k][5], eps, CT, kt);
-        const unsigned bm = cutoff_bits(F.qm[k][5], F.qm[k][4], F.qm[k][3], F.qm[k][2], F.qm[k][1], eps, CT, kt);
+        const unsigned bp = cutoff_bits(F.qp[k][1], F.qp[k][2], F.qp[k][3], F.qp[k][4], F.qp[k][5], cut);
+        const unsigned bm = cutoff_bits(F.qm[k][5], F.qm[k][4], F.qm[k][3], F.qm[k][2], F.qm[k][1], cut);
         F.word |= bp << (3 * k);
         F.word |= bm << (3 * (4 + k));
     }
@@ -269,8 +269,7 @@ __global__ void __launch_bounds__(WPB * 32, 1) xsweep2d_kernel(const Stage2D p) 
     for (int q = lane; q < 91; q += 32) s_coef[warp][q] = coef<T>(q);
     const T alpha = alpha2d_in<T, HALO>(p, ctl, 0);
     const T gm1 = pick<T>(p.gamma - 1.0, p.f_gm1);
-    const T eps = pick<T>(p.eps_x, p.f_eps_x), CT = pick<T>(p.CT, p.f_CT);
-    const T kt = keep_all_factor(CT);
+    const Cut64 cut = cut64(p.eps_x, p.CT, p.kt);
     const T *Us = static_cast<const T *>(p.Us);
     T *R = static_cast<T *>(p.R);
     const int nx = p.nx, ny = p.ny;
@@ -306,7 +305,7 @@ __global__ void __launch_bounds__(WPB * 32, 1) xsweep2d_kernel(const Stage2D p) 
         Face2D<T> F;
         face2d_bits<T, 0>(
             F, [&](int q, int t) { return spr[q][lane + t]; }, [&](int c, int t) { return sgp[c][lane + t]; },
-            [&](int c, int t) { return sgm[c][lane + t]; }, gm1, eps, CT, kt);
+            [&](int c, int t) { return sgm[c][lane + t]; }, gm1, cut);
         const unsigned wl = __shfl_up_sync(0xffffffffu, F.word, 1);
         const unsigned wr = __shfl_down_sync(0xffffffffu, F.word, 1);
         T fh[4];
@@ -374,8 +373,7 @@ __global__ void __launch_bounds__(WPB * 32, 1) ysweep2d_kernel(const Stage2D p) 
     const int x0 = blockIdx.x * YB_COLS, r0 = blockIdx.y * YB_ROWS;
     const T alpha = alpha2d_in<T, HALO>(p, ctl, 1);
     const T gamma = pick<T>(p.gamma, p.f_gamma), gm1 = pick<T>(p.gamma - 1.0, p.f_gm1);
-    const T eps = pick<T>(p.eps_y, p.f_eps_y), CT = pick<T>(p.CT, p.f_CT);
-    const T kt = keep_all_factor(CT);
+    const Cut64 cut = cut64(p.eps_y, p.CT, p.kt);
     const T *Us = static_cast<const T *>(p.Us);
     for (int q = tid; q < 91; q += blockDim.x) s_coef[q] = coef<T>(q);
 
@@ -407,7 +405,7 @@ __global__ void __launch_bounds__(WPB * 32, 1) ysweep2d_kernel(const Stage2D p) 
         face2d_bits<T, 1>(
             F, [&](int q, int t) { return at(s_pr, q, lane + t, col); },
             [&](int c, int t) { return at(s_gp, c, lane + t, col); },
-            [&](int c, int t) { return at(s_gm, c, lane + t, col); }, gm1, eps, CT, kt);
+            [&](int c, int t) { return at(s_gm, c, lane + t, col); }, gm1, cut);
         const unsigned wl = __shfl_up_sync(0xffffffffu, F.word, 1);
         const unsigned wr = __shfl_down_sync(0xffffffffu, F.word, 1);
         T fh[4];
@@ -711,7 +709,7 @@ __global__ void __launch_bounds__(WPB * 32, 2) xsweep2d_f32_kernel(const Stage2D
     fill_delta_table(s_cf);
     const float alpha = alpha2d_in<float, HALO>(p, ctl, 0);
     const float gm1 = p.f_gm1, eps4 = 4.f * p.f_eps_x, CT = p.f_CT;
-    const float kt = keep_all_factor(CT);
+    const float kt = p.f_kt;
     const float idx = 1.f / p.f_dx;
     const double idxD = 1.0 / p.dx;
     const S *Us = static_cast<const S *>(p.Us);
@@ -846,7 +844,7 @@ __global__ void __launch_bounds__(WPB * 32, 2) ysweep2d_f32_kernel(const Stage2D
     const int x0 = blockIdx.x * YB_COLS, r0 = blockIdx.y * YB_ROWS;
     const float alpha = alpha2d_in<float, HALO>(p, ctl, 1);
     const float gamma = p.f_gamma, gm1 = p.f_gm1, eps4 = 4.f * p.f_eps_y, CT = p.f_CT;
-    const float kt = keep_all_factor(CT);
+    const float kt = p.f_kt;
     const S *Us = static_cast<const S *>(p.Us);
     fill_delta_table(s_cf);
 
@@ -1217,7 +1215,7 @@ __global__ void __launch_bounds__(WPB * 32, 2) xsweep2d_f32fp_kernel(const Stage
     fill_delta_table(s_cf);
     const float alpha = alpha2d_in<float, HALO>(p, ctl, 0);
     const float gm1 = p.f_gm1, eps4 = 4.f * p.f_eps_x, CT = p.f_CT;
-    const float kt = keep_all_factor(CT);
+    const float kt = p.f_kt;
     const float idx = 1.f / p.f_dx;
     const float *Us = static_cast<const float *>(p.Us);
     float *R = static_cast<float *>(p.R);
@@ -1371,7 +1369,7 @@ __global__ void __launch_bounds__(WPB * 32, 2) ysweep2d_f32p_kernel(const Stage2
     const int nbx = (nx + YB_COLS - 1) / YB_COLS, nblocks = nbx * ((ny + YB_ROWS - 1) / YB_ROWS);
     const float alpha = alpha2d_in<float, HALO>(p, ctl, 1);
     const float gamma = p.f_gamma, gm1 = p.f_gm1, eps4 = 4.f * p.f_eps_y, CT = p.f_CT;
-    const float kt = keep_all_factor(CT);
+    const float kt = p.f_kt;
     const float *Us = static_cast<const float *>(p.Us);
     const float *R = static_cast<const float *>(p.R);
     const float *U0 = static_cast<const float *>(p.U0);
@@ -1540,7 +1538,8 @@ __global__ void __launch_bounds__(WPB * 32, 2) ysweep2d_f32p_kernel(const Stage2
 }
 
 template <typename S, bool HALO = false>
-cudaError_t launch_stage2d_paired(const Stage2D &p, cudaStream_t st) {
+cudaError_t launch_stage2d_paired(const Stage2D &p_, cudaStream_t st) {
+    const Stage2D p = with_kt(p_);
     const int ntx = (p.nx + WT - 1) / WT;
     long ntiles = (long)ntx * p.ny;
     long gx = (ntiles + WPB - 1) / WPB;
@@ -1579,10 +1578,11 @@ cudaError_t launch_stage2d_paired(const Stage2D &p, cudaStream_t st) {
 }
 
 template <typename T, bool HALO = false>
-cudaError_t launch_stage2d(const Stage2D &p, cudaStream_t st) {
+cudaError_t launch_stage2d(const Stage2D &p_, cudaStream_t st) {
     if constexpr (sizeof(T) == 4) {
-        return launch_stage2d_paired<float, HALO>(p, st);
+        return launch_stage2d_paired<float, HALO>(p_, st);
     } else {
+    const Stage2D p = with_kt(p_);
     const int ntx = (p.nx + WT - 1) / WT;
     long ntiles = (long)ntx * p.ny;
     long gx = (ntiles + WPB - 1) / WPB;

@@ -1,0 +1,58 @@
+// Host check of teno7_f64math.cuh: the FP32-decided cutoff bits against the
+// FP64 evaluation.  Prints "<what> <cases> <differences>" per line.
+#include <cstdio>
+#include <random>
+
+#include "teno7_f64math.cuh"
+
+using namespace t7;
+
+static void check_cutoff() {
+    std::mt19937_64 r(3);
+    std::uniform_real_distribution<double> u(-1, 1);
+    long bad = 0, total = 0;
+    for (double CT : {1e-5, 1e-7, 1e-3, 0.2, 0.5, 1e-300})
+        for (double eps : {1e-60, 1e-40, 1e-18, 1e-12, 2.4e-7, 1e-3}) {
+            const double kt = keep_all_factor(CT);
+            const Cut64 K = cut64(eps, CT, kt);
+            for (int i = 0; i < 40000; i++) {
+                const double base = u(r) * pow(10, u(r) * 3), amp = pow(10, u(r) * 8 - 8 + (i % 3) * 4);
+                const double d0 = u(r), d1 = u(r), d2 = u(r);
+                double w[5];
+                for (int t = 0; t < 5; t++) {
+                    const double x = t - 2;
+                    switch (i % 7) {
+                        case 0: w[t] = base + amp * u(r); break;                                         // noise
+                        case 1: w[t] = base + amp * (d0 * x + 0.1 * d1 * x * x + 0.01 * d2 * x * x * x); break;  // smooth
+                        case 2: w[t] = base + (t > 2 ? amp * d0 : 0) + 1e-3 * amp * u(r); break;         // jumps
+                        case 3: w[t] = base + (t > 1 ? amp * d0 : 0) + 1e-9 * amp * u(r); break;
+                        case 4: w[t] = base; break;                                                      // constant
+                        case 5: w[t] = base + amp * u(r) * (t == 2); break;                              // a spike
+                        default: w[t] = amp * (t > 2 ? d0 * x * x : d1 * x) * (i % 2 ? 1 : 1e-20); break;  // a kink
+                    }
+                }
+                total++;
+                bad += cutoff_bits(w[0], w[1], w[2], w[3], w[4], K) !=
+                       cutoff_bits_f64(w[0], w[1], w[2], w[3], w[4], eps, CT, kt);
+            }
+        }
+    printf("cutoff %ld %ld\n", total, bad);
+    // zeros, subnormals, magnitudes beyond FP32, infinities and NaN in every place
+    const double s[] = {0.0, -0.0, 1e-310, 1e-40, 1e-20, 1.0, 1e20, 1e60, 1e300, INFINITY, NAN};
+    const Cut64 K = cut64(2.4e-7, 1e-5, keep_all_factor(1e-5));
+    total = bad = 0;
+    for (double a : s)
+        for (double b : s)
+            for (double c : s)
+                for (double d : s)
+                    for (double e : s) {
+                        total++;
+                        bad += cutoff_bits(a, b, c, d, e, K) != cutoff_bits_f64(a, b, c, d, e, K.eps, K.CT, K.kt);
+                    }
+    printf("cutoff_special %ld %ld\n", total, bad);
+}
+
+int main() {
+    check_cutoff();
+    return 0;
+}
