@@ -50,6 +50,17 @@ T7_HD float f32_of(uint32_t b) {
     return x;
 #endif
 }
+// Tests and maxima that would otherwise be FP64-pipe comparisons.
+T7_HD bool f64_finite(double x) { return ((uint32_t)(f64_bits(x) >> 32) & 0x7fffffffu) < 0x7ff00000u; }
+T7_HD bool f64_positive(double x) {  // x > 0 (false for NaN)
+    const uint64_t b = f64_bits(x);
+    return b - 1u < 0x7ff0000000000000ull;
+}
+// fmax of a non-negative x (not NaN) and a non-negative y or NaN
+T7_HD double f64_max_pos(double x, double y) {
+    const uint64_t bx = f64_bits(x), by = f64_bits(y);
+    return f64_of(by > bx && by <= 0x7ff0000000000000ull ? by : bx);
+}
 T7_HD float f32_rcp(float x) {  // approximate reciprocal, within 2 ulp
 #ifdef __CUDA_ARCH__
     float r;

@@ -238,6 +238,18 @@ __device__ __forceinline__ T warp_max(T v) {
 
 // Largest characteristic speed of one cell (1D systems) and its validity.
 // FP64 follows the oracle's expression order; FP32 uses fast reciprocals.
+template <typename T>
+__device__ __forceinline__ int cell_flag1d(const T *Uc, T p) {
+    // a non-finite cell is reported as such; a finite one needs rho > 0, p > 0
+    if constexpr (sizeof(T) == 8) {
+        if (!f64_finite(Uc[0]) || !f64_finite(Uc[1]) || !f64_finite(Uc[2])) return ERR_NONFINITE;
+        return f64_positive(Uc[0]) && f64_positive(p) ? 0 : ERR_NONPHYSICAL;
+    } else {
+        if (!isfinite(Uc[0]) || !isfinite(Uc[1]) || !isfinite(Uc[2])) return ERR_NONFINITE;
+        return (Uc[0] > T(0)) && (p > T(0)) ? 0 : ERR_NONPHYSICAL;
+    }
+}
+
 template <typename T, int SYS>
 __device__ __forceinline__ T wavespeed1d(const T *Uc, T gm1, T gamma, T a, int *flag) {
     if (SYS == SYS_ADV) return absval(a);
@@ -248,7 +260,7 @@ __device__ __forceinline__ T wavespeed1d(const T *Uc, T gm1, T gamma, T a, int *
     T u, p, c;
     if constexpr (sizeof(T) == 8) {
         u = Uc[1] / Uc[0];
-        p = gm1 * (Uc[2] - T(0.5) * Uc[1] * u);
+        p = gm1 * __fma_rn(-0.5, Uc[1] * u, Uc[2]);  // U2 - (U1/2) u, the half exact
         c = sq_root(gamma * p / Uc[0]);
     } else {
         const float ri = __frcp_rn(Uc[0]);
@@ -256,11 +268,7 @@ __device__ __forceinline__ T wavespeed1d(const T *Uc, T gm1, T gamma, T a, int *
         p = gm1 * (Uc[2] - 0.5f * Uc[1] * u);
         c = __fsqrt_rn(gamma * p * ri);
     }
-    // a non-finite cell is reported as such; a finite one needs rho > 0, p > 0
-    if (!isfinite(Uc[0]) || !isfinite(Uc[1]) || !isfinite(Uc[2]))
-        *flag |= ERR_NONFINITE;
-    else if (!(Uc[0] > T(0)) || !(p > T(0)))
-        *flag |= ERR_NONPHYSICAL;
+    *flag |= cell_flag1d<T>(Uc, p);
     return absval(u) + c;
 }
 
@@ -272,7 +280,7 @@ __device__ __forceinline__ void wavespeeds1d(const T *Uc, T gm1, T gamma, T w[3]
     T u, p, c;
     if constexpr (sizeof(T) == 8) {
         u = Uc[1] / Uc[0];
-        p = gm1 * (Uc[2] - T(0.5) * Uc[1] * u);
+        p = gm1 * __fma_rn(-0.5, Uc[1] * u, Uc[2]);
         c = sq_root(gamma * p / Uc[0]);
     } else {
         const float ri = __frcp_rn(Uc[0]);
@@ -280,10 +288,7 @@ __device__ __forceinline__ void wavespeeds1d(const T *Uc, T gm1, T gamma, T w[3]
         p = gm1 * (Uc[2] - 0.5f * Uc[1] * u);
         c = __fsqrt_rn(gamma * p * ri);
     }
-    if (!isfinite(Uc[0]) || !isfinite(Uc[1]) || !isfinite(Uc[2]))
-        *flag |= ERR_NONFINITE;
-    else if (!(Uc[0] > T(0)) || !(p > T(0)))
-        *flag |= ERR_NONPHYSICAL;
+    *flag |= cell_flag1d<T>(Uc, p);
     w[0] = absval(u - c);
     w[1] = absval(u);
     w[2] = absval(u + c);
@@ -440,17 +445,104 @@ __device__ __forceinline__ int ghost_or_halo(int l, int n, int bc_lo, int bc_hi,
     return ghost_map(l, n, bc_lo, bc_hi);
 }
 
+// --------------------------------------------------------------------------
+// FP64 arithmetic of one cell and one face, 1D Euler.  Every value is the
+// oracle's, rounding by rounding, up to a power of two that the next step takes
+// back: 2 G+- = F +- alpha U is staged without its half, the rows of L of
+// fields u -+ c are kept without theirs, so the characteristic values of those
+// fields carry a factor 4 and the others 2 (epsilon is scaled alike), and the
+// face flux a factor 4 that the division by 4 dx removes.  A remaining exact
+// factor (1/2, 1/4, 2) rides in an FMA, whose product is exact.  Powers of two
+// commute with rounding, so no bit changes (values within a factor 16 of the
+// subnormal range or of overflow aside).  The third products of the three
+// fields are one, b1 g2.  Against the expressions written plainly this takes 13
+// instead of 15 FP64 instructions per projected cell and split, 15 instead of
+// 20 per staged cell and 16 instead of 31 per frame (divisions and roots apart).
+// --------------------------------------------------------------------------
+constexpr int FLUX_SCALE_EULER = 4, FLUX_SCALE_SCALAR = 2;
+
+// Flux F, velocity u, total enthalpy H and sqrt(rho) of a state.
+__device__ __forceinline__ void cell1d_f64(const double U[3], double gm1, double F[3], double pr[3]) {
+    const double u = U[1] / U[0];
+    const double m = U[1] * u;
+    const double p = gm1 * __fma_rn(-0.5, m, U[2]);
+    const double e = U[2] + p;
+    F[0] = U[1];
+    F[1] = m + p;
+    F[2] = u * e;
+    pr[0] = u;
+    pr[1] = e / U[0];
+    pr[2] = sqrt(U[0]);
+}
+
+// Roe frame of a face: rows 0 and 2 of L doubled (l0, l2; their third entry is
+// b1, and row 1's is -b1), the Roe state, and X = u~^2.
+struct Roe64 {
+    double l0[2], l1[2], l2[2], b1, ut, cc, Ht, X;
+    int flag;
+};
+__device__ __forceinline__ Roe64 roe_frame_f64(double ul, double ur, double Hl, double Hr, double sl, double sr,
+                                               double gm1) {
+    Roe64 R;
+    const double S = sl + sr;
+    R.ut = (sl * ul + sr * ur) / S;
+    R.Ht = (sl * Hl + sr * Hr) / S;
+    R.X = R.ut * R.ut;
+    const double c2 = gm1 * __fma_rn(-0.5, R.X, R.Ht);
+    R.cc = sqrt(c2);
+    R.b1 = gm1 / c2;
+    const double t = R.X * R.b1;  // 2 b2
+    const double uc = R.ut / R.cc, rc = 1.0 / R.cc;
+    const double b1u = R.b1 * R.ut;
+    R.l0[0] = __fma_rn(0.5, t, uc);
+    R.l0[1] = -(b1u + rc);
+    R.l1[0] = __fma_rn(-0.5, t, 1.0);
+    R.l1[1] = b1u;
+    R.l2[0] = __fma_rn(0.5, t, -uc);
+    R.l2[1] = -(b1u - rc);
+    R.flag = f64_positive(c2) ? 0 : (f64_finite(c2) ? ERR_NONPHYSICAL : ERR_NONFINITE);
+    return R;
+}
+
+// L g (rows 0 and 2 doubled).
+__device__ __forceinline__ void project_f64(const Roe64 &R, double g0, double g1, double g2, double q[3]) {
+    const double p = R.b1 * g2;
+    q[0] = (R.l0[0] * g0 + R.l0[1] * g1) + p;
+    q[1] = (R.l1[0] * g0 + R.l1[1] * g1) - p;
+    q[2] = (R.l2[0] * g0 + R.l2[1] * g1) + p;
+}
+
+// R f for f[0], f[2] scaled by 4 and f[1] by 2: the face flux scaled by 4.
+__device__ __forceinline__ void back_project_f64(const Roe64 &R, const double f[3], double fh[3]) {
+    const double w = R.ut * R.cc;
+    fh[0] = __fma_rn(2.0, f[1], f[0]) + f[2];
+    fh[1] = __fma_rn(2.0, R.ut * f[1], (R.ut - R.cc) * f[0]) + (R.ut + R.cc) * f[2];
+    fh[2] = ((R.Ht - w) * f[0] + R.X * f[1]) + (R.Ht + w) * f[2];
+}
+
+// Shu-Osher combination of RK stage k (v = us + dt r; U^n = u0).
+__device__ __forceinline__ double rk_combine_f64(int stage, double us, double dt, double r, double u0) {
+    const double v = us + dt * r;
+    if (stage == 0) return v;
+    if (stage == 1) return __fma_rn(0.25, v, 0.75 * u0);
+    return (1.0 / 3.0) * u0 + (2.0 / 3.0) * v;
+}
+
 // PF (1D Euler, TENO7-ext): per-field alphas A.alf -- each field's split values
 // (L_k F +- alf[k] L_k U) / 2 from the staged flux (sgp) and state (sU), in the
 // oracle's operation order; ws3 receives the output's three characteristic
 // speed maxima (the function then returns 0).
+//
+// Bound by the FP64 pipe (one warp instruction per 19 cycles and SM, against 2
+// to 4 per cycle for the others): the two splits run through one loop body, each
+// as seven upwind-ordered taps, and a split whose staged fluxes are all zero
+// (advection: F - alpha U for a > 0) is not reconstructed.
 template <typename T, int SYS, int SCH = SCH_TENO7EXT, bool PF = false>
 __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)[WC], T (*sgm)[WC], T (*spr)[WC],
                                      const T *scoef, int tile0, int tstride, int tile_end = 0x7fffffff,
                                      T *ws3 = nullptr) {
+    static_assert(sizeof(T) == 8, "the FP64 tiles");
     constexpr int M = (SYS == SYS_EULER1D) ? 3 : 1;
-    constexpr int NP = (SYS == SYS_EULER1D) ? 3 : 1;  // u, H, sqrt(rho)
-    constexpr bool F64 = sizeof(T) == 8;
     const int lane = threadIdx.x & 31;
     const T *Us = A.Us;
     const T *U0 = A.U0;
@@ -458,13 +550,16 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
     const int n = A.n;
     const size_t cs = A.cs;
     const int ntiles = min((n + WT - 1) / WT, tile_end);  // tiles tile0, tile0 + tstride, ... below it
-    const T alpha = A.alpha, dtT = A.dtT, gamma = A.gamma, gm1 = A.gm1, a = A.a, eps = A.eps, CT = A.CT;
-    const Cut64 cut = cut64(eps, CT, A.kt);
+    const T alpha = A.alpha, dtT = A.dtT, gamma = A.gamma, gm1 = A.gm1, a = A.a;
+    const T dxs = (M == 3 ? FLUX_SCALE_EULER : FLUX_SCALE_SCALAR) * A.dx;
+    // epsilon times the square of the characteristic values' factor
+    const Cut64 cut2 = cut64(4.0 * A.eps, A.CT, A.kt), cut4 = cut64(16.0 * A.eps, A.CT, A.kt);
     DevCtl *ctl = A.ctl;
     T wsmax = T(0);
     for (int tile = tile0; tile < ntiles; tile += tstride) {
         const int c0 = tile * WT;
         // ---- stage cells c0-5 .. c0+33 -----------------------------------
+        bool zero[2] = {M == 1 && A.kt > T(0), M == 1 && A.kt > T(0)};  // scalar laws: a split vanishes
         for (int c = lane; c < WS; c += 32) {
             int gi = c0 - 5 + c;
             if (gi < 0 || gi >= n) gi = ghost_or_halo(gi, n, A.bc_lo, A.bc_hi, A.halo);
@@ -472,31 +567,15 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
             T U[M], F[M];
 #pragma unroll
             for (int k = 0; k < M; k++) U[k] = Us[(size_t)k * cs + gi];
-            if (SYS == SYS_ADV) {
+            if constexpr (SYS == SYS_ADV) {
                 F[0] = a * U[0];
-            } else if (SYS == SYS_BURGERS) {
+            } else if constexpr (SYS == SYS_BURGERS) {
                 F[0] = T(0.5) * U[0] * U[0];
             } else {
-                if constexpr (F64) {
-                    T u = U[1] / U[0];
-                    T pr = gm1 * (U[2] - T(0.5) * U[1] * u);
-                    F[0] = U[1];
-                    F[1] = U[1] * u + pr;
-                    F[2] = u * (U[2] + pr);
-                    spr[0][c] = u;
-                    spr[NP > 1 ? 1 : 0][c] = (U[2] + pr) / U[0];
-                    spr[NP > 2 ? 2 : 0][c] = sq_root(U[0]);
-                } else {
-                    const float ri = __frcp_rn(U[0]);
-                    const float u = U[1] * ri;
-                    const float pr = gm1 * (U[2] - 0.5f * U[1] * u);
-                    F[0] = U[1];
-                    F[1] = U[1] * u + pr;
-                    F[2] = u * (U[2] + pr);
-                    spr[0][c] = u;
-                    spr[NP > 1 ? 1 : 0][c] = (U[2] + pr) * ri;
-                    spr[NP > 2 ? 2 : 0][c] = __fsqrt_rn(U[0]);
-                }
+                T pr[3];
+                cell1d_f64(U, gm1, F, pr);
+#pragma unroll
+                for (int q = 0; q < 3; q++) spr[q][c] = pr[q];
             }
 #pragma unroll
             for (int k = 0; k < M; k++) {
@@ -504,176 +583,113 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
                 if constexpr (PF) {
                     sgp[k][c] = F[k];
                 } else {
-                    sgp[k][c] = T(0.5) * (F[k] + alpha * U[k]);
-                    sgm[k][c] = T(0.5) * (F[k] - alpha * U[k]);
+                    const T aU = alpha * U[k];
+                    const T gp = F[k] + aU, gm = F[k] - aU;
+                    sgp[k][c] = gp;
+                    sgm[k][c] = gm;
+                    zero[0] = zero[0] && f64_bits(gp) == 0;
+                    zero[1] = zero[1] && f64_bits(gm) == 0;
                 }
             }
         }
         __syncwarp();
 
-        // ---- face j+1/2: frame, projection, cutoff bits --------------------
+        // ---- face j+1/2: frame; then, split by split, projection, cutoff
+        // bits, neighbours' bits, selection and polynomial ------------------
         const int j = c0 - 2 + lane;
-        T L[M][M];
-        T ut = T(0), cc = T(0), Ht = T(0);
-        int flag = 0;
-        if (SYS == SYS_EULER1D) {
-            const T ul = spr[0][lane + 3], ur = spr[0][lane + 4];
-            const T Hl = spr[NP > 1 ? 1 : 0][lane + 3], Hr = spr[NP > 1 ? 1 : 0][lane + 4];
-            const T sl = spr[NP > 2 ? 2 : 0][lane + 3], sr = spr[NP > 2 ? 2 : 0][lane + 4];
-            if constexpr (F64) {
-                // Roe average and eigenvectors in the oracle's operation order
-                ut = (sl * ul + sr * ur) / (sl + sr);
-                Ht = (sl * Hl + sr * Hr) / (sl + sr);
-                const T c2 = gm1 * (Ht - T(0.5) * ut * ut);
-                cc = sq_root(c2);
-                const T b1 = gm1 / c2;
-                const T b2 = T(0.5) * ut * ut * b1;
-                L[0][0] = T(0.5) * (b2 + ut / cc);
-                L[0][1 % M] = T(-0.5) * (b1 * ut + T(1) / cc);
-                L[0][2 % M] = T(0.5) * b1;
-                L[1 % M][0] = T(1) - b2;
-                L[1 % M][1 % M] = b1 * ut;
-                L[1 % M][2 % M] = -b1;
-                L[2 % M][0] = T(0.5) * (b2 - ut / cc);
-                L[2 % M][1 % M] = T(-0.5) * (b1 * ut - T(1) / cc);
-                L[2 % M][2 % M] = T(0.5) * b1;
-                if (!(c2 > T(0))) flag |= isfinite(c2) ? ERR_NONPHYSICAL : ERR_NONFINITE;
-            } else {
-                const float w = __frcp_rn(sl + sr);
-                ut = (sl * ul + sr * ur) * w;
-                Ht = (sl * Hl + sr * Hr) * w;
-                const float c2 = gm1 * (Ht - 0.5f * ut * ut);
-                const float rc = rsqrtf(c2);  // 1/c
-                cc = c2 * rc;
-                const float b1 = gm1 * (rc * rc);
-                const float b2 = 0.5f * ut * ut * b1;
-                const float uc = ut * rc;
-                L[0][0] = 0.5f * (b2 + uc);
-                L[0][1 % M] = -0.5f * (b1 * ut + rc);
-                L[0][2 % M] = 0.5f * b1;
-                L[1 % M][0] = 1.f - b2;
-                L[1 % M][1 % M] = b1 * ut;
-                L[1 % M][2 % M] = -b1;
-                L[2 % M][0] = 0.5f * (b2 - uc);
-                L[2 % M][1 % M] = -0.5f * (b1 * ut - rc);
-                L[2 % M][2 % M] = 0.5f * b1;
-                if (!(c2 > 0.f)) flag |= isfinite(c2) ? ERR_NONPHYSICAL : ERR_NONFINITE;
-            }
-        } else {
-            L[0][0] = T(1);
-        }
-
-        T qp[M][7], qm[M][7];
-        unsigned word = 0;
-#pragma unroll
-        for (int k = 0; k < M; k++) {
-#pragma unroll
-            for (int t = 0; t < 7; t++) {
-                if (SCH == SCH_TENO5 && (t == 0 || t == 6)) {  // five-point stencils
-                    qp[k][t] = qm[k][t] = T(0);
-                    continue;
-                }
-                if constexpr (PF) {
-                    // '+' at cell lane+t, '-' at cell lane+1+t (forward order, as qm)
-                    T lf = L[k][0] * sgp[0][lane + t], lu = L[k][0] * sU[0][lane + t];
-                    T mf = L[k][0] * sgp[0][lane + 1 + t], mu = L[k][0] * sU[0][lane + 1 + t];
-#pragma unroll
-                    for (int c = 1; c < M; c++) {
-                        lf = lf + L[k][c] * sgp[c][lane + t];
-                        lu = lu + L[k][c] * sU[c][lane + t];
-                        mf = mf + L[k][c] * sgp[c][lane + 1 + t];
-                        mu = mu + L[k][c] * sU[c][lane + 1 + t];
-                    }
-                    qp[k][t] = T(0.5) * (lf + A.alf[k] * lu);
-                    qm[k][t] = T(0.5) * (mf - A.alf[k] * mu);
-                } else if (M == 1) {
-                    qp[k][t] = sgp[0][lane + t];
-                    qm[k][t] = sgm[0][lane + 1 + t];
-                } else {
-                    T sp = L[k][0] * sgp[0][lane + t];
-                    T sm = L[k][0] * sgm[0][lane + 1 + t];
-#pragma unroll
-                    for (int c = 1; c < M; c++) {
-                        sp = sp + L[k][c] * sgp[c][lane + t];
-                        sm = sm + L[k][c] * sgm[c][lane + 1 + t];
-                    }
-                    qp[k][t] = sp;
-                    qm[k][t] = sm;
-                }
-            }
-            const unsigned bp = cutoff_bits(qp[k][1], qp[k][2], qp[k][3], qp[k][4], qp[k][5], cut);
-            const unsigned bm = cutoff_bits(qm[k][5], qm[k][4], qm[k][3], qm[k][2], qm[k][1], cut);
-            word |= bp << (3 * k);
-            word |= bm << (3 * (M + k));
-        }
-        // ---- selection, polynomial, back-projection ------------------------
         const bool face_out = lane >= 1 && lane <= 30;
+        Roe64 R;
+        int flag = 0;
+        if constexpr (M == 3) {
+            R = roe_frame_f64(spr[0][lane + 3], spr[0][lane + 4], spr[1][lane + 3], spr[1][lane + 4],
+                              spr[2][lane + 3], spr[2][lane + 4], gm1);
+            flag = R.flag;
+        }
         T f[M];
-        if constexpr (SCH == SCH_TENO5) {
-            // TENO5: the face's own code picks a Table co1 row; '+' taps are
-            // cells j-2 .. j+2, '-' taps cells j+3 .. j-1
+#pragma unroll 1
+        for (int s = 0; s < 2; s++) {
+            T fs[M];
+            unsigned D[M];  // codes
+            if (M == 1 && !PF && __all_sync(0xffffffffu, s == 0 ? zero[0] : zero[1])) {
+                // every window of the split is zero: all stencils kept, flux +0
+                fs[0] = T(0);
+                D[0] = SCH == SCH_TENO5 ? 7u : 31u;
+            } else {
+                // taps in upwind order: '+' cells j-3+t, '-' cells j+4-t
+                T (*sg)[WC] = (PF || s == 0) ? sgp : sgm;
+                const int o = s == 0 ? lane : lane + 7, dir = s == 0 ? 1 : -1;
+                T P[M][7];
+                unsigned word = 0;
+#pragma unroll
+                for (int t = 0; t < 7; t++) {
+                    const int c = o + dir * t;
+                    if constexpr (M == 1) {
+                        P[0][t] = sg[0][c];
+                    } else if (SCH == SCH_TENO5 && (t == 0 || t == 6)) {  // five-point stencils
+                        P[0][t] = P[1][t] = P[2][t] = T(0);
+                    } else {
+                        T q[3];
+                        project_f64(R, sg[0][c], sg[1][c], sg[2][c], q);
+                        if constexpr (PF) {
+                            T qu[3];
+                            project_f64(R, sU[0][c], sU[1][c], sU[2][c], qu);
+#pragma unroll
+                            for (int k = 0; k < 3; k++)
+                                q[k] = s == 0 ? q[k] + A.alf[k] * qu[k] : q[k] - A.alf[k] * qu[k];
+                        }
+#pragma unroll
+                        for (int k = 0; k < 3; k++) P[k][t] = q[k];
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < M; k++)
+                    word |= cutoff_bits(P[k][1], P[k][2], P[k][3], P[k][4], P[k][5],
+                                        M == 3 && k != 1 ? cut4 : cut2)
+                            << (3 * k);
+                if constexpr (SCH == SCH_TENO5) {
+                    // the face's own code picks a Table co1 row on the taps 1 .. 5
+#pragma unroll
+                    for (int k = 0; k < M; k++) {
+                        D[k] = (word >> (3 * k)) & 7u;
+                        int r = sel5(D[k]);
+                        if (r == 7) {
+                            r = 0;
+                            if (face_out) flag |= ERR_NOEXIST;
+                        }
+                        fs[k] = poly5(scoef + 5 * r, P[k][1], P[k][2], P[k][3], P[k][4], P[k][5]);
+                    }
+                } else {
+                    const unsigned wl = __shfl_up_sync(0xffffffffu, word, 1);
+                    const unsigned wr = __shfl_down_sync(0xffffffffu, word, 1);
+                    const unsigned wu = s == 0 ? wl : wr, wd = s == 0 ? wr : wl;  // upwind, downwind face
+#pragma unroll
+                    for (int k = 0; k < M; k++) {
+                        D[k] = (unsigned)pack_delta(wu >> (3 * k), word >> (3 * k), wd >> (3 * k));
+                        int m = lut_select((int)D[k]);
+                        if (m == 15) {
+                            m = 11;
+                            if (face_out) flag |= ERR_NOEXIST;
+                        }
+                        if (m == 0)
+                            fs[k] = poly_f0(P[k][0], P[k][1], P[k][2], P[k][3], P[k][4], P[k][5], P[k][6]);
+                        else
+                            fs[k] = poly7(scoef + 7 * m, P[k][0], P[k][1], P[k][2], P[k][3], P[k][4], P[k][5],
+                                          P[k][6]);
+                    }
+                }
+            }
 #pragma unroll
             for (int k = 0; k < M; k++) {
-                const unsigned bp = (word >> (3 * k)) & 7u, bm = (word >> (3 * (M + k))) & 7u;
-                int rp = sel5(bp), rm = sel5(bm);
-                if (rp == 7) {
-                    rp = 0;
-                    if (face_out) flag |= ERR_NOEXIST;
-                }
-                if (rm == 7) {
-                    rm = 0;
-                    if (face_out) flag |= ERR_NOEXIST;
-                }
-                const T fp = poly5(scoef + 5 * rp, qp[k][1], qp[k][2], qp[k][3], qp[k][4], qp[k][5]);
-                const T fm = poly5(scoef + 5 * rm, qm[k][5], qm[k][4], qm[k][3], qm[k][2], qm[k][1]);
-                f[k] = fp + fm;
-                if (A.masks && face_out && j >= -1 && j <= n - 1) {
-                    A.masks[(size_t)(0 * M + k) * (n + 1) + (j + 1)] = (uint8_t)bp;
-                    A.masks[(size_t)(1 * M + k) * (n + 1) + (j + 1)] = (uint8_t)bm;
-                }
-            }
-        } else {
-        const unsigned wl = __shfl_up_sync(0xffffffffu, word, 1);
-        const unsigned wr = __shfl_down_sync(0xffffffffu, word, 1);
-#pragma unroll
-        for (int k = 0; k < M; k++) {
-            const int Dp = pack_delta(wl >> (3 * k), word >> (3 * k), wr >> (3 * k));
-            const int Dm = pack_delta(wr >> (3 * (M + k)), word >> (3 * (M + k)), wl >> (3 * (M + k)));
-            int mp = lut_select(Dp), mm = lut_select(Dm);
-            if (mp == 15) {
-                mp = 11;
-                if (face_out) flag |= ERR_NOEXIST;
-            }
-            if (mm == 15) {
-                mm = 11;
-                if (face_out) flag |= ERR_NOEXIST;
-            }
-            T fp, fm;
-            if (mp == 0)
-                fp = poly_f0(qp[k][0], qp[k][1], qp[k][2], qp[k][3], qp[k][4], qp[k][5], qp[k][6]);
-            else
-                fp = poly7(scoef + 7 * mp, qp[k][0], qp[k][1], qp[k][2], qp[k][3], qp[k][4], qp[k][5], qp[k][6]);
-            if (mm == 0)
-                fm = poly_f0(qm[k][6], qm[k][5], qm[k][4], qm[k][3], qm[k][2], qm[k][1], qm[k][0]);
-            else
-                fm = poly7(scoef + 7 * mm, qm[k][6], qm[k][5], qm[k][4], qm[k][3], qm[k][2], qm[k][1], qm[k][0]);
-            f[k] = fp + fm;
-            if (A.masks && face_out && j >= -1 && j <= n - 1) {
-                A.masks[(size_t)(0 * M + k) * (n + 1) + (j + 1)] = (uint8_t)Dp;
-                A.masks[(size_t)(1 * M + k) * (n + 1) + (j + 1)] = (uint8_t)Dm;
+                f[k] = s == 0 ? fs[k] : f[k] + fs[k];
+                if (A.masks && face_out && j >= -1 && j <= n - 1)
+                    A.masks[(size_t)(s * M + k) * (n + 1) + (j + 1)] = (uint8_t)D[k];
             }
         }
-        }  // TENO7-ext
         T fh[M];
-        if (SYS == SYS_EULER1D) {
-            // R columns: eigenvectors of u-c, u, u+c at the Roe state
-            const T R20 = Ht - ut * cc, R21 = T(0.5) * ut * ut, R22 = Ht + ut * cc;
-            fh[0] = f[0] + f[1 % M] + f[2 % M];
-            fh[1 % M] = (ut - cc) * f[0] + ut * f[1 % M] + (ut + cc) * f[2 % M];
-            fh[2 % M] = R20 * f[0] + R21 * f[1 % M] + R22 * f[2 % M];
-        } else {
+        if constexpr (M == 3)
+            back_project_f64(R, f, fh);
+        else
             fh[0] = f[0];
-        }
         if (flag && face_out && j >= -2 && j <= n)
             latch_error(ctl, (flag & (ERR_NONPHYSICAL | ERR_NONFINITE)) | ((flag & ERR_NOEXIST) ? ERR_NONFINITE : 0),
                         A.ebase + j);
@@ -686,14 +702,8 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
         if (lane >= 2 && lane <= 30 && i < n) {
             const int ii = chk(ctl, i, 0, n);
             T r[M];
-            if constexpr (F64) {
 #pragma unroll
-                for (int k = 0; k < M; k++) r[k] = (fprev[k] - fh[k]) / A.dx;
-            } else {
-                const float idx = __frcp_rn(A.f_dx);
-#pragma unroll
-                for (int k = 0; k < M; k++) r[k] = (fprev[k] - fh[k]) * idx;
-            }
+            for (int k = 0; k < M; k++) r[k] = (fprev[k] - fh[k]) / dxs;
             if (A.rhs_mode) {
 #pragma unroll
                 for (int k = 0; k < M; k++) out[(size_t)k * A.cso + ii] = r[k];
@@ -701,21 +711,8 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
                 T o[M];
 #pragma unroll
                 for (int k = 0; k < M; k++) {
-                    const T us = sU[k][lane + 3];
-                    if (A.stage == 0) {
-                        o[k] = us + dtT * r[k];
-                    } else if (A.stage == 1) {
-                        o[k] = T(0.75) * U0[(size_t)k * cs + ii] + T(0.25) * (us + dtT * r[k]);
-                    } else {
-                        if constexpr (F64) {
-                            o[k] = T(1.0 / 3.0) * U0[(size_t)k * cs + ii] + T(2.0 / 3.0) * (us + dtT * r[k]);
-                        } else {
-                            // in FP32, float(1/3) + float(2/3) = 1 + 6e-8 would grow the
-                            // solution by that factor every step: use u0 + 2/3 (v - u0)
-                            const T u0 = U0[(size_t)k * cs + ii];
-                            o[k] = fmaf(2.0f / 3.0f, (us + dtT * r[k]) - u0, u0);
-                        }
-                    }
+                    o[k] = rk_combine_f64(A.stage, sU[k][lane + 3], dtT, r[k],
+                                          A.stage == 0 ? T(0) : U0[(size_t)k * cs + ii]);
                     out[(size_t)k * A.cso + ii] = o[k];
                 }
                 int wflag = 0;
@@ -723,9 +720,9 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
                     T w[3];
                     wavespeeds1d<T>(o, gm1, gamma, w, &wflag);
 #pragma unroll
-                    for (int q = 0; q < 3; q++) ws3[q] = fmax(ws3[q], w[q]);
+                    for (int q = 0; q < 3; q++) ws3[q] = f64_max_pos(ws3[q], w[q]);
                 } else {
-                    wsmax = fmax(wsmax, wavespeed1d<T, SYS>(o, gm1, gamma, a, &wflag));
+                    wsmax = f64_max_pos(wsmax, wavespeed1d<T, SYS>(o, gm1, gamma, a, &wflag));
                 }
                 if (wflag) latch_error(ctl, wflag, A.ebase + i);
             }

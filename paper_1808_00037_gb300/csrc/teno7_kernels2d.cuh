@@ -29,148 +29,166 @@ __device__ __forceinline__ int flat_cell(int y, int x, int nx, int ny = 0x7fffff
     return y * nx + x;
 }
 
-// Per-face state of one 2D sweep: characteristic projections of the 8 stencil
-// cells, Roe state, cutoff word ('+' codes at bits 3k, '-' at 3(4+k)).
-template <typename T>
-struct Face2D {
-    T qp[4][7], qm[4][7];
-    T un, vt, c, Ht, q2;
-    unsigned word;
-    int flag;
-};
-
 // Rotated index of physical component c for sweep direction DIR (1 <-> 2 in y).
 template <int DIR>
 __device__ __forceinline__ constexpr int rot(int c) {
     return DIR == 0 ? c : (c == 1 ? 2 : (c == 2 ? 1 : c));
 }
 
-// Frame, projection and cutoff bits of one face.  pr(q, t): staged primitive q
-// (0 normal velocity, 1 tangential velocity, 2 H, 3 sqrt(rho)) of local cell t;
-// gp(c, t) / gm(c, t): physical component c of the split fluxes of local cell
-// t; local cell t = 0 .. 7 is cell j-3+t of face j+1/2.
-template <typename T, int DIR, typename PR, typename GP, typename GM>
-__device__ __forceinline__ void face2d_bits(Face2D<T> &F, PR pr, GP gp, GM gm, T gm1, const Cut64 &cut) {
-    const T unl = pr(0, 3), unr = pr(0, 4), utl = pr(1, 3), utr = pr(1, 4);
-    const T Hl = pr(2, 3), Hr = pr(2, 4), sl = pr(3, 3), sr = pr(3, 4);
-    F.un = (sl * unl + sr * unr) / (sl + sr);
-    F.vt = (sl * utl + sr * utr) / (sl + sr);
-    F.Ht = (sl * Hl + sr * Hr) / (sl + sr);
-    F.q2 = T(0.5) * (F.un * F.un + F.vt * F.vt);
-    const T c2 = gm1 * (F.Ht - F.q2);
-    F.c = sq_root(c2);
-    const T b1 = gm1 / c2;
-    const T b2 = F.q2 * b1;
-    const T un = F.un, vt = F.vt, c = F.c;
-    const T Lr[4][4] = {
-        {T(0.5) * (b2 + un / c), T(-0.5) * (b1 * un + T(1) / c), T(-0.5) * (b1 * vt), T(0.5) * b1},
-        {T(1) - b2, b1 * un, b1 * vt, -b1},
-        {-vt, T(0), T(1), T(0)},
-        {T(0.5) * (b2 - un / c), T(-0.5) * (b1 * un - T(1) / c), T(-0.5) * (b1 * vt), T(0.5) * b1},
-    };
-    F.flag = (c2 > T(0)) ? 0 : (isfinite(c2) ? ERR_NONPHYSICAL : ERR_NONFINITE);
-    F.word = 0;
+// FP64 face of one 2D sweep, with the exact powers of two of the 1D form
+// (roe_frame_f64): rows un -+ c of L doubled, 2 G+- staged, so the fields 0 and
+// 3 carry a factor 4, the entropy and shear fields 1 and 2 a factor 2, and the
+// face flux 4.  The products b1 v_t g_t and b1 g_E serve three fields each, and
+// the shear row (-v_t, 0, 1, 0) costs one product and one sum (adding 0 g could
+// only change the sign of a zero): 19 instead of 28 FP64 instructions per
+// projected cell and split.
+struct Roe2D64 {
+    double l0[2], l1[2], l3[2], b1, b1v, un, vt, cc, Ht, X;
+    int flag;
+};
+
+// pr(q, t): staged primitive q (0 normal velocity, 1 tangential velocity, 2 H, 3
+// sqrt(rho)) of local cell t; local cell t = 0 .. 7 is cell j-3+t of face j+1/2.
+template <typename PR>
+__device__ __forceinline__ Roe2D64 roe_frame2d_f64(PR pr, double gm1) {
+    Roe2D64 R;
+    const double sl = pr(3, 3), sr = pr(3, 4), S = sl + sr;
+    R.un = (sl * pr(0, 3) + sr * pr(0, 4)) / S;
+    R.vt = (sl * pr(1, 3) + sr * pr(1, 4)) / S;
+    R.Ht = (sl * pr(2, 3) + sr * pr(2, 4)) / S;
+    R.X = R.un * R.un + R.vt * R.vt;
+    const double c2 = gm1 * __fma_rn(-0.5, R.X, R.Ht);
+    R.cc = sqrt(c2);
+    R.b1 = gm1 / c2;
+    const double t = R.X * R.b1;  // 2 b2
+    const double uc = R.un / R.cc, rc = 1.0 / R.cc;
+    const double b1u = R.b1 * R.un;
+    R.b1v = R.b1 * R.vt;
+    R.l0[0] = __fma_rn(0.5, t, uc);
+    R.l0[1] = -(b1u + rc);
+    R.l1[0] = __fma_rn(-0.5, t, 1.0);
+    R.l1[1] = b1u;
+    R.l3[0] = __fma_rn(0.5, t, -uc);
+    R.l3[1] = -(b1u - rc);
+    R.flag = f64_positive(c2) ? 0 : (f64_finite(c2) ? ERR_NONPHYSICAL : ERR_NONFINITE);
+    return R;
+}
+
+// Characteristic values of one cell's split flux g (physical components; the
+// sums run in physical order, so along y the tangential term comes second).
+template <int DIR>
+__device__ __forceinline__ void project2d_f64(const Roe2D64 &R, const double g[4], double q[4]) {
+    const double gn = g[rot<DIR>(1)], gt = g[rot<DIR>(2)];
+    const double pt = R.b1v * gt, pe = R.b1 * g[3];
+    const double n0 = R.l0[1] * gn, n1 = R.l1[1] * gn, n3 = R.l3[1] * gn;
+    if constexpr (DIR == 0) {
+        q[0] = ((R.l0[0] * g[0] + n0) - pt) + pe;
+        q[1] = ((R.l1[0] * g[0] + n1) + pt) - pe;
+        q[3] = ((R.l3[0] * g[0] + n3) - pt) + pe;
+    } else {
+        q[0] = ((R.l0[0] * g[0] - pt) + n0) + pe;
+        q[1] = ((R.l1[0] * g[0] + pt) + n1) - pe;
+        q[3] = ((R.l3[0] * g[0] - pt) + n3) + pe;
+    }
+    q[2] = gt - R.vt * g[0];
+}
+
+// Flux of one face (scaled by 4) from the staged cells, split by split:
+// projection, cutoff bits, the neighbour faces' bits (adjacent lanes), selection
+// and polynomial, then the back-projection.  gp(c, t) / gm(c, t): component c of
+// 2 G+ / 2 G- of local cell t.  Returns the error flags; D[0..3] and D[4..7]
+// receive the Delta codes of the '+' and '-' splits.  Call with a whole warp.
+template <int DIR, typename PR, typename G>
+__device__ __forceinline__ int face2d_f64(PR pr, G g, double gm1, const Cut64 &cut2, const Cut64 &cut4,
+                                          const double *coef, double fh[4], int D[8]) {
+    const Roe2D64 R = roe_frame2d_f64(pr, gm1);
+    int flag = R.flag;
+    double f[4];
 #pragma unroll
-    for (int k = 0; k < 4; k++) {
+    for (int s = 0; s < 2; s++) {
+        double P[4][7];
+        unsigned word = 0;
 #pragma unroll
         for (int t = 0; t < 7; t++) {
-            // physical component order c = 0..3, L[k][c] = Lr[k][rot(c)]
-            T sp = Lr[k][0] * gp(0, t);
-            T sm = Lr[k][0] * gm(0, t + 1);
-            sp = sp + Lr[k][rot<DIR>(1)] * gp(1, t);
-            sm = sm + Lr[k][rot<DIR>(1)] * gm(1, t + 1);
-            sp = sp + Lr[k][rot<DIR>(2)] * gp(2, t);
-            sm = sm + Lr[k][rot<DIR>(2)] * gm(2, t + 1);
-            sp = sp + Lr[k][3] * gp(3, t);
-            sm = sm + Lr[k][3] * gm(3, t + 1);
-            F.qp[k][t] = sp;
-            F.qm[k][t] = sm;
+            // upwind order: '+' cells j-3+t, '-' cells j+4-t
+            const int c = s == 0 ? t : 7 - t;
+            const double gc[4] = {g(s, 0, c), g(s, 1, c), g(s, 2, c), g(s, 3, c)};
+            double q[4];
+            project2d_f64<DIR>(R, gc, q);
+#pragma unroll
+            for (int k = 0; k < 4; k++) P[k][t] = q[k];
         }
-        const unsigned bp = cutoff_bits(F.qp[k][1], F.qp[k][2], F.qp[k][3], F.qp[k][4], F.qp[k][5], cut);
-        const unsigned bm = cutoff_bits(F.qm[k][5], F.qm[k][4], F.qm[k][3], F.qm[k][2], F.qm[k][1], cut);
-        F.word |= bp << (3 * k);
-        F.word |= bm << (3 * (4 + k));
+#pragma unroll
+        for (int k = 0; k < 4; k++)
+            word |= cutoff_bits(P[k][1], P[k][2], P[k][3], P[k][4], P[k][5], k == 0 || k == 3 ? cut4 : cut2)
+                    << (3 * k);
+        const unsigned wl = __shfl_up_sync(0xffffffffu, word, 1);
+        const unsigned wr = __shfl_down_sync(0xffffffffu, word, 1);
+        const unsigned wu = s == 0 ? wl : wr, wd = s == 0 ? wr : wl;  // upwind, downwind face
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const int Dk = pack_delta(wu >> (3 * k), word >> (3 * k), wd >> (3 * k));
+            int m = lut_select(Dk);
+            if (m == 15) {
+                m = 11;
+                flag |= ERR_NOEXIST;
+            }
+            double v;
+            if (m == 0)
+                v = poly_f0(P[k][0], P[k][1], P[k][2], P[k][3], P[k][4], P[k][5], P[k][6]);
+            else
+                v = poly7(coef + 7 * m, P[k][0], P[k][1], P[k][2], P[k][3], P[k][4], P[k][5], P[k][6]);
+            f[k] = s == 0 ? v : f[k] + v;
+            D[4 * s + k] = Dk;
+        }
     }
+    // right eigenvectors (columns un-c, un, shear, un+c) in rotated rows; f[1]
+    // and f[2] are doubled on the way, the sums in the fields' order
+    const double w = R.un * R.cc, f1 = 2.0 * f[1];
+    double q[4];
+    q[0] = (f[0] + f1) + f[3];
+    q[1] = ((R.un - R.cc) * f[0] + R.un * f1) + (R.un + R.cc) * f[3];
+    q[2] = __fma_rn(2.0, f[2], R.vt * f[0] + R.vt * f1) + R.vt * f[3];
+    q[3] = __fma_rn(2.0, R.vt * f[2], (R.Ht - w) * f[0] + R.X * f[1]) + (R.Ht + w) * f[3];
+#pragma unroll
+    for (int c = 0; c < 4; c++) fh[c] = q[rot<DIR>(c)];
+    return flag;
 }
 
-// Selection, polynomial and back-projection of one face given the neighbours'
-// words.  Writes the physical face flux fh[4] and (if D != nullptr) the Delta
-// codes D[0..3] ('+') and D[4..7] ('-').
-template <typename T, int DIR>
-__device__ __forceinline__ void face2d_flux(Face2D<T> &F, unsigned wl, unsigned wr, const T *coef, T fh[4],
-                                            int *D) {
-    T f[4];
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-        const int Dp = pack_delta(wl >> (3 * k), F.word >> (3 * k), wr >> (3 * k));
-        const int Dm = pack_delta(wr >> (3 * (4 + k)), F.word >> (3 * (4 + k)), wl >> (3 * (4 + k)));
-        int mp = lut_select(Dp), mm = lut_select(Dm);
-        if (mp == 15) {
-            mp = 11;
-            F.flag |= ERR_NOEXIST;
-        }
-        if (mm == 15) {
-            mm = 11;
-            F.flag |= ERR_NOEXIST;
-        }
-        const T *cp = coef + 7 * mp, *cm = coef + 7 * mm;
-        const T fp = poly7(cp, F.qp[k][0], F.qp[k][1], F.qp[k][2], F.qp[k][3], F.qp[k][4], F.qp[k][5], F.qp[k][6]);
-        const T fm = poly7(cm, F.qm[k][6], F.qm[k][5], F.qm[k][4], F.qm[k][3], F.qm[k][2], F.qm[k][1], F.qm[k][0]);
-        f[k] = fp + fm;
-        if (D) {
-            D[k] = Dp;
-            D[4 + k] = Dm;
-        }
-    }
-    const T un = F.un, vt = F.vt, c = F.c, Ht = F.Ht, q2 = F.q2;
-    // rotated right eigenvectors (columns un-c, un, shear, un+c), rows in rotated order
-    const T Rr[4][4] = {
-        {T(1), T(1), T(0), T(1)},
-        {un - c, un, T(0), un + c},
-        {vt, vt, T(1), vt},
-        {Ht - un * c, q2, vt, Ht + un * c},
-    };
-#pragma unroll
-    for (int cc = 0; cc < 4; cc++) {
-        const int r = rot<DIR>(cc);
-        T s = Rr[r][0] * f[0];
-        s = s + Rr[r][1] * f[1];
-        s = s + Rr[r][2] * f[2];
-        s = s + Rr[r][3] * f[3];
-        fh[cc] = s;
-    }
-}
-
-// Per-cell primitives and split fluxes of one 2D state along DIR, in the
-// oracle's expression order.  prim = (normal velocity, tangential velocity, H,
-// sqrt(rho)).
-template <typename T, int DIR>
-__device__ __forceinline__ void cell2d(const T U[4], T gm1, T alpha, T prim[4], T gp[4], T gm[4]) {
-    const T u = U[1] / U[0];
-    const T v = U[2] / U[0];
-    const T p = gm1 * (U[3] - T(0.5) * (U[1] * u + U[2] * v));
-    T F[4];
+// Per-cell primitives and twice the split fluxes of one 2D state along DIR, in
+// the oracle's expression order.  prim = (normal velocity, tangential velocity,
+// H, sqrt(rho)).
+template <int DIR>
+__device__ __forceinline__ void cell2d_f64(const double U[4], double gm1, double alpha, double prim[4], double gp[4],
+                                           double gm[4]) {
+    const double u = U[1] / U[0];
+    const double v = U[2] / U[0];
+    const double mu = U[1] * u, mv = U[2] * v;
+    const double p = gm1 * __fma_rn(-0.5, mu + mv, U[3]);
+    const double e = U[3] + p;
+    double F[4];
     if (DIR == 0) {
         F[0] = U[1];
-        F[1] = U[1] * u + p;
+        F[1] = mu + p;
         F[2] = U[2] * u;
-        F[3] = u * (U[3] + p);
+        F[3] = u * e;
         prim[0] = u;
         prim[1] = v;
     } else {
         F[0] = U[2];
         F[1] = U[1] * v;
-        F[2] = U[2] * v + p;
-        F[3] = v * (U[3] + p);
+        F[2] = mv + p;
+        F[3] = v * e;
         prim[0] = v;
         prim[1] = u;
     }
-    prim[2] = (U[3] + p) / U[0];
-    prim[3] = sq_root(U[0]);
+    prim[2] = e / U[0];
+    prim[3] = sqrt(U[0]);
 #pragma unroll
     for (int k = 0; k < 4; k++) {
-        gp[k] = T(0.5) * (F[k] + alpha * U[k]);
-        gm[k] = T(0.5) * (F[k] - alpha * U[k]);
+        const double aU = alpha * U[k];
+        gp[k] = F[k] + aU;
+        gm[k] = F[k] - aU;
     }
 }
 
@@ -186,14 +204,21 @@ __device__ __forceinline__ void wavespeed2d(const T U[4], T gm1, T gamma, T &sx,
         p = __fmul_rn(gm1, __fmaf_rn(-0.5f, __fmaf_rn(U[1], u, __fmul_rn(U[2], v)), U[3]));
         c = sqrtf(__fdiv_rn(__fmul_rn(gamma, p), U[0]));
     } else {
-        p = gm1 * (U[3] - T(0.5) * (U[1] * u + U[2] * v));
+        p = gm1 * __fma_rn(-0.5, U[1] * u + U[2] * v, U[3]);
         c = sq_root(gamma * p / U[0]);
     }
     // a non-finite cell is reported as such; a finite one needs rho > 0, p > 0
-    if (!isfinite(U[0]) || !isfinite(U[1]) || !isfinite(U[2]) || !isfinite(U[3]))
-        *flag |= ERR_NONFINITE;
-    else if (!(U[0] > T(0)) || !(p > T(0)))
-        *flag |= ERR_NONPHYSICAL;
+    if constexpr (sizeof(T) == 8) {
+        if (!f64_finite(U[0]) || !f64_finite(U[1]) || !f64_finite(U[2]) || !f64_finite(U[3]))
+            *flag |= ERR_NONFINITE;
+        else if (!f64_positive(U[0]) || !f64_positive(p))
+            *flag |= ERR_NONPHYSICAL;
+    } else {
+        if (!isfinite(U[0]) || !isfinite(U[1]) || !isfinite(U[2]) || !isfinite(U[3]))
+            *flag |= ERR_NONFINITE;
+        else if (!(U[0] > T(0)) || !(p > T(0)))
+            *flag |= ERR_NONPHYSICAL;
+    }
     if constexpr (sizeof(T) == 4) {
         sx = __fadd_rn(fabsf(u), c);
         sy = __fadd_rn(fabsf(v), c);
@@ -269,7 +294,8 @@ __global__ void __launch_bounds__(WPB * 32, 1) xsweep2d_kernel(const Stage2D p) 
     for (int q = lane; q < 91; q += 32) s_coef[warp][q] = coef<T>(q);
     const T alpha = alpha2d_in<T, HALO>(p, ctl, 0);
     const T gm1 = pick<T>(p.gamma - 1.0, p.f_gm1);
-    const Cut64 cut = cut64(p.eps_x, p.CT, p.kt);
+    const Cut64 cut2 = cut64(4.0 * p.eps_x, p.CT, p.kt), cut4 = cut64(16.0 * p.eps_x, p.CT, p.kt);
+    const T dx4 = FLUX_SCALE_EULER * p.dx;
     const T *Us = static_cast<const T *>(p.Us);
     T *R = static_cast<T *>(p.R);
     const int nx = p.nx, ny = p.ny;
@@ -292,7 +318,7 @@ __global__ void __launch_bounds__(WPB * 32, 1) xsweep2d_kernel(const Stage2D p) 
             T U[4], pr[4], gp[4], gm[4];
 #pragma unroll
             for (int k = 0; k < 4; k++) U[k] = row[(size_t)k * sv + gi];
-            cell2d<T, 0>(U, gm1, alpha, pr, gp, gm);
+            cell2d_f64<0>(U, gm1, alpha, pr, gp, gm);
 #pragma unroll
             for (int k = 0; k < 4; k++) {
                 spr[k][c] = pr[k];
@@ -302,23 +328,19 @@ __global__ void __launch_bounds__(WPB * 32, 1) xsweep2d_kernel(const Stage2D p) 
         }
         __syncwarp();
         const int j = c0 - 2 + lane;
-        Face2D<T> F;
-        face2d_bits<T, 0>(
-            F, [&](int q, int t) { return spr[q][lane + t]; }, [&](int c, int t) { return sgp[c][lane + t]; },
-            [&](int c, int t) { return sgm[c][lane + t]; }, gm1, cut);
-        const unsigned wl = __shfl_up_sync(0xffffffffu, F.word, 1);
-        const unsigned wr = __shfl_down_sync(0xffffffffu, F.word, 1);
         T fh[4];
         int D[8];
-        face2d_flux<T, 0>(F, wl, wr, s_coef[warp], fh, D);
+        const int flag = face2d_f64<0>([&](int q, int t) { return spr[q][lane + t]; },
+                                       [&](int s, int c, int t) { return (s == 0 ? sgp : sgm)[c][lane + t]; }, gm1,
+                                       cut2, cut4, s_coef[warp], fh, D);
         const bool face_out = lane >= 1 && lane <= 30;
         if (p.rhs_mode && p.masks && face_out && j >= -1 && j <= nx - 1) {
 #pragma unroll
             for (int sk = 0; sk < 8; sk++)
                 p.masks[((size_t)sk * ny + y) * (nx + 1) + (j + 1)] = (uint8_t)D[sk];
         }
-        if (F.flag && face_out && j >= -2 && j <= nx)
-            latch_error(ctl, (F.flag & (ERR_NONPHYSICAL | ERR_NONFINITE)) | ((F.flag & ERR_NOEXIST) ? ERR_NONFINITE : 0),
+        if (flag && face_out && j >= -2 && j <= nx)
+            latch_error(ctl, (flag & (ERR_NONPHYSICAL | ERR_NONFINITE)) | ((flag & ERR_NOEXIST) ? ERR_NONFINITE : 0),
                         flat_cell(y, j, nx));
         T fprev[4];
 #pragma unroll
@@ -326,12 +348,7 @@ __global__ void __launch_bounds__(WPB * 32, 1) xsweep2d_kernel(const Stage2D p) 
         if (lane >= 2 && lane <= 30 && j < nx) {
 #pragma unroll
             for (int k = 0; k < 4; k++) {
-                T r;
-                if constexpr (sizeof(T) == 8) {
-                    r = (fprev[k] - fh[k]) / p.dx;
-                } else {
-                    r = (fprev[k] - fh[k]) * (1.f / p.f_dx);
-                }
+                const T r = (fprev[k] - fh[k]) / dx4;
                 R[(size_t)k * N + (size_t)y * nx + chk(p.ctl, j, 0, p.nx)] = r;
             }
         }
@@ -373,7 +390,8 @@ __global__ void __launch_bounds__(WPB * 32, 1) ysweep2d_kernel(const Stage2D p) 
     const int x0 = blockIdx.x * YB_COLS, r0 = blockIdx.y * YB_ROWS;
     const T alpha = alpha2d_in<T, HALO>(p, ctl, 1);
     const T gamma = pick<T>(p.gamma, p.f_gamma), gm1 = pick<T>(p.gamma - 1.0, p.f_gm1);
-    const Cut64 cut = cut64(p.eps_y, p.CT, p.kt);
+    const Cut64 cut2 = cut64(4.0 * p.eps_y, p.CT, p.kt), cut4 = cut64(16.0 * p.eps_y, p.CT, p.kt);
+    const T dy4 = FLUX_SCALE_EULER * p.dy;
     const T *Us = static_cast<const T *>(p.Us);
     for (int q = tid; q < 91; q += blockDim.x) s_coef[q] = coef<T>(q);
 
@@ -386,7 +404,7 @@ __global__ void __launch_bounds__(WPB * 32, 1) ysweep2d_kernel(const Stage2D p) 
         T U[4], pr[4], gp[4], gm[4];
 #pragma unroll
         for (int k = 0; k < 4; k++) U[k] = Us[st_at<HALO>(k, sv, y, nx, chk(p.ctl, x, 0, p.nx))];
-        cell2d<T, 1>(U, gm1, alpha, pr, gp, gm);
+        cell2d_f64<1>(U, gm1, alpha, pr, gp, gm);
 #pragma unroll
         for (int k = 0; k < 4; k++) {
             at(s_pr, k, r, col) = pr[k];
@@ -401,24 +419,19 @@ __global__ void __launch_bounds__(WPB * 32, 1) ysweep2d_kernel(const Stage2D p) 
         const int x = x0 + col;
         if (x >= nx) break;
         const int j = r0 - 2 + lane;  // face j+1/2 along y
-        Face2D<T> F;
-        face2d_bits<T, 1>(
-            F, [&](int q, int t) { return at(s_pr, q, lane + t, col); },
-            [&](int c, int t) { return at(s_gp, c, lane + t, col); },
-            [&](int c, int t) { return at(s_gm, c, lane + t, col); }, gm1, cut);
-        const unsigned wl = __shfl_up_sync(0xffffffffu, F.word, 1);
-        const unsigned wr = __shfl_down_sync(0xffffffffu, F.word, 1);
         T fh[4];
         int D[8];
-        face2d_flux<T, 1>(F, wl, wr, s_coef, fh, D);
+        const int flag = face2d_f64<1>([&](int q, int t) { return at(s_pr, q, lane + t, col); },
+                                       [&](int s, int c, int t) { return at(s == 0 ? s_gp : s_gm, c, lane + t, col); },
+                                       gm1, cut2, cut4, s_coef, fh, D);
         const bool face_out = lane >= 1 && lane <= 30;
         if (p.rhs_mode && p.masks && face_out && j >= -1 && j <= ny - 1) {
             uint8_t *ym = p.masks + (size_t)8 * ny * (nx + 1);
 #pragma unroll
             for (int sk = 0; sk < 8; sk++) ym[((size_t)sk * nx + x) * (ny + 1) + (j + 1)] = (uint8_t)D[sk];
         }
-        if (F.flag && face_out && j >= -2 && j <= ny)
-            latch_error(ctl, (F.flag & (ERR_NONPHYSICAL | ERR_NONFINITE)) | ((F.flag & ERR_NOEXIST) ? ERR_NONFINITE : 0),
+        if (flag && face_out && j >= -2 && j <= ny)
+            latch_error(ctl, (flag & (ERR_NONPHYSICAL | ERR_NONFINITE)) | ((flag & ERR_NOEXIST) ? ERR_NONFINITE : 0),
                         flat_cell(j, x, nx, ny));
         T fprev[4];
 #pragma unroll
@@ -426,12 +439,7 @@ __global__ void __launch_bounds__(WPB * 32, 1) ysweep2d_kernel(const Stage2D p) 
         if (lane >= 2 && lane <= 30) {
 #pragma unroll
             for (int k = 0; k < 4; k++) {
-                T r;
-                if constexpr (sizeof(T) == 8) {
-                    r = (fprev[k] - fh[k]) / p.dy;
-                } else {
-                    r = (fprev[k] - fh[k]) * (1.f / p.f_dy);
-                }
+                const T r = (fprev[k] - fh[k]) / dy4;
                 s_ry[(k * YB_ROWS + (lane - 2)) * YB_LD + col] = r;
             }
         }
@@ -463,19 +471,8 @@ __global__ void __launch_bounds__(WPB * 32, 1) ysweep2d_kernel(const Stage2D p) 
                 out[(size_t)k * svo + g] = rr;
                 continue;
             }
-            const T us = Us[(size_t)k * sv + g];
-            if (p.stage == 0) {
-                o[k] = us + dtT * rr;
-            } else if (p.stage == 1) {
-                o[k] = T(0.75) * U0[(size_t)k * sv + g] + T(0.25) * (us + dtT * rr);
-            } else {
-                if constexpr (sizeof(T) == 8) {
-                    o[k] = T(1.0 / 3.0) * U0[(size_t)k * sv + g] + T(2.0 / 3.0) * (us + dtT * rr);
-                } else {
-                    const T u0 = U0[(size_t)k * sv + g];
-                    o[k] = fmaf(2.0f / 3.0f, (us + dtT * rr) - u0, u0);
-                }
-            }
+            o[k] = rk_combine_f64(p.stage, Us[(size_t)k * sv + g], dtT, rr,
+                                  p.stage == 0 ? T(0) : U0[(size_t)k * sv + g]);
             out[(size_t)k * svo + g] = o[k];
         }
         if (!p.rhs_mode) {
@@ -483,8 +480,8 @@ __global__ void __launch_bounds__(WPB * 32, 1) ysweep2d_kernel(const Stage2D p) 
             T sx, sy;
             wavespeed2d<T>(o, gm1, gamma, sx, sy, &wflag);
             if (wflag) latch_error(ctl, wflag, (int)g);
-            mx = fmax(mx, sx);
-            my = fmax(my, sy);
+            mx = f64_max_pos(mx, sx);
+            my = f64_max_pos(my, sy);
         }
     }
     if (!p.rhs_mode) {
