@@ -61,14 +61,122 @@ T7_HD double f64_max_pos(double x, double y) {
     const uint64_t bx = f64_bits(x), by = f64_bits(y);
     return f64_of(by > bx && by <= 0x7ff0000000000000ull ? by : bx);
 }
-T7_HD float f32_rcp(float x) {  // approximate reciprocal, within 2 ulp
+T7_HD int f32_to_int(float x) {  // nearest integer, |x| < 2^31
+#ifdef __CUDA_ARCH__
+    return __float2int_rn(x);
+#else
+    return (int)lrintf(x);
+#endif
+}
+// Approximate reciprocal, within 2 ulp.  (T7_HOST_ERR: a host check may scale the
+// approximations by their error bound.)
+#ifndef T7_HOST_ERR
+#define T7_HOST_ERR
+#endif
+T7_HD float f32_rcp(float x) {
 #ifdef __CUDA_ARCH__
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 #else
-    return 1.0f / x;
+    return (1.0f / x) T7_HOST_ERR;
 #endif
+}
+
+T7_HD float f32_rsqrt(float x) {  // approximate 1/sqrt, within 2^-22
+#ifdef __CUDA_ARCH__
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+#else
+    return (float)(1.0 / sqrt((double)x)) T7_HOST_ERR;
+#endif
+}
+
+// --------------------------------------------------------------------------
+// Correctly rounded FP64 quotient and square root without FP64 instructions
+// (as FP64 code they take 140 to 165 cycles per warp and SM): a quotient of
+// some 43 bits from FP32, its exact remainder modulo 2^64 from 32-bit integer
+// products, one integer correction, and the remainder's comparison with half
+// the divisor for the last bit.  No result lies on a rounding tie (a 54-bit
+// quotient or root of 53-bit numbers never ends there).  Operands or results
+// that are zero, subnormal, infinite or NaN go to the FP64 operation (zero
+// numerators, common in resting gas, are answered at once).
+//
+// Quotient, with A, B the 53-bit mantissas and s = 1 if A < B, else 0: the FP32
+// pair (qh, ql) approximates A/B within 2^-44, so Q0 = the integer nearest to it
+// times 2^(52+s) is within 2^10 of A 2^(52+s) / B and the remainder
+// A 2^(52+s) - Q0 B below 2^63; the FP32 correction then leaves a remainder of
+// at most B (1/2 + 2^-10).
+// --------------------------------------------------------------------------
+T7_HD double div64(double a, double b) {
+    const uint64_t xa = f64_bits(a), xb = f64_bits(b);
+    const uint32_t ha = (uint32_t)(xa >> 32), hb = (uint32_t)(xb >> 32), la = (uint32_t)xa, lb = (uint32_t)xb;
+    const int ea = (int)((ha >> 20) & 0x7ffu), eb = (int)((hb >> 20) & 0x7ffu);
+    const uint32_t ma = (ha & 0xfffffu) | 0x100000u, mb = (hb & 0xfffffu) | 0x100000u;
+    const uint32_t sign = (ha ^ hb) & 0x80000000u;
+    const int s = (ma < mb || (ma == mb && la < lb)) ? 1 : 0;
+    const int e = ea - eb + 1022 - s;  // exponent field of the result, less one
+    if ((uint32_t)(ea - 1) >= 2046u || (uint32_t)(eb - 1) >= 2046u || (uint32_t)(e - 1) >= 2044u) {
+        if (((ha << 1) | la) == 0u && (uint32_t)(eb - 1) < 2046u) return f64_of((uint64_t)sign << 32);
+        return a / b;
+    }
+    // leading 24 bits in [1, 2) and the other 29
+    const float ah = f32_of(0x3f800000u | ((ma << 3) & 0x7fffffu) | (la >> 29));
+    const float bh = f32_of(0x3f800000u | ((mb << 3) & 0x7fffffu) | (lb >> 29));
+    const float al = (float)(la & 0x1fffffffu) * 2.220446049250313e-16f;
+    const float bl = (float)(lb & 0x1fffffffu) * 2.220446049250313e-16f;
+    float r = f32_rcp(bh);
+    r = fmaf(r, fmaf(-r, bl, fmaf(-r, bh, 1.f)), r);  // 1/B within 2^-23
+    const float qh = ah * r;
+    const float ql = fmaf(-qh, bl, fmaf(-qh, bh, ah) + al) * r;
+    const int ih = (int)(qh * 16777216.f);                              // exact (qh > 1/2)
+    const int il = f32_to_int(ql * (s ? 35184372088832.f : 17592186044416.f));  // ql 2^(44+s)
+    const uint64_t Q0 = ((uint64_t)(uint32_t)ih << (28 + s)) + ((uint64_t)(int64_t)il << 8);
+    const uint32_t q0 = (uint32_t)Q0, q1 = (uint32_t)(Q0 >> 32);
+    const uint64_t A = (uint64_t)(la << (20 + s)) << 32;  // A 2^(52+s) mod 2^64
+    const uint64_t R = A - ((uint64_t)q0 * lb + ((uint64_t)(q0 * mb + q1 * lb) << 32));
+    const int c = f32_to_int((float)(int32_t)(R >> 32) * r * 9.5367431640625e-07f);  // R / B
+    const uint64_t B = ((uint64_t)mb << 32) | lb;
+    const int64_t R1 = (int64_t)(R - (uint64_t)(int64_t)c * B);
+    const int64_t twice = R1 * 2;
+    uint64_t Q = Q0 + (uint64_t)(int64_t)c;
+    if (twice > (int64_t)B) Q++;
+    if (twice < -(int64_t)B) Q--;
+    return f64_of(((uint64_t)(sign | ((uint32_t)e << 20)) << 32) + Q);
+}
+
+// Square root of M 2^52, M = m 2^52 with m in [1, 4) and an even exponent: S0
+// within 2^9 of it, the remainder M 2^52 - S0^2 modulo 2^64, one correction, and
+// the last bit from M 2^52 <> (S +- 1/2)^2.
+T7_HD double sqrt64(double x) {
+    const uint64_t b = f64_bits(x);
+    const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
+    const int e = (int)(hi >> 20);  // sign included
+    if ((uint32_t)(e - 1) >= 2046u) return sqrt(x);
+    const int odd = (e & 1) ^ 1;  // the bias 1023 is odd
+    const uint32_t m = (hi & 0xfffffu) | 0x100000u;
+    const float scale = odd ? 2.f : 1.f;
+    const float mh = f32_of(0x3f800000u | ((m << 3) & 0x7fffffu) | (lo >> 29)) * scale;
+    const float ml = (float)(lo & 0x1fffffffu) * 2.220446049250313e-16f * scale;
+    float y = f32_rsqrt(mh);
+    float sh = mh * y;
+    y = fmaf(0.5f * y, fmaf(-sh, y, 1.f), y);
+    sh = mh * y;
+    const float sl = (fmaf(-sh, sh, mh) + ml) * (0.5f * y);
+    const int ih = (int)(sh * 16777216.f);                // exact (sh > 1/2)
+    const int il = f32_to_int(sl * 4503599627370496.f);  // sl 2^52
+    const uint64_t S0 = ((uint64_t)(uint32_t)ih << 28) + (uint64_t)(int64_t)il;
+    const uint32_t s0 = (uint32_t)S0, s1 = (uint32_t)(S0 >> 32);
+    const uint64_t M = (uint64_t)(lo << (20 + odd)) << 32;
+    const uint64_t R = M - ((uint64_t)s0 * s0 + ((uint64_t)(2u * s0 * s1) << 32));
+    const int c = f32_to_int((float)(int32_t)(R >> 32) * y * 4.76837158203125e-07f);  // R / (2 S)
+    const uint64_t cc = (uint64_t)(int64_t)c;
+    uint64_t S = S0 + cc;
+    const int64_t R1 = (int64_t)(R - cc * (2u * S0 + cc));
+    if (R1 > (int64_t)S) S++;
+    else if (R1 <= -(int64_t)S) S--;
+    return f64_of(((uint64_t)(uint32_t)(((e - 1023 - odd) >> 1) + 1022) << 52) + S);
 }
 
 // --------------------------------------------------------------------------

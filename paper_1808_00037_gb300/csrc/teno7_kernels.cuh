@@ -259,9 +259,9 @@ __device__ __forceinline__ T wavespeed1d(const T *Uc, T gm1, T gamma, T a, int *
     }
     T u, p, c;
     if constexpr (sizeof(T) == 8) {
-        u = Uc[1] / Uc[0];
+        u = div64(Uc[1], Uc[0]);
         p = gm1 * __fma_rn(-0.5, Uc[1] * u, Uc[2]);  // U2 - (U1/2) u, the half exact
-        c = sq_root(gamma * p / Uc[0]);
+        c = sqrt64(div64(gamma * p, Uc[0]));
     } else {
         const float ri = __frcp_rn(Uc[0]);
         u = Uc[1] * ri;
@@ -279,9 +279,9 @@ template <typename T>
 __device__ __forceinline__ void wavespeeds1d(const T *Uc, T gm1, T gamma, T w[3], int *flag) {
     T u, p, c;
     if constexpr (sizeof(T) == 8) {
-        u = Uc[1] / Uc[0];
+        u = div64(Uc[1], Uc[0]);
         p = gm1 * __fma_rn(-0.5, Uc[1] * u, Uc[2]);
-        c = sq_root(gamma * p / Uc[0]);
+        c = sqrt64(div64(gamma * p, Uc[0]));
     } else {
         const float ri = __frcp_rn(Uc[0]);
         u = Uc[1] * ri;
@@ -463,7 +463,7 @@ constexpr int FLUX_SCALE_EULER = 4, FLUX_SCALE_SCALAR = 2;
 
 // Flux F, velocity u, total enthalpy H and sqrt(rho) of a state.
 __device__ __forceinline__ void cell1d_f64(const double U[3], double gm1, double F[3], double pr[3]) {
-    const double u = U[1] / U[0];
+    const double u = div64(U[1], U[0]);
     const double m = U[1] * u;
     const double p = gm1 * __fma_rn(-0.5, m, U[2]);
     const double e = U[2] + p;
@@ -471,8 +471,8 @@ __device__ __forceinline__ void cell1d_f64(const double U[3], double gm1, double
     F[1] = m + p;
     F[2] = u * e;
     pr[0] = u;
-    pr[1] = e / U[0];
-    pr[2] = sqrt(U[0]);
+    pr[1] = div64(e, U[0]);
+    pr[2] = sqrt64(U[0]);
 }
 
 // Roe frame of a face: rows 0 and 2 of L doubled (l0, l2; their third entry is
@@ -485,14 +485,14 @@ __device__ __forceinline__ Roe64 roe_frame_f64(double ul, double ur, double Hl, 
                                                double gm1) {
     Roe64 R;
     const double S = sl + sr;
-    R.ut = (sl * ul + sr * ur) / S;
-    R.Ht = (sl * Hl + sr * Hr) / S;
+    R.ut = div64(sl * ul + sr * ur, S);
+    R.Ht = div64(sl * Hl + sr * Hr, S);
     R.X = R.ut * R.ut;
     const double c2 = gm1 * __fma_rn(-0.5, R.X, R.Ht);
-    R.cc = sqrt(c2);
-    R.b1 = gm1 / c2;
+    R.cc = sqrt64(c2);
+    R.b1 = div64(gm1, c2);
     const double t = R.X * R.b1;  // 2 b2
-    const double uc = R.ut / R.cc, rc = 1.0 / R.cc;
+    const double uc = div64(R.ut, R.cc), rc = div64(1.0, R.cc);
     const double b1u = R.b1 * R.ut;
     R.l0[0] = __fma_rn(0.5, t, uc);
     R.l0[1] = -(b1u + rc);
@@ -703,7 +703,7 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
             const int ii = chk(ctl, i, 0, n);
             T r[M];
 #pragma unroll
-            for (int k = 0; k < M; k++) r[k] = (fprev[k] - fh[k]) / dxs;
+            for (int k = 0; k < M; k++) r[k] = div64(fprev[k] - fh[k], dxs);
             if (A.rhs_mode) {
 #pragma unroll
                 for (int k = 0; k < M; k++) out[(size_t)k * A.cso + ii] = r[k];

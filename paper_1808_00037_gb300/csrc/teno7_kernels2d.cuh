@@ -53,15 +53,15 @@ template <typename PR>
 __device__ __forceinline__ Roe2D64 roe_frame2d_f64(PR pr, double gm1) {
     Roe2D64 R;
     const double sl = pr(3, 3), sr = pr(3, 4), S = sl + sr;
-    R.un = (sl * pr(0, 3) + sr * pr(0, 4)) / S;
-    R.vt = (sl * pr(1, 3) + sr * pr(1, 4)) / S;
-    R.Ht = (sl * pr(2, 3) + sr * pr(2, 4)) / S;
+    R.un = div64(sl * pr(0, 3) + sr * pr(0, 4), S);
+    R.vt = div64(sl * pr(1, 3) + sr * pr(1, 4), S);
+    R.Ht = div64(sl * pr(2, 3) + sr * pr(2, 4), S);
     R.X = R.un * R.un + R.vt * R.vt;
     const double c2 = gm1 * __fma_rn(-0.5, R.X, R.Ht);
-    R.cc = sqrt(c2);
-    R.b1 = gm1 / c2;
+    R.cc = sqrt64(c2);
+    R.b1 = div64(gm1, c2);
     const double t = R.X * R.b1;  // 2 b2
-    const double uc = R.un / R.cc, rc = 1.0 / R.cc;
+    const double uc = div64(R.un, R.cc), rc = div64(1.0, R.cc);
     const double b1u = R.b1 * R.un;
     R.b1v = R.b1 * R.vt;
     R.l0[0] = __fma_rn(0.5, t, uc);
@@ -161,8 +161,8 @@ __device__ __forceinline__ int face2d_f64(PR pr, G g, double gm1, const Cut64 &c
 template <int DIR>
 __device__ __forceinline__ void cell2d_f64(const double U[4], double gm1, double alpha, double prim[4], double gp[4],
                                            double gm[4]) {
-    const double u = U[1] / U[0];
-    const double v = U[2] / U[0];
+    const double u = div64(U[1], U[0]);
+    const double v = div64(U[2], U[0]);
     const double mu = U[1] * u, mv = U[2] * v;
     const double p = gm1 * __fma_rn(-0.5, mu + mv, U[3]);
     const double e = U[3] + p;
@@ -182,8 +182,8 @@ __device__ __forceinline__ void cell2d_f64(const double U[4], double gm1, double
         prim[0] = v;
         prim[1] = u;
     }
-    prim[2] = e / U[0];
-    prim[3] = sqrt(U[0]);
+    prim[2] = div64(e, U[0]);
+    prim[3] = sqrt64(U[0]);
 #pragma unroll
     for (int k = 0; k < 4; k++) {
         const double aU = alpha * U[k];
@@ -197,15 +197,17 @@ __device__ __forceinline__ void cell2d_f64(const double U[4], double gm1, double
 // compiler), so that every instantiation of a kernel gives the same bits.
 template <typename T>
 __device__ __forceinline__ void wavespeed2d(const T U[4], T gm1, T gamma, T &sx, T &sy, int *flag) {
-    const T u = U[1] / U[0];
-    const T v = U[2] / U[0];
-    T p, c;
+    T u, v, p, c;
     if constexpr (sizeof(T) == 4) {
+        u = U[1] / U[0];
+        v = U[2] / U[0];
         p = __fmul_rn(gm1, __fmaf_rn(-0.5f, __fmaf_rn(U[1], u, __fmul_rn(U[2], v)), U[3]));
         c = sqrtf(__fdiv_rn(__fmul_rn(gamma, p), U[0]));
     } else {
+        u = div64(U[1], U[0]);
+        v = div64(U[2], U[0]);
         p = gm1 * __fma_rn(-0.5, U[1] * u + U[2] * v, U[3]);
-        c = sq_root(gamma * p / U[0]);
+        c = sqrt64(div64(gamma * p, U[0]));
     }
     // a non-finite cell is reported as such; a finite one needs rho > 0, p > 0
     if constexpr (sizeof(T) == 8) {
@@ -348,7 +350,7 @@ __global__ void __launch_bounds__(WPB * 32, 1) xsweep2d_kernel(const Stage2D p) 
         if (lane >= 2 && lane <= 30 && j < nx) {
 #pragma unroll
             for (int k = 0; k < 4; k++) {
-                const T r = (fprev[k] - fh[k]) / dx4;
+                const T r = div64(fprev[k] - fh[k], dx4);
                 R[(size_t)k * N + (size_t)y * nx + chk(p.ctl, j, 0, p.nx)] = r;
             }
         }
@@ -439,7 +441,7 @@ __global__ void __launch_bounds__(WPB * 32, 1) ysweep2d_kernel(const Stage2D p) 
         if (lane >= 2 && lane <= 30) {
 #pragma unroll
             for (int k = 0; k < 4; k++) {
-                const T r = (fprev[k] - fh[k]) / dy4;
+                const T r = div64(fprev[k] - fh[k], dy4);
                 s_ry[(k * YB_ROWS + (lane - 2)) * YB_LD + col] = r;
             }
         }

@@ -3,6 +3,10 @@
 #include <cstdio>
 #include <random>
 
+// the device's approximate reciprocal and root are off by up to 2^-22: check at
+// both ends of that
+static float host_err = 1.f;
+#define T7_HOST_ERR *host_err
 #include "teno7_f64math.cuh"
 
 using namespace t7;
@@ -52,7 +56,56 @@ static void check_cutoff() {
     printf("cutoff_special %ld %ld\n", total, bad);
 }
 
+static bool same(double x, double y) { return f64_bits(x) == f64_bits(y) || (x != x && y != y); }
+
+// quotients and roots: random mantissas (short and long) and exponents, results
+// around powers of two, operands next to exact results, and special values
+static void check_div_sqrt() {
+    std::mt19937_64 r(11);
+    long nd = 0, bd = 0, ns = 0, bs = 0;
+    auto mantissa = [&](int kind) {
+        uint64_t m = r() & 0xfffffffffffffull;
+        if (kind == 1) m &= ~0ull << (r() % 52);
+        if (kind == 2) m = 0xfffffffffffffull - (m >> (20 + r() % 32));
+        if (kind == 3) m >>= 20 + r() % 32;
+        return m;
+    };
+    for (float err : {1.f, 1.f + 2.4e-7f, 1.f - 2.4e-7f}) {
+        host_err = err;
+        for (int i = 0; i < 3000000; i++) {
+            const int spread = i % 16 == 0 ? 1000 : 40;
+            auto draw = [&](int kind) {
+                const uint64_t e = 1023 - spread + r() % (2 * spread + 1);
+                return f64_of(((r() & 1) << 63) | (e << 52) | mantissa(kind));
+            };
+            double a = draw(i % 4), b = draw((i / 4) % 4);
+            if (i % 5 == 1) a = b * f64_of(f64_bits(a));                      // a quotient near a double
+            if (i % 5 == 2) a = f64_of(f64_bits(b * a) + r() % 3 - 1);        // and one beside it
+            if (i % 5 == 3) a = f64_of(f64_bits(b) + r() % 5 - 2);            // near one
+            nd++;
+            bd += !same(div64(a, b), a / b);
+            double x = fabs(a);
+            if (i % 3 == 1) x = b * b;
+            if (i % 3 == 2) x = f64_of(f64_bits(b * b) + r() % 5 - 2);
+            ns++;
+            bs += !same(sqrt64(x), sqrt(x));
+        }
+        const double s[] = {0.0, -0.0, 5e-324, 1e-310, 2.2250738585072014e-308, 1e-300, 0.5, 1.0, 1.5, 2.0, 3.0, 4.0,
+                            1e300, 1.7976931348623157e308, INFINITY, NAN, -1.0, -1e-310, -INFINITY};
+        for (double a : s) {
+            ns++;
+            bs += !same(sqrt64(a), sqrt(a));
+            for (double b : s) {
+                nd++;
+                bd += !same(div64(a, b), a / b);
+            }
+        }
+    }
+    printf("div %ld %ld\nsqrt %ld %ld\n", nd, bd, ns, bs);
+}
+
 int main() {
     check_cutoff();
+    check_div_sqrt();
     return 0;
 }
