@@ -180,6 +180,56 @@ T7_HD double sqrt64(double x) {
 }
 
 // --------------------------------------------------------------------------
+// Correctly rounded FP64 product on the integer pipe: four 32 x 32 -> 64-bit
+// products of the mantissas, rounded to nearest even from the exact 117 bits.
+// About 24 integer instructions (12 cycles per warp and SM, against 19 on the
+// FP64 pipe, which meanwhile runs the sums).  One factor is prepared once
+// (MulOp: mantissa left-justified in 64 bits, sign and exponent word less the
+// bias); it may be zero.  The other, and a nonzero prepared one, must have a
+// magnitude in [2^-400, 2^400): mul_ranged().
+// --------------------------------------------------------------------------
+struct MulOp {
+    uint32_t xl, xh, e, mask;
+};
+// 0 when |x| is in [2^-400, 2^400), so that results of several values can be or-ed
+T7_HD uint32_t mul_unranged(double x) {
+    const uint32_t a = (uint32_t)(f64_bits(x) >> 32) & 0x7fffffffu;
+    return a - ((1023u - 400u) << 20) >= (800u << 20) ? 1u : 0u;
+}
+T7_HD MulOp mul_op(double x) {
+    const uint64_t b = f64_bits(x);
+    const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
+    MulOp o;
+    o.mask = ((hi << 1) | lo) == 0u ? 0u : ~0u;
+    o.xh = ((((hi & 0xfffffu) | 0x100000u) << 11) | (lo >> 21)) & o.mask;
+    o.xl = lo << 11;
+    o.e = (hi & 0xfff00000u) - 0x40000000u;
+    return o;
+}
+T7_HD double mul64(const MulOp &x, double g) {
+    const uint64_t b = f64_bits(g);
+    const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b, gh = (hi & 0xfffffu) | 0x100000u;
+    const uint64_t p0 = (uint64_t)x.xl * lo;
+    const uint64_t p1 = (uint64_t)x.xh * lo + (p0 >> 32);
+    const uint64_t p2 = (uint64_t)x.xl * gh + (uint32_t)p1;
+    const uint64_t h = (uint64_t)x.xh * gh + (p1 >> 32) + (p2 >> 32);  // product >> 64: 53 or 52 bits
+    const uint32_t hh = (uint32_t)(h >> 32), hl = (uint32_t)h, ll = (uint32_t)p0, lh = (uint32_t)p2;
+    const int s = (hh & 0x100000u) ? 0 : 1;
+    // 53-bit mantissa (mh, ml) and the 64 bits below it (rh, rl)
+#ifdef __CUDA_ARCH__
+    const uint32_t mh = __funnelshift_l(hl, hh, s), ml = __funnelshift_l(lh, hl, s), rh = __funnelshift_l(ll, lh, s);
+#else
+    const uint32_t mh = s ? (hh << 1) | (hl >> 31) : hh, ml = s ? (hl << 1) | (lh >> 31) : hl;
+    const uint32_t rh = s ? (lh << 1) | (ll >> 31) : lh;
+#endif
+    const uint32_t up = ((ml & 1u) | (ll << s)) != 0u ? 0x80000000u : 0x7fffffffu;  // nearest, ties to even
+    const uint64_t carry = ((uint64_t)rh + up) >> 32;
+    const uint64_t m = (((uint64_t)mh << 32) | ml) + carry;
+    const uint32_t rhi = (uint32_t)(m >> 32) + (x.e + (hi & 0xfff00000u) + (hh & 0x100000u));
+    return f64_of(((uint64_t)(rhi & x.mask) << 32) | (uint32_t)m);
+}
+
+// --------------------------------------------------------------------------
 // Shortcut of the cutoff test.  If tau < kt (beta_min + eps), every
 // g_k = 1 + tau / (beta_k + eps) lies in [1, 1 + kt), so
 // chi_k = g_k^6 / sum_j g_j^6 >= 1 / (3 (1 + kt)^6).  With

@@ -433,6 +433,7 @@ struct TileArgs {
     double dtD;      // FP64 step (mixed precision: FP64 state, FP32 reconstruction)
     int rhs_mode, stage;
     int ebase;       // added to cell/face indices in error reports
+    bool imul;       // FP64: products on the integer pipe (see tiles1d)
     int halo;        // the arrays hold HALO_CELLS filled ghost cells per side (slab mode)
     DevCtl *ctl;
 };
@@ -475,10 +476,10 @@ __device__ __forceinline__ void cell1d_f64(const double U[3], double gm1, double
     pr[2] = sqrt64(U[0]);
 }
 
-// Roe frame of a face: rows 0 and 2 of L doubled (l0, l2; their third entry is
-// b1, and row 1's is -b1), the Roe state, and X = u~^2.
+// Roe frame of a face: rows of L, 0 and 2 doubled (their third entry is b1, row
+// 1's is -b1), the Roe state, and X = u~^2.
 struct Roe64 {
-    double l0[2], l1[2], l2[2], b1, ut, cc, Ht, X;
+    double l[3][2], b1, ut, cc, Ht, X;
     int flag;
 };
 __device__ __forceinline__ Roe64 roe_frame_f64(double ul, double ur, double Hl, double Hr, double sl, double sr,
@@ -494,22 +495,29 @@ __device__ __forceinline__ Roe64 roe_frame_f64(double ul, double ur, double Hl, 
     const double t = R.X * R.b1;  // 2 b2
     const double uc = div64(R.ut, R.cc), rc = div64(1.0, R.cc);
     const double b1u = R.b1 * R.ut;
-    R.l0[0] = __fma_rn(0.5, t, uc);
-    R.l0[1] = -(b1u + rc);
-    R.l1[0] = __fma_rn(-0.5, t, 1.0);
-    R.l1[1] = b1u;
-    R.l2[0] = __fma_rn(0.5, t, -uc);
-    R.l2[1] = -(b1u - rc);
+    R.l[0][0] = __fma_rn(0.5, t, uc);
+    R.l[0][1] = -(b1u + rc);
+    R.l[1][0] = __fma_rn(-0.5, t, 1.0);
+    R.l[1][1] = b1u;
+    R.l[2][0] = __fma_rn(0.5, t, -uc);
+    R.l[2][1] = -(b1u - rc);
     R.flag = f64_positive(c2) ? 0 : (f64_finite(c2) ? ERR_NONPHYSICAL : ERR_NONFINITE);
     return R;
 }
 
-// L g (rows 0 and 2 doubled).
-__device__ __forceinline__ void project_f64(const Roe64 &R, double g0, double g1, double g2, double q[3]) {
-    const double p = R.b1 * g2;
-    q[0] = (R.l0[0] * g0 + R.l0[1] * g1) + p;
-    q[1] = (R.l1[0] * g0 + R.l1[1] * g1) - p;
-    q[2] = (R.l2[0] * g0 + R.l2[1] * g1) + p;
+// A factor of a frame mul64 does not take (zero it does).
+__device__ __forceinline__ uint32_t factor_unranged(double x) { return x != 0.0 ? mul_unranged(x) : 0u; }
+
+// poly_f0 with its products on the integer pipe (every tap in mul64's range)
+__device__ __forceinline__ double poly_f0_imul(const double v[7]) {
+    double s = mul64(mul_op(-1.0 / 140.0), v[0]);
+    s = s + mul64(mul_op(5.0 / 84.0), v[1]);
+    s = s + mul64(mul_op(-101.0 / 420.0), v[2]);
+    s = s + mul64(mul_op(319.0 / 420.0), v[3]);
+    s = s + mul64(mul_op(107.0 / 210.0), v[4]);
+    s = s + mul64(mul_op(-19.0 / 210.0), v[5]);
+    s = s + mul64(mul_op(1.0 / 105.0), v[6]);
+    return s;
 }
 
 // R f for f[0], f[2] scaled by 4 and f[1] by 2: the face flux scaled by 4.
@@ -536,8 +544,11 @@ __device__ __forceinline__ double rk_combine_f64(int stage, double us, double dt
 // Bound by the FP64 pipe (one warp instruction per 19 cycles and SM, against 2
 // to 4 per cycle for the others): the two splits run through one loop body, each
 // as seven upwind-ordered taps, and a split whose staged fluxes are all zero
-// (advection: F - alpha U for a > 0) is not reconstructed.
-template <typename T, int SYS, int SCH = SCH_TENO7EXT, bool PF = false>
+// (advection: F - alpha U for a > 0) is not reconstructed.  NF fields are
+// projected together: one (128 registers, 16 warps per SM, products by mul64
+// where A.imul allows and the values are in its range; at 1M cells the FP64 pipe
+// is 69% busy, issue 41%) or all three (8 warps, FP64 products, the third shared).
+template <typename T, int SYS, int SCH = SCH_TENO7EXT, bool PF = false, int NF = 1>
 __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)[WC], T (*sgm)[WC], T (*spr)[WC],
                                      const T *scoef, int tile0, int tstride, int tile_end = 0x7fffffff,
                                      T *ws3 = nullptr) {
@@ -560,6 +571,7 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
         const int c0 = tile * WT;
         // ---- stage cells c0-5 .. c0+33 -----------------------------------
         bool zero[2] = {M == 1 && A.kt > T(0), M == 1 && A.kt > T(0)};  // scalar laws: a split vanishes
+        uint32_t unranged = 0u;  // a value mul64 does not take
         for (int c = lane; c < WS; c += 32) {
             int gi = c0 - 5 + c;
             if (gi < 0 || gi >= n) gi = ghost_or_halo(gi, n, A.bc_lo, A.bc_hi, A.halo);
@@ -589,6 +601,7 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
                     sgm[k][c] = gm;
                     zero[0] = zero[0] && f64_bits(gp) == 0;
                     zero[1] = zero[1] && f64_bits(gm) == 0;
+                    if (M == 3) unranged |= mul_unranged(gp) | mul_unranged(gm);
                 }
             }
         }
@@ -604,85 +617,125 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
             R = roe_frame_f64(spr[0][lane + 3], spr[0][lane + 4], spr[1][lane + 3], spr[1][lane + 4],
                               spr[2][lane + 3], spr[2][lane + 4], gm1);
             flag = R.flag;
+            unranged |= mul_unranged(R.b1);
+#pragma unroll
+            for (int k = 0; k < 3; k++) unranged |= factor_unranged(R.l[k][0]) | factor_unranged(R.l[k][1]);
         }
+        const bool imul = A.imul && !__any_sync(0xffffffffu, unranged != 0u);
         T f[M];
 #pragma unroll 1
         for (int s = 0; s < 2; s++) {
-            T fs[M];
-            unsigned D[M];  // codes
-            if (M == 1 && !PF && __all_sync(0xffffffffu, s == 0 ? zero[0] : zero[1])) {
-                // every window of the split is zero: all stencils kept, flux +0
-                fs[0] = T(0);
-                D[0] = SCH == SCH_TENO5 ? 7u : 31u;
-            } else {
-                // taps in upwind order: '+' cells j-3+t, '-' cells j+4-t
-                T (*sg)[WC] = (PF || s == 0) ? sgp : sgm;
-                const int o = s == 0 ? lane : lane + 7, dir = s == 0 ? 1 : -1;
-                T P[M][7];
-                unsigned word = 0;
+            // taps in upwind order: '+' cells j-3+t, '-' cells j+4-t
+            T (*sg)[WC] = (PF || s == 0) ? sgp : sgm;
+            const int o = s == 0 ? lane : lane + 7, dir = s == 0 ? 1 : -1;
+            // every window of the split zero: all stencils kept, flux +0
+            const bool vanishes = M == 1 && !PF && __all_sync(0xffffffffu, s == 0 ? zero[0] : zero[1]);
 #pragma unroll
-                for (int t = 0; t < 7; t++) {
-                    const int c = o + dir * t;
-                    if constexpr (M == 1) {
-                        P[0][t] = sg[0][c];
-                    } else if (SCH == SCH_TENO5 && (t == 0 || t == 6)) {  // five-point stencils
-                        P[0][t] = P[1][t] = P[2][t] = T(0);
-                    } else {
-                        T q[3];
-                        project_f64(R, sg[0][c], sg[1][c], sg[2][c], q);
-                        if constexpr (PF) {
-                            T qu[3];
-                            project_f64(R, sU[0][c], sU[1][c], sU[2][c], qu);
+            for (int k0 = 0; k0 < M; k0 += NF) {
+                T P[NF][7];
+                if (vanishes) {
+                } else if constexpr (M == 1) {
 #pragma unroll
-                            for (int k = 0; k < 3; k++)
-                                q[k] = s == 0 ? q[k] + A.alf[k] * qu[k] : q[k] - A.alf[k] * qu[k];
+                    for (int t = 0; t < 7; t++) P[0][t] = sg[0][o + dir * t];
+                } else if constexpr (PF) {
+#pragma unroll
+                    for (int t = 0; t < 7; t++) {
+                        const int c = o + dir * t;
+#pragma unroll
+                        for (int i = 0; i < NF; i++) {
+                            const int k = k0 + i;
+                            const T b = k == 1 ? -R.b1 : R.b1;
+                            const T lf = (R.l[k][0] * sg[0][c] + R.l[k][1] * sg[1][c]) + b * sg[2][c];
+                            const T lu = (R.l[k][0] * sU[0][c] + R.l[k][1] * sU[1][c]) + b * sU[2][c];
+                            P[i][t] = s == 0 ? lf + A.alf[k] * lu : lf - A.alf[k] * lu;
                         }
+                    }
+                } else if (NF == 1 && imul) {
+                    const MulOp b = mul_op(R.b1);
+                    MulOp m0[NF], m1[NF];
 #pragma unroll
-                        for (int k = 0; k < 3; k++) P[k][t] = q[k];
+                    for (int i = 0; i < NF; i++) {
+                        m0[i] = mul_op(R.l[k0 + i][0]);
+                        m1[i] = mul_op(R.l[k0 + i][1]);
+                    }
+#pragma unroll
+                    for (int t = 0; t < 7; t++) {
+                        const int c = o + dir * t;
+                        if (SCH == SCH_TENO5 && (t == 0 || t == 6)) continue;  // five-point stencils
+                        const T g0 = sg[0][c], g1 = sg[1][c], p = mul64(b, sg[2][c]);
+#pragma unroll
+                        for (int i = 0; i < NF; i++)
+                            P[i][t] = (mul64(m0[i], g0) + mul64(m1[i], g1)) + (k0 + i == 1 ? -p : p);
+                    }
+                } else {
+#pragma unroll
+                    for (int t = 0; t < 7; t++) {
+                        const int c = o + dir * t;
+                        if (SCH == SCH_TENO5 && (t == 0 || t == 6)) continue;
+                        const T g0 = sg[0][c], g1 = sg[1][c], p = R.b1 * sg[2][c];
+#pragma unroll
+                        for (int i = 0; i < NF; i++)
+                            P[i][t] = (R.l[k0 + i][0] * g0 + R.l[k0 + i][1] * g1) + (k0 + i == 1 ? -p : p);
                     }
                 }
+                unsigned word = 0;
+                if (!vanishes) {
 #pragma unroll
-                for (int k = 0; k < M; k++)
-                    word |= cutoff_bits(P[k][1], P[k][2], P[k][3], P[k][4], P[k][5],
-                                        M == 3 && k != 1 ? cut4 : cut2)
-                            << (3 * k);
-                if constexpr (SCH == SCH_TENO5) {
-                    // the face's own code picks a Table co1 row on the taps 1 .. 5
+                    for (int i = 0; i < NF; i++)
+                        word |= cutoff_bits(P[i][1], P[i][2], P[i][3], P[i][4], P[i][5],
+                                            M == 3 && k0 + i != 1 ? cut4 : cut2)
+                                << (3 * i);
+                }
+                constexpr unsigned KEPT = (1u << (3 * NF)) - 1u;
+                const bool smooth = vanishes || __all_sync(0xffffffffu, word == KEPT);
+                unsigned wu = word, wd = word;  // upwind and downwind neighbour faces
+                if (SCH != SCH_TENO5 && !smooth) {
+                    const unsigned wl = __shfl_up_sync(0xffffffffu, word, 1);
+                    const unsigned wr = __shfl_down_sync(0xffffffffu, word, 1);
+                    wu = s == 0 ? wl : wr;
+                    wd = s == 0 ? wr : wl;
+                }
 #pragma unroll
-                    for (int k = 0; k < M; k++) {
-                        D[k] = (word >> (3 * k)) & 7u;
-                        int r = sel5(D[k]);
+                for (int i = 0; i < NF; i++) {
+                    const int k = k0 + i;
+                    T fs = T(0);
+                    unsigned D = SCH == SCH_TENO5 ? 7u : 31u;
+                    if (vanishes) {
+                    } else if constexpr (SCH == SCH_TENO5) {
+                        // the face's own code picks a Table co1 row on the taps 1 .. 5
+                        D = (word >> (3 * i)) & 7u;
+                        int r = sel5(D);
                         if (r == 7) {
                             r = 0;
                             if (face_out) flag |= ERR_NOEXIST;
                         }
-                        fs[k] = poly5(scoef + 5 * r, P[k][1], P[k][2], P[k][3], P[k][4], P[k][5]);
-                    }
-                } else {
-                    const unsigned wl = __shfl_up_sync(0xffffffffu, word, 1);
-                    const unsigned wr = __shfl_down_sync(0xffffffffu, word, 1);
-                    const unsigned wu = s == 0 ? wl : wr, wd = s == 0 ? wr : wl;  // upwind, downwind face
-#pragma unroll
-                    for (int k = 0; k < M; k++) {
-                        D[k] = (unsigned)pack_delta(wu >> (3 * k), word >> (3 * k), wd >> (3 * k));
-                        int m = lut_select((int)D[k]);
-                        if (m == 15) {
-                            m = 11;
-                            if (face_out) flag |= ERR_NOEXIST;
+                        fs = poly5(scoef + 5 * r, P[i][1], P[i][2], P[i][3], P[i][4], P[i][5]);
+                    } else {
+                        int m = 0;
+                        if (!smooth) {
+                            D = (unsigned)pack_delta(wu >> (3 * i), word >> (3 * i), wd >> (3 * i));
+                            m = lut_select((int)D);
+                            if (m == 15) {
+                                m = 11;
+                                if (face_out) flag |= ERR_NOEXIST;
+                            }
                         }
-                        if (m == 0)
-                            fs[k] = poly_f0(P[k][0], P[k][1], P[k][2], P[k][3], P[k][4], P[k][5], P[k][6]);
-                        else
-                            fs[k] = poly7(scoef + 7 * m, P[k][0], P[k][1], P[k][2], P[k][3], P[k][4], P[k][5],
-                                          P[k][6]);
-                    }
-                }
-            }
+                        uint32_t bad = (uint32_t)m;
+                        if (NF == 1 && A.imul) {
 #pragma unroll
-            for (int k = 0; k < M; k++) {
-                f[k] = s == 0 ? fs[k] : f[k] + fs[k];
-                if (A.masks && face_out && j >= -1 && j <= n - 1)
-                    A.masks[(size_t)(s * M + k) * (n + 1) + (j + 1)] = (uint8_t)D[k];
+                            for (int t = 0; t < 7; t++) bad |= mul_unranged(P[i][t]);
+                        }
+                        if (__any_sync(0xffffffffu, bad != 0u))
+                            fs = poly7(scoef + 7 * m, P[i][0], P[i][1], P[i][2], P[i][3], P[i][4], P[i][5], P[i][6]);
+                        else if (NF == 1 && A.imul)
+                            fs = poly_f0_imul(P[i]);
+                        else
+                            fs = poly_f0(P[i][0], P[i][1], P[i][2], P[i][3], P[i][4], P[i][5], P[i][6]);
+                    }
+                    f[k] = s == 0 ? fs : f[k] + fs;
+                    if (A.masks && face_out && j >= -1 && j <= n - 1)
+                        A.masks[(size_t)(s * M + k) * (n + 1) + (j + 1)] = (uint8_t)D;
+                }
             }
         }
         T fh[M];
@@ -736,8 +789,8 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
 // ==========================================================================
 // Fused 1D stage kernel (grid-wide), SYS in {SYS_ADV, SYS_BURGERS, SYS_EULER1D}.
 // ==========================================================================
-template <typename T, int SYS, int SCH, bool PF = false>
-__global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 ? 2 : 1)) stage1d_kernel(const Stage1D p) {
+template <typename T, int SYS, int SCH, bool PF = false, int NF = 1>
+__global__ void __launch_bounds__(WPB * 32, NF == 1 ? 2 : 1) stage1d_kernel(const Stage1D p) {
     constexpr int M = (SYS == SYS_EULER1D) ? 3 : 1;
     constexpr int NP = (SYS == SYS_EULER1D) ? 3 : 1;
     __shared__ T s_U[WPB][M][WC];
@@ -792,13 +845,14 @@ __global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 ? 2 : 1)) stage1d_ke
     A.rhs_mode = p.rhs_mode;
     A.stage = p.stage;
     A.ebase = 0;
+    A.imul = NF == 1 && nw == WPB;
     A.ctl = ctl;
     __syncwarp();
     constexpr int NA = PF ? 3 : 1;
     T ws[NA];
 #pragma unroll
     for (int q = 0; q < NA; q++) ws[q] = T(0);
-    const T w0 = tiles1d<T, SYS, SCH, PF>(A, s_U[warp], s_gp[warp], s_gm[warp], s_pr[warp], s_coef[warp],
+    const T w0 = tiles1d<T, SYS, SCH, PF, NF>(A, s_U[warp], s_gp[warp], s_gm[warp], s_pr[warp], s_coef[warp],
                                           p.tile_lo + blockIdx.x * nw + warp, gridDim.x * nw,
                                           p.tile_hi > 0 ? p.tile_hi : 0x7fffffff, ws);
     if constexpr (!PF) ws[0] = w0;
@@ -2319,6 +2373,13 @@ cudaError_t launch_stage1d(const Stage1D &p_, cudaStream_t st) {
         if (grid > resident) grid = resident;
         if (p.scheme != SCH_TENO7EXT && p.scheme != SCH_TENO5) return cudaErrorInvalidValue;
         const bool t5 = p.scheme == SCH_TENO5;
+        // Eight tiles per SM and more fill two CTAs per SM, for which one field at
+        // a time leaves the registers and whose products go to the integer pipe
+        // (Euler, 20 steps: 40,000 cells 4.3 -> 3.0 ms; 1M cells, 2 steps: 5.08 ->
+        // 4.10 ms); below, few warps share an SM, each waits on its own chain, and
+        // all fields together with FP64 products are shorter (1600 cells, 256
+        // steps: 18.0 against 20.2 ms).
+        const bool many = ntiles >= 8 * num_sms();
         if (p.alpha_mode) {  // per-field alphas: 1D Euler with TENO7-ext only
             if (p.sys != SYS_EULER1D || t5) return cudaErrorInvalidValue;
             stage1d_kernel<T, SYS_EULER1D, SCH_TENO7EXT, true><<<grid, nw * 32, 0, st>>>(p);
@@ -2334,8 +2395,10 @@ cudaError_t launch_stage1d(const Stage1D &p_, cudaStream_t st) {
                 else stage1d_kernel<T, SYS_BURGERS, SCH_TENO7EXT><<<grid, nw * 32, 0, st>>>(p);
                 break;
             case SYS_EULER1D:
-                if (t5) stage1d_kernel<T, SYS_EULER1D, SCH_TENO5><<<grid, nw * 32, 0, st>>>(p);
-                else stage1d_kernel<T, SYS_EULER1D, SCH_TENO7EXT><<<grid, nw * 32, 0, st>>>(p);
+                if (t5 && many) stage1d_kernel<T, SYS_EULER1D, SCH_TENO5><<<grid, nw * 32, 0, st>>>(p);
+                else if (t5) stage1d_kernel<T, SYS_EULER1D, SCH_TENO5, false, 3><<<grid, nw * 32, 0, st>>>(p);
+                else if (many) stage1d_kernel<T, SYS_EULER1D, SCH_TENO7EXT><<<grid, nw * 32, 0, st>>>(p);
+                else stage1d_kernel<T, SYS_EULER1D, SCH_TENO7EXT, false, 3><<<grid, nw * 32, 0, st>>>(p);
                 break;
             default: return cudaErrorInvalidValue;
         }
@@ -2466,6 +2529,7 @@ __global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 ? 2 : 1)) batch1d_ke
         A.rhs_mode = 0;
         A.ebase = (int)off;
         A.halo = 0;
+        A.imul = false;
         A.ctl = p.ctl;
         A.U0 = U + off;
         T *ins[3] = {U + off, W1 + off, W2 + off};
@@ -2485,7 +2549,7 @@ __global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 ? 2 : 1)) batch1d_ke
                 A.alpha = alpha;
                 T ws;
                 if constexpr (F64) {
-                    ws = tiles1d<T, SYS_EULER1D>(A, s_U[warp], s_gp[warp], s_gm[warp], s_pr[warp], s_coef[warp], wg, G);
+                    ws = tiles1d<T, SYS_EULER1D, SCH_TENO7EXT, false, 3>(A, s_U[warp], s_gp[warp], s_gm[warp], s_pr[warp], s_coef[warp], wg, G);
                 } else {
                     ws = tiles1d_f32<SYS_EULER1D>(A, s_U[warp], s_gp[warp], s_gm[warp], s_pr[warp], s_cf, wg, G);
                 }
@@ -2563,14 +2627,18 @@ cudaError_t launch_batch1d_alpha(const Batch1D &p, double *alpha_out, cudaStream
 }
 
 template <typename T>
-int batch1d_groups(int group_warps) {
+int batch1d_per_sm() {
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch1d_kernel<T>, WPB * 32, 0) != cudaSuccess) {
         cudaGetLastError();
         per_sm = 1;
     }
-    if (per_sm < 1) per_sm = 1;
-    return num_sms() * per_sm * (WPB / (group_warps > 0 ? group_warps : WPB));
+    return per_sm < 1 ? 1 : per_sm;
+}
+
+template <typename T>
+int batch1d_groups(int group_warps) {
+    return num_sms() * batch1d_per_sm<T>() * (WPB / (group_warps > 0 ? group_warps : WPB));
 }
 
 template <typename T>
@@ -2578,11 +2646,7 @@ cudaError_t launch_batch1d(const Batch1D &p, cudaStream_t st) {
     if (p.group_warps != 1 && p.group_warps != 2 && p.group_warps != 4 && p.group_warps != 8)
         return cudaErrorInvalidValue;
     if (p.nbig < 0 || p.nbig > p.ntubes) return cudaErrorInvalidValue;
-    int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch1d_kernel<T>, WPB * 32, 0);
-    if (e != cudaSuccess) return e;
-    if (per_sm < 1) per_sm = 1;
-    batch1d_kernel<T><<<num_sms() * per_sm, WPB * 32, 0, st>>>(with_kt(p));
+    batch1d_kernel<T><<<num_sms() * batch1d_per_sm<T>(), WPB * 32, 0, st>>>(with_kt(p));
     return cudaGetLastError();
 }
 

@@ -38,12 +38,12 @@ __device__ __forceinline__ constexpr int rot(int c) {
 // FP64 face of one 2D sweep, with the exact powers of two of the 1D form
 // (roe_frame_f64): rows un -+ c of L doubled, 2 G+- staged, so the fields 0 and
 // 3 carry a factor 4, the entropy and shear fields 1 and 2 a factor 2, and the
-// face flux 4.  The products b1 v_t g_t and b1 g_E serve three fields each, and
-// the shear row (-v_t, 0, 1, 0) costs one product and one sum (adding 0 g could
-// only change the sign of a zero): 19 instead of 28 FP64 instructions per
-// projected cell and split.
+// face flux 4.  l[k] holds the factors of row k's density and normal-momentum
+// components, k = 0, 1, 3; its tangential one is -+ b1 v_t and its energy one
+// +- b1.  The shear row (-v_t, 0, 1, 0) costs one product and one sum (adding 0 g
+// could only change the sign of a zero).
 struct Roe2D64 {
-    double l0[2], l1[2], l3[2], b1, b1v, un, vt, cc, Ht, X;
+    double l[4][2], b1, b1v, un, vt, cc, Ht, X;
     int flag;
 };
 
@@ -64,82 +64,93 @@ __device__ __forceinline__ Roe2D64 roe_frame2d_f64(PR pr, double gm1) {
     const double uc = div64(R.un, R.cc), rc = div64(1.0, R.cc);
     const double b1u = R.b1 * R.un;
     R.b1v = R.b1 * R.vt;
-    R.l0[0] = __fma_rn(0.5, t, uc);
-    R.l0[1] = -(b1u + rc);
-    R.l1[0] = __fma_rn(-0.5, t, 1.0);
-    R.l1[1] = b1u;
-    R.l3[0] = __fma_rn(0.5, t, -uc);
-    R.l3[1] = -(b1u - rc);
+    R.l[0][0] = __fma_rn(0.5, t, uc);
+    R.l[0][1] = -(b1u + rc);
+    R.l[1][0] = __fma_rn(-0.5, t, 1.0);
+    R.l[1][1] = b1u;
+    R.l[3][0] = __fma_rn(0.5, t, -uc);
+    R.l[3][1] = -(b1u - rc);
     R.flag = f64_positive(c2) ? 0 : (f64_finite(c2) ? ERR_NONPHYSICAL : ERR_NONFINITE);
     return R;
 }
 
-// Characteristic values of one cell's split flux g (physical components; the
-// sums run in physical order, so along y the tangential term comes second).
-template <int DIR>
-__device__ __forceinline__ void project2d_f64(const Roe2D64 &R, const double g[4], double q[4]) {
-    const double gn = g[rot<DIR>(1)], gt = g[rot<DIR>(2)];
-    const double pt = R.b1v * gt, pe = R.b1 * g[3];
-    const double n0 = R.l0[1] * gn, n1 = R.l1[1] * gn, n3 = R.l3[1] * gn;
-    if constexpr (DIR == 0) {
-        q[0] = ((R.l0[0] * g[0] + n0) - pt) + pe;
-        q[1] = ((R.l1[0] * g[0] + n1) + pt) - pe;
-        q[3] = ((R.l3[0] * g[0] + n3) - pt) + pe;
-    } else {
-        q[0] = ((R.l0[0] * g[0] - pt) + n0) + pe;
-        q[1] = ((R.l1[0] * g[0] + pt) + n1) - pe;
-        q[3] = ((R.l3[0] * g[0] - pt) + n3) + pe;
-    }
-    q[2] = gt - R.vt * g[0];
-}
-
-// Flux of one face (scaled by 4) from the staged cells, split by split:
+// Flux of one face (scaled by 4) from the staged cells: split by split and field
+// by field (one field's seven taps live at a time, so that 16 warps fit an SM),
 // projection, cutoff bits, the neighbour faces' bits (adjacent lanes), selection
-// and polynomial, then the back-projection.  gp(c, t) / gm(c, t): component c of
-// 2 G+ / 2 G- of local cell t.  Returns the error flags; D[0..3] and D[4..7]
-// receive the Delta codes of the '+' and '-' splits.  Call with a whole warp.
-template <int DIR, typename PR, typename G>
-__device__ __forceinline__ int face2d_f64(PR pr, G g, double gm1, const Cut64 &cut2, const Cut64 &cut4,
-                                          const double *coef, double fh[4], int D[8]) {
+// and polynomial; then the back-projection.  g(s, c, t): component c of 2 G+ (s
+// = 0) or 2 G- of local cell t; the sums run in physical order, so along y the
+// tangential term comes second.  imul: every staged value is one mul64 takes;
+// the products then run on the integer pipe beside the FP64 sums.  Returns the
+// error flags; code(s, k, D) receives the Delta codes.  Call with a whole warp.
+template <int DIR, typename PR, typename G, typename CODE>
+__device__ __forceinline__ int face2d_f64(PR pr, G g, CODE code, double gm1, const Cut64 &cut2, const Cut64 &cut4,
+                                          bool imul, const double *coef, double fh[4]) {
     const Roe2D64 R = roe_frame2d_f64(pr, gm1);
     int flag = R.flag;
+    uint32_t unranged = mul_unranged(R.b1) | factor_unranged(R.b1v) | factor_unranged(R.vt);
+#pragma unroll
+    for (int k = 0; k < 4; k++)
+        if (k != 2) unranged |= factor_unranged(R.l[k][0]) | factor_unranged(R.l[k][1]);
+    imul = imul && !__any_sync(0xffffffffu, unranged != 0u);
+    constexpr int N = rot<DIR>(1), T = rot<DIR>(2);  // physical normal and tangential components
     double f[4];
-#pragma unroll
+#pragma unroll 1
     for (int s = 0; s < 2; s++) {
-        double P[4][7];
-        unsigned word = 0;
-#pragma unroll
-        for (int t = 0; t < 7; t++) {
-            // upwind order: '+' cells j-3+t, '-' cells j+4-t
-            const int c = s == 0 ? t : 7 - t;
-            const double gc[4] = {g(s, 0, c), g(s, 1, c), g(s, 2, c), g(s, 3, c)};
-            double q[4];
-            project2d_f64<DIR>(R, gc, q);
-#pragma unroll
-            for (int k = 0; k < 4; k++) P[k][t] = q[k];
-        }
-#pragma unroll
-        for (int k = 0; k < 4; k++)
-            word |= cutoff_bits(P[k][1], P[k][2], P[k][3], P[k][4], P[k][5], k == 0 || k == 3 ? cut4 : cut2)
-                    << (3 * k);
-        const unsigned wl = __shfl_up_sync(0xffffffffu, word, 1);
-        const unsigned wr = __shfl_down_sync(0xffffffffu, word, 1);
-        const unsigned wu = s == 0 ? wl : wr, wd = s == 0 ? wr : wl;  // upwind, downwind face
+        const int o = s == 0 ? 0 : 7, dir = s == 0 ? 1 : -1;  // upwind order: '+' cells j-3+t, '-' cells j+4-t
 #pragma unroll
         for (int k = 0; k < 4; k++) {
-            const int Dk = pack_delta(wu >> (3 * k), word >> (3 * k), wd >> (3 * k));
-            int m = lut_select(Dk);
-            if (m == 15) {
-                m = 11;
-                flag |= ERR_NOEXIST;
+            double P[7];
+            const double lt = k == 1 ? R.b1v : -R.b1v, le = k == 1 ? -R.b1 : R.b1;
+            if (imul) {
+                if (k == 2) {
+                    const MulOp m = mul_op(R.vt);
+#pragma unroll
+                    for (int t = 0; t < 7; t++) P[t] = g(s, T, o + dir * t) - mul64(m, g(s, 0, o + dir * t));
+                } else {
+                    const MulOp m0 = mul_op(R.l[k][0]), mn = mul_op(R.l[k][1]), mt = mul_op(lt), me = mul_op(le);
+#pragma unroll
+                    for (int t = 0; t < 7; t++) {
+                        const int c = o + dir * t;
+                        const double p0 = mul64(m0, g(s, 0, c)), pn = mul64(mn, g(s, N, c));
+                        const double pt = mul64(mt, g(s, T, c)), pe = mul64(me, g(s, 3, c));
+                        P[t] = DIR == 0 ? ((p0 + pn) + pt) + pe : ((p0 + pt) + pn) + pe;
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int t = 0; t < 7; t++) {
+                    const int c = o + dir * t;
+                    if (k == 2) {
+                        P[t] = g(s, T, c) - R.vt * g(s, 0, c);
+                    } else {
+                        const double p0 = R.l[k][0] * g(s, 0, c), pn = R.l[k][1] * g(s, N, c);
+                        const double pt = lt * g(s, T, c), pe = le * g(s, 3, c);
+                        P[t] = DIR == 0 ? ((p0 + pn) + pt) + pe : ((p0 + pt) + pn) + pe;
+                    }
+                }
             }
+            const unsigned w = cutoff_bits(P[1], P[2], P[3], P[4], P[5], k == 0 || k == 3 ? cut4 : cut2);
+            int D = 31, m = 0;
+            if (!__all_sync(0xffffffffu, w == 7u)) {
+                const unsigned wl = __shfl_up_sync(0xffffffffu, w, 1);
+                const unsigned wr = __shfl_down_sync(0xffffffffu, w, 1);
+                D = s == 0 ? pack_delta(wl, w, wr) : pack_delta(wr, w, wl);
+                m = lut_select(D);
+                if (m == 15) {
+                    m = 11;
+                    flag |= ERR_NOEXIST;
+                }
+            }
+            uint32_t bad = (uint32_t)m;
+#pragma unroll
+            for (int t = 0; t < 7; t++) bad |= mul_unranged(P[t]);
             double v;
-            if (m == 0)
-                v = poly_f0(P[k][0], P[k][1], P[k][2], P[k][3], P[k][4], P[k][5], P[k][6]);
+            if (!__any_sync(0xffffffffu, bad != 0u))
+                v = poly_f0_imul(P);
             else
-                v = poly7(coef + 7 * m, P[k][0], P[k][1], P[k][2], P[k][3], P[k][4], P[k][5], P[k][6]);
+                v = poly7(coef + 7 * m, P[0], P[1], P[2], P[3], P[4], P[5], P[6]);
             f[k] = s == 0 ? v : f[k] + v;
-            D[4 * s + k] = Dk;
+            code(s, k, D);
         }
     }
     // right eigenvectors (columns un-c, un, shear, un+c) in rotated rows; f[1]
@@ -284,7 +295,7 @@ __device__ __forceinline__ T alpha2d_in(const Stage2D &p, const DevCtl *ctl, int
 // x sweep: R = Lx(U), warp tiles of 29 cells along rows.
 // --------------------------------------------------------------------------
 template <typename T, bool HALO>
-__global__ void __launch_bounds__(WPB * 32, 1) xsweep2d_kernel(const Stage2D p) {
+__global__ void __launch_bounds__(WPB * 32, 2) xsweep2d_kernel(const Stage2D p) {
     __shared__ T s_gp[WPB][4][WC];
     __shared__ T s_gm[WPB][4][WC];
     __shared__ T s_pr[WPB][4][WC];
@@ -313,6 +324,7 @@ __global__ void __launch_bounds__(WPB * 32, 1) xsweep2d_kernel(const Stage2D p) 
         const int y = (int)(tile / ntx);
         const int c0 = (int)(tile % ntx) * WT;
         const T *row = Us + (size_t)y * nx;
+        uint32_t unranged = 0u;  // a value mul64 does not take
         for (int c = lane; c < WS; c += 32) {
             int gi = c0 - 5 + c;
             if (gi < 0 || gi >= nx) gi = ghost_map(gi, nx, p.bc[0], p.bc[1]);
@@ -326,21 +338,21 @@ __global__ void __launch_bounds__(WPB * 32, 1) xsweep2d_kernel(const Stage2D p) 
                 spr[k][c] = pr[k];
                 sgp[k][c] = gp[k];
                 sgm[k][c] = gm[k];
+                unranged |= mul_unranged(gp[k]) | mul_unranged(gm[k]);
             }
         }
         __syncwarp();
         const int j = c0 - 2 + lane;
-        T fh[4];
-        int D[8];
-        const int flag = face2d_f64<0>([&](int q, int t) { return spr[q][lane + t]; },
-                                       [&](int s, int c, int t) { return (s == 0 ? sgp : sgm)[c][lane + t]; }, gm1,
-                                       cut2, cut4, s_coef[warp], fh, D);
         const bool face_out = lane >= 1 && lane <= 30;
-        if (p.rhs_mode && p.masks && face_out && j >= -1 && j <= nx - 1) {
-#pragma unroll
-            for (int sk = 0; sk < 8; sk++)
-                p.masks[((size_t)sk * ny + y) * (nx + 1) + (j + 1)] = (uint8_t)D[sk];
-        }
+        const bool masks = p.rhs_mode && p.masks && face_out && j >= -1 && j <= nx - 1;
+        T fh[4];
+        const int flag = face2d_f64<0>(
+            [&](int q, int t) { return spr[q][lane + t]; },
+            [&](int s, int c, int t) { return (s == 0 ? sgp : sgm)[c][lane + t]; },
+            [&](int s, int k, int D) {
+                if (masks) p.masks[((size_t)(4 * s + k) * ny + y) * (nx + 1) + (j + 1)] = (uint8_t)D;
+            },
+            gm1, cut2, cut4, !__any_sync(0xffffffffu, unranged != 0u), s_coef[warp], fh);
         if (flag && face_out && j >= -2 && j <= nx)
             latch_error(ctl, (flag & (ERR_NONPHYSICAL | ERR_NONFINITE)) | ((flag & ERR_NOEXIST) ? ERR_NONFINITE : 0),
                         flat_cell(y, j, nx));
@@ -364,14 +376,15 @@ __global__ void __launch_bounds__(WPB * 32, 1) xsweep2d_kernel(const Stage2D p) 
 //   gp, gm, pr  [4][39][33] each; ry [4][29][33]; coef [92]; reductions.
 // --------------------------------------------------------------------------
 constexpr int YB_COLS = 32, YB_ROWS = WT, YB_STAGE = WS, YB_LD = 33;
+constexpr int YW64 = 16;  // warps of an FP64 y-sweep CTA (its shared memory allows one CTA per SM)
 
 template <typename T>
 constexpr size_t ysweep_smem_bytes() {
-    return sizeof(T) * (3 * 4 * YB_STAGE * YB_LD + 4 * YB_ROWS * YB_LD + 92) + 2 * WPB * sizeof(T);
+    return sizeof(T) * (3 * 4 * YB_STAGE * YB_LD + 4 * YB_ROWS * YB_LD + 92) + 2 * YW64 * sizeof(T);
 }
 
 template <typename T, bool HALO>
-__global__ void __launch_bounds__(WPB * 32, 1) ysweep2d_kernel(const Stage2D p) {
+__global__ void __launch_bounds__(YW64 * 32, 1) ysweep2d_kernel(const Stage2D p) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *sm = reinterpret_cast<T *>(smem_raw);
     T *s_gp = sm;                                 // [4][39][33]
@@ -379,7 +392,7 @@ __global__ void __launch_bounds__(WPB * 32, 1) ysweep2d_kernel(const Stage2D p) 
     T *s_pr = s_gm + 4 * YB_STAGE * YB_LD;        // [4][39][33]
     T *s_ry = s_pr + 4 * YB_STAGE * YB_LD;        // [4][29][33]
     T *s_coef = s_ry + 4 * YB_ROWS * YB_LD;       // [92]
-    T *s_red = s_coef + 92;                       // [2][WPB]
+    T *s_red = s_coef + 92;                       // [2][YW64]
     auto at = [](T *base, int c, int r, int col) -> T & { return base[(c * YB_STAGE + r) * YB_LD + col]; };
 
     DevCtl *ctl = p.ctl;
@@ -398,6 +411,7 @@ __global__ void __launch_bounds__(WPB * 32, 1) ysweep2d_kernel(const Stage2D p) 
     for (int q = tid; q < 91; q += blockDim.x) s_coef[q] = coef<T>(q);
 
     // ---- stage rows r0-5 .. r0+33 of columns x0 .. x0+31 (coalesced along x)
+    uint32_t any_unranged = 0u;
     for (int idx = tid; idx < YB_STAGE * YB_COLS; idx += blockDim.x) {
         const int r = idx / YB_COLS, col = idx % YB_COLS, x = x0 + col;
         if (x >= nx) continue;
@@ -407,31 +421,35 @@ __global__ void __launch_bounds__(WPB * 32, 1) ysweep2d_kernel(const Stage2D p) 
 #pragma unroll
         for (int k = 0; k < 4; k++) U[k] = Us[st_at<HALO>(k, sv, y, nx, chk(p.ctl, x, 0, p.nx))];
         cell2d_f64<1>(U, gm1, alpha, pr, gp, gm);
+        uint32_t unranged = 0u;  // a value mul64 does not take
 #pragma unroll
         for (int k = 0; k < 4; k++) {
             at(s_pr, k, r, col) = pr[k];
             at(s_gp, k, r, col) = gp[k];
             at(s_gm, k, r, col) = gm[k];
+            unranged |= mul_unranged(gp[k]) | mul_unranged(gm[k]);
         }
+        any_unranged |= unranged;
     }
-    __syncthreads();
+    const bool imul = !__syncthreads_or(any_unranged != 0u);
 
-    // ---- faces down the columns: warp w takes columns w, w+8, w+16, w+24
-    for (int col = warp; col < YB_COLS; col += WPB) {
+    // ---- faces down the columns: warp w takes columns w and w+16
+    for (int col = warp; col < YB_COLS; col += YW64) {
         const int x = x0 + col;
         if (x >= nx) break;
         const int j = r0 - 2 + lane;  // face j+1/2 along y
-        T fh[4];
-        int D[8];
-        const int flag = face2d_f64<1>([&](int q, int t) { return at(s_pr, q, lane + t, col); },
-                                       [&](int s, int c, int t) { return at(s == 0 ? s_gp : s_gm, c, lane + t, col); },
-                                       gm1, cut2, cut4, s_coef, fh, D);
         const bool face_out = lane >= 1 && lane <= 30;
-        if (p.rhs_mode && p.masks && face_out && j >= -1 && j <= ny - 1) {
-            uint8_t *ym = p.masks + (size_t)8 * ny * (nx + 1);
-#pragma unroll
-            for (int sk = 0; sk < 8; sk++) ym[((size_t)sk * nx + x) * (ny + 1) + (j + 1)] = (uint8_t)D[sk];
-        }
+        uint8_t *ym = p.rhs_mode && p.masks && face_out && j >= -1 && j <= ny - 1
+                          ? p.masks + (size_t)8 * ny * (nx + 1) + (size_t)x * (ny + 1) + (j + 1)
+                          : nullptr;
+        T fh[4];
+        const int flag = face2d_f64<1>(
+            [&](int q, int t) { return at(s_pr, q, lane + t, col); },
+            [&](int s, int c, int t) { return at(s == 0 ? s_gp : s_gm, c, lane + t, col); },
+            [&](int s, int k, int D) {
+                if (ym) ym[(size_t)(4 * s + k) * nx * (ny + 1)] = (uint8_t)D;
+            },
+            gm1, cut2, cut4, imul, s_coef, fh);
         if (flag && face_out && j >= -2 && j <= ny)
             latch_error(ctl, (flag & (ERR_NONPHYSICAL | ERR_NONFINITE)) | ((flag & ERR_NOEXIST) ? ERR_NONFINITE : 0),
                         flat_cell(j, x, nx, ny));
@@ -491,14 +509,14 @@ __global__ void __launch_bounds__(WPB * 32, 1) ysweep2d_kernel(const Stage2D p) 
         my = warp_max(my);
         if (lane == 0) {
             s_red[warp] = mx;
-            s_red[WPB + warp] = my;
+            s_red[YW64 + warp] = my;
         }
         __syncthreads();
         if (tid == 0) {
-            T vx = s_red[0], vy = s_red[WPB];
-            for (int w = 1; w < WPB; w++) {
+            T vx = s_red[0], vy = s_red[YW64];
+            for (int w = 1; w < YW64; w++) {
                 vx = fmax(vx, s_red[w]);
-                vy = fmax(vy, s_red[WPB + w]);
+                vy = fmax(vy, s_red[YW64 + w]);
             }
             const int so = (p.stage + 1) % 3;
             atomicMax(&ctl->amax[so][0], (unsigned long long)__double_as_longlong((double)vx));
@@ -1594,7 +1612,7 @@ cudaError_t launch_stage2d(const Stage2D &p_, cudaStream_t st) {
     e = cudaFuncSetAttribute(ysweep2d_kernel<T, HALO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((p.nx + YB_COLS - 1) / YB_COLS, (p.ny + YB_ROWS - 1) / YB_ROWS);
-    ysweep2d_kernel<T, HALO><<<grid, WPB * 32, smem, st>>>(p);
+    ysweep2d_kernel<T, HALO><<<grid, YW64 * 32, smem, st>>>(p);
     return cudaGetLastError();
     }
 }

@@ -104,8 +104,32 @@ static void check_div_sqrt() {
     printf("div %ld %ld\nsqrt %ld %ld\n", nd, bd, ns, bs);
 }
 
+// products, over the range mul64 takes: random, short mantissas (exact products
+// and ties), and mantissas of ones
+static void check_mul() {
+    std::mt19937_64 r(5);
+    long n = 0, bad = 0;
+    for (int i = 0; i < 4000000; i++) {
+        auto draw = [&](int kind) {
+            uint64_t m = r() & 0xfffffffffffffull;
+            if (kind == 1) m &= ~0ull << (20 + r() % 32);
+            if (kind == 2) m = 0xfffffffffffffull - (m >> (20 + r() % 32));
+            if (kind == 3) m &= ~0ull << (24 + r() % 4);
+            return f64_of(((r() & 1) << 63) | ((623 + r() % 800) << 52) | m);
+        };
+        const double x = i % 1000 == 0 ? 0.0 : draw(i % 4), g = draw((i / 4) % 4);
+        if (mul_unranged(g) || (x != 0.0 && mul_unranged(x))) bad++;
+        n++;
+        const double p = mul64(mul_op(x), g);
+        bad += p != x * g;
+    }
+    for (double v : {0.0, 1e-130, 1e130, (double)INFINITY, (double)NAN, 5e-324}) bad += mul_unranged(v) != 1;
+    printf("mul %ld %ld\n", n, bad);
+}
+
 int main() {
     check_cutoff();
+    check_mul();
     check_div_sqrt();
     return 0;
 }

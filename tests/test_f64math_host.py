@@ -22,7 +22,7 @@ def results(tmp_path_factory):
     return {k: (int(n), int(bad)) for k, n, bad in (line.split() for line in out.splitlines())}
 
 
-@pytest.mark.parametrize("what", ["cutoff", "cutoff_special", "div", "sqrt"])
+@pytest.mark.parametrize("what", ["cutoff", "cutoff_special", "div", "sqrt", "mul"])
 def test_same_as_fp64(results, what):
     n, bad = results[what]
     assert n > 10000 and bad == 0
