@@ -48,6 +48,7 @@ struct t7_ctx {
     cudaEvent_t g_in, g_out;
     cudaGraphExec_t gexec;
     void *g_U;
+    unsigned run_tag;      // next stage tag of the cooperative run kernels
     // t7_run_host with a known step count: the last stage is launched in parts
     // and each finished part is copied to the host array on cstream
     cudaStream_t cstream;
@@ -82,6 +83,10 @@ t7_status cuda_fail(t7_ctx *c, cudaError_t e, const char *what) {
 }
 
 int nvars(int sys) { return sys == T7_EULER1D ? 3 : (sys == T7_EULER2D ? 4 : 1); }
+
+// The control block, and after it the slots of the cooperative run kernels.
+constexpr size_t CTL_SLOTS = (sizeof(t7::DevCtl) + 255) / 256 * 256;
+constexpr size_t CTL_BYTES = CTL_SLOTS + 2 * t7::RUN_MAX_CTAS * sizeof(t7::RunSlot);
 
 bool is_1d(int sys) { return sys == T7_SCALAR_ADVECTION || sys == T7_EULER1D || sys == T7_BURGERS; }
 
@@ -292,6 +297,8 @@ t7_status collect(t7_ctx *c) {
         cudaMemcpy(&c->ctl->err_index, &big, sizeof(int), cudaMemcpyHostToDevice);
         if (err & t7::ERR_INDEX)
             return fail(c, T7_EINDEX, "index check failed (checked build): index %d", idx);
+        if (err & t7::ERR_TIMEOUT)
+            return fail(c, T7_ETIMEOUT, "a wait between the blocks of a run launch gave up");
         if (err & t7::ERR_NONPHYSICAL)
             return fail(c, T7_ENONPHYSICAL, "non-physical state (rho <= 0, p <= 0 or c^2 <= 0) near index %d", idx);
         return fail(c, T7_ENONFINITE, "non-finite state or unreachable stencil pattern near index %d", idx);
@@ -342,12 +349,13 @@ t7_status t7_create(const t7_grid *g, void *stream, t7_ctx **out) {
     c->esize = g->prec == T7_F32 ? 4 : 8;
     c->ncell = (size_t)g->nx * g->ny;
     c->stream = (cudaStream_t)stream;
+    c->run_tag = 1;  // the slots start at zero
     cudaGetDevice(&c->device);
     size_t bytes = c->ncell * c->m * c->esize;
     if (cudaMalloc(&c->U1, bytes) != cudaSuccess || cudaMalloc(&c->U2, bytes) != cudaSuccess ||
         cudaMalloc(&c->Uhost, bytes) != cudaSuccess ||
         (g->sys == T7_EULER2D && cudaMalloc(&c->R, bytes) != cudaSuccess) ||
-        cudaMalloc((void **)&c->ctl, sizeof(t7::DevCtl)) != cudaSuccess ||
+        cudaMalloc((void **)&c->ctl, CTL_BYTES) != cudaSuccess ||
         cudaMallocHost((void **)&c->ctl_host, sizeof(t7::DevCtl)) != cudaSuccess) {
         t7_destroy(c);
         cudaGetLastError();
@@ -357,7 +365,8 @@ t7_status t7_create(const t7_grid *g, void *stream, t7_ctx **out) {
     memset(&init, 0, sizeof(init));
     init.err_index = 0x7fffffff;
     init.max_steps = 0;
-    if (cudaMemcpy(c->ctl, &init, sizeof(init), cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (cudaMemset(c->ctl, 0, CTL_BYTES) != cudaSuccess ||
+        cudaMemcpy(c->ctl, &init, sizeof(init), cudaMemcpyHostToDevice) != cudaSuccess) {
         t7_destroy(c);
         cudaGetLastError();
         return T7_ECUDA;
@@ -659,7 +668,6 @@ extern "C" t7_status t7_slab_stage(t7_ctx *c, int k, const void *Us, const void 
 // dominates; above it the 3 launches per step cost nothing measurable).
 constexpr int RUN_CHUNK = 64;
 constexpr size_t GRAPH_MAX_VALUES = size_t(1) << 21;
-
 // One chunk of RUN_CHUNK steps of U as a replayed graph (captured on first use
 // for this U).  Returns 1 when the chunk was enqueued; 0, with no work
 // enqueued, if the graph cannot be made or launched (the caller then launches
@@ -706,6 +714,38 @@ static int run_chunk_graph(t7_ctx *c, void *U) {
     return 1;
 }
 
+// Whether a run towards a finite t_end goes on (waits for the work queued so
+// far); false with *e set if that failed.
+static bool run_poll(t7_ctx *c, double t_end, cudaError_t *e) {
+    *e = cudaMemcpyAsync(c->ctl_host, c->ctl, sizeof(t7::DevCtl), cudaMemcpyDeviceToHost, c->stream);
+    if (*e == cudaSuccess) *e = cudaStreamSynchronize(c->stream);
+    if (*e != cudaSuccess) return false;
+    return c->ctl_host->active && !c->ctl_host->err && c->ctl_host->t < t_end;
+}
+
+// k steps of U in one cooperative launch.  Returns false, with nothing enqueued,
+// when the problem is not one for it or the launch is refused.
+static bool run_steps_coop(t7_ctx *c, void *U, int k) {
+    t7::Run1D q;
+    memset(&q, 0, sizeof(q));
+    q.p = stage_params(c, nullptr, nullptr, nullptr);
+    q.U = U;
+    q.U1 = c->U1;
+    q.U2 = c->U2;
+    q.nsteps = k;
+    q.slots = reinterpret_cast<t7::RunSlot *>(reinterpret_cast<char *>(c->ctl) + CTL_SLOTS);
+    q.tag = c->run_tag;
+    cudaError_t e = c->g.prec == T7_MIXED ? t7::launch_run1d_mixed(q, c->stream)
+                    : c->g.prec == T7_F64 ? t7::launch_run1d_f64(q, c->stream)
+                                          : t7::launch_run1d_f32(q, c->stream);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    c->run_tag += 3u * (unsigned)k;
+    return true;
+}
+
 // t7_run's loop; host_out (nullable, 1D, only with t_end = inf) receives a
 // copy of the result of the last step, made while its last stage computes.
 static t7_status run_core(t7_ctx *c, void *U, double cfl, double t_end, int max_steps, int *steps_out, double *t_out,
@@ -717,11 +757,20 @@ static t7_status run_core(t7_ctx *c, void *U, double cfl, double t_end, int max_
     if (e != cudaSuccess) return cuda_fail(c, e, "alpha");
     // Steps are launched in chunks; between chunks the host polls whether the
     // device-side clock has reached t_end (a step past it is a no-op anyway).
+    const bool coop = is_1d(c->g.sys);
     const bool graphs = is_1d(c->g.sys) && c->ncell * c->m <= GRAPH_MAX_VALUES;
     int launched = 0;
     while (launched < max_steps) {
         int k = max_steps - launched < RUN_CHUNK ? max_steps - launched : RUN_CHUNK;
         const bool last_chunk = host_out && launched + k == max_steps;
+        if (coop && !last_chunk && run_steps_coop(c, U, k)) {
+            launched += k;
+            if (isfinite(t_end) && !run_poll(c, t_end, &e)) {
+                if (e != cudaSuccess) return cuda_fail(c, e, "poll");
+                break;
+            }
+            continue;
+        }
         const int g = (graphs && k == RUN_CHUNK && !last_chunk) ? run_chunk_graph(c, U) : 0;
         if (g < 0) return cuda_fail(c, cudaGetLastError(), "ordering a graph chunk");
         if (g == 0) {
@@ -731,12 +780,9 @@ static t7_status run_core(t7_ctx *c, void *U, double cfl, double t_end, int max_
             }
         }
         launched += k;
-        if (isfinite(t_end)) {
-            if ((e = cudaMemcpyAsync(c->ctl_host, c->ctl, sizeof(t7::DevCtl), cudaMemcpyDeviceToHost, c->stream)) !=
-                cudaSuccess)
-                return cuda_fail(c, e, "poll");
-            if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return cuda_fail(c, e, "sync");
-            if (!c->ctl_host->active || c->ctl_host->err || !(c->ctl_host->t < t_end)) break;
+        if (isfinite(t_end) && !run_poll(c, t_end, &e)) {
+            if (e != cudaSuccess) return cuda_fail(c, e, "poll");
+            break;
         }
     }
     if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return cuda_fail(c, e, "sync");

@@ -8,7 +8,7 @@ namespace t7 {
 
 enum { SYS_ADV = 0, SYS_EULER1D = 1, SYS_EULER2D = 2, SYS_BURGERS = 3 };
 enum { BC_PERIODIC = 0, BC_ZG = 1 };
-enum { ERR_NONPHYSICAL = 1, ERR_NONFINITE = 2, ERR_NOEXIST = 4, ERR_INDEX = 8 };
+enum { ERR_NONPHYSICAL = 1, ERR_NONFINITE = 2, ERR_NOEXIST = 4, ERR_INDEX = 8, ERR_TIMEOUT = 16 };
 
 // Device-resident control block of a context.  amax[slot][dir] holds the bit
 // pattern of a non-negative double (max characteristic speed) so that it can
@@ -62,6 +62,22 @@ struct Stage1D {
     int alpha_mode;          // t7_alpha_mode: 1 = one alpha per characteristic field (1D Euler)
     double kt;               // keep_all_factor(CT), set by the launchers (here and below)
     float f_kt;
+};
+
+// Several RK3 steps of a 1D problem in one cooperative launch (small problems).
+// Each CTA publishes its maximum of every stage's output in its own slot, tagged
+// with the stage's number, and waits for the others' (see grid_max).
+constexpr int RUN_MAX_CTAS = 512;
+struct RunSlot {
+    unsigned long long w[2];  // tag << 32 | high, low half of the maximum's bits
+};
+struct Run1D {
+    Stage1D p;       // grid and parameters (Us, U0, out, stage, slot_in unused)
+    void *U, *U1, *U2;
+    int nsteps;
+    RunSlot *slots;  // [2][RUN_MAX_CTAS]
+    unsigned tag;    // tag of the launch's first stage; 3 nsteps tags are used
+    int cluster;     // the grid is one thread-block cluster (set by the launcher)
 };
 
 // Ghost cells per side of a slab (the stencil reach of the scheme, Eq. app:
@@ -198,6 +214,10 @@ struct Recon {
 cudaError_t launch_stage1d_f64(const Stage1D &p, cudaStream_t s);
 cudaError_t launch_stage1d_f32(const Stage1D &p, cudaStream_t s);
 cudaError_t launch_stage1d_mixed(const Stage1D &p, cudaStream_t s);  // FP64 state, FP32 reconstruction
+// cooperative launches; cudaErrorNotSupported: not for this problem
+cudaError_t launch_run1d_f64(const Run1D &p, cudaStream_t s);
+cudaError_t launch_run1d_f32(const Run1D &p, cudaStream_t s);
+cudaError_t launch_run1d_mixed(const Run1D &p, cudaStream_t s);
 cudaError_t launch_alpha1d_f64(const Alpha1D &p, cudaStream_t s);
 cudaError_t launch_alpha1d_f32(const Alpha1D &p, cudaStream_t s);
 cudaError_t launch_recon_f64(const Recon &p, cudaStream_t s);

@@ -786,29 +786,220 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
     return wsmax;
 }
 
+// --------------------------------------------------------------------------
+// FP64 1D Euler with one tile per CTA of eight warps, for problems of a few tiles
+// per SM.  A lone warp issues an FP64 instruction every 64 cycles where four or
+// more share an SM's pipe at 19, so a tile's ~330 instructions, 21,000 cycles as
+// one warp's chain, are spread over the warps: staging by component (warp pairs),
+// the Roe averages, the roots and quotients of the frame, the six (field, split)
+// reconstructions -- one warp each, products by mul64 beside the FP64 sums -- and
+// the three components' update.  The same operations in the same order as
+// tiles1d.  Every thread of the CTA calls it; the returned maximum is warp 0's.
+// --------------------------------------------------------------------------
+struct SplitSmem {
+    double U[3][WC], gp[3][WC], gm[3][WC], pr[3][WC];
+    double ut[32], Ht[32], X[32], cc[32], uc[32], rc[32], b1[32], t[32], b1u[32];
+    double f[2][3][32], o[3][32], coef[92];
+};
+
+template <int SCH>
+__device__ __forceinline__ double tiles1d_split(const TileArgs<double> &A, SplitSmem &s, int tile0, int tstride) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int n = A.n, ntiles = (n + WT - 1) / WT;
+    const size_t cs = A.cs;
+    DevCtl *ctl = A.ctl;
+    const double gm1 = A.gm1, dx4 = FLUX_SCALE_EULER * A.dx;
+    double wsmax = 0.0;
+    for (int tile = tile0; tile < ntiles; tile += tstride) {
+        const int c0 = tile * WT, j = c0 - 2 + lane;
+        const bool face_out = lane >= 1 && lane <= 30, cell_out = lane >= 2 && lane <= 30 && j < n;
+        // ---- staging: warps 2 r' + h take cells lane + 32 h, in four roles ----
+        const int c = lane + 32 * (warp & 1), role = warp >> 1;
+        double u0 = 0.0;  // U^n of the update (warps 0 .. 2)
+        if (!A.rhs_mode && A.stage > 0 && warp < 3 && cell_out) u0 = A.U0[(size_t)warp * cs + chk(ctl, j, 0, n)];
+        if (c < WS) {
+            int gi = c0 - 5 + c;
+            if (gi < 0 || gi >= n) gi = ghost_or_halo(gi, n, A.bc_lo, A.bc_hi, A.halo);
+            gi = chk(ctl, gi, A.halo ? -HALO_CELLS : 0, n + (A.halo ? HALO_CELLS : 0));
+            const double U0 = A.Us[gi], U1 = A.Us[cs + gi], U2 = A.Us[2 * cs + gi];
+            if (role == 3) {
+                s.pr[2][c] = sqrt64(U0);
+                s.U[0][c] = U0;
+                s.U[1][c] = U1;
+                s.U[2][c] = U2;
+            } else {
+                const double u = div64(U1, U0), m = U1 * u;
+                const double p = gm1 * __fma_rn(-0.5, m, U2);
+                if (role == 0) {
+                    const double a0 = A.alpha * U0, a1 = A.alpha * U1, F1 = m + p;
+                    s.gp[0][c] = U1 + a0;
+                    s.gm[0][c] = U1 - a0;
+                    s.gp[1][c] = F1 + a1;
+                    s.gm[1][c] = F1 - a1;
+                } else {
+                    const double e = U2 + p;
+                    if (role == 1) {
+                        const double a2 = A.alpha * U2, F2 = u * e;
+                        s.gp[2][c] = F2 + a2;
+                        s.gm[2][c] = F2 - a2;
+                    } else {
+                        s.pr[0][c] = u;
+                        s.pr[1][c] = div64(e, U0);
+                    }
+                }
+            }
+        }
+        __syncthreads();
+        // ---- Roe averages (warps 0, 1) ----------------------------------------
+        if (warp < 2) {
+            const double sl = s.pr[2][lane + 3], sr = s.pr[2][lane + 4];
+            (warp == 0 ? s.ut : s.Ht)[lane] = div64(sl * s.pr[warp][lane + 3] + sr * s.pr[warp][lane + 4], sl + sr);
+        }
+        __syncthreads();
+        // ---- c, u/c, 1/c (warp 0); b1, 2 b2, b1 u (warp 1) ---------------------
+        if (warp < 2) {
+            const double ut = s.ut[lane], X = ut * ut;
+            const double c2 = gm1 * __fma_rn(-0.5, X, s.Ht[lane]);
+            if (warp == 0) {
+                const double cc = sqrt64(c2);
+                s.X[lane] = X;
+                s.cc[lane] = cc;
+                s.uc[lane] = div64(ut, cc);
+                s.rc[lane] = div64(1.0, cc);
+                if (!f64_positive(c2) && face_out && j >= -2 && j <= n)
+                    latch_error(ctl, f64_finite(c2) ? ERR_NONPHYSICAL : ERR_NONFINITE, A.ebase + j);
+            } else {
+                const double b1 = div64(gm1, c2);
+                s.b1[lane] = b1;
+                s.t[lane] = X * b1;
+                s.b1u[lane] = b1 * ut;
+            }
+        }
+        __syncthreads();
+        // ---- reconstruction: warp 3 sp + k, split sp of field k ------------------
+        if (warp < 6) {
+            const int k = warp % 3, sp = warp / 3;
+            const double t = s.t[lane], b1 = k == 1 ? -s.b1[lane] : s.b1[lane];
+            double l0, l1;
+            if (k == 1) {
+                l0 = __fma_rn(-0.5, t, 1.0);
+                l1 = s.b1u[lane];
+            } else {
+                l0 = __fma_rn(0.5, t, k == 0 ? s.uc[lane] : -s.uc[lane]);
+                l1 = -(s.b1u[lane] + (k == 0 ? s.rc[lane] : -s.rc[lane]));
+            }
+            const double (*sg)[WC] = sp == 0 ? s.gp : s.gm;
+            const int o = sp == 0 ? lane : lane + 7, dir = sp == 0 ? 1 : -1;
+            uint32_t unranged = mul_unranged(b1) | factor_unranged(l0) | factor_unranged(l1);
+            double g[3][7], P[7];
+#pragma unroll
+            for (int q = 0; q < 7; q++)
+#pragma unroll
+                for (int m = 0; m < 3; m++) {
+                    g[m][q] = sg[m][o + dir * q];
+                    unranged |= mul_unranged(g[m][q]);
+                }
+            if (!__any_sync(0xffffffffu, unranged != 0u)) {
+                const MulOp m0 = mul_op(l0), m1 = mul_op(l1), m2 = mul_op(b1);
+#pragma unroll
+                for (int q = 0; q < 7; q++) P[q] = (mul64(m0, g[0][q]) + mul64(m1, g[1][q])) + mul64(m2, g[2][q]);
+            } else {
+#pragma unroll
+                for (int q = 0; q < 7; q++) P[q] = (l0 * g[0][q] + l1 * g[1][q]) + b1 * g[2][q];
+            }
+            const double e = k == 1 ? 4.0 : 16.0;
+            const unsigned w = cutoff_bits(P[1], P[2], P[3], P[4], P[5], cut64(e * A.eps, A.CT, A.kt));
+            unsigned D;
+            int m;
+            double v;
+            if constexpr (SCH == SCH_TENO5) {
+                D = w;
+                m = sel5(w);
+                if (m == 7) m = 15;
+            } else {
+                const unsigned wl = __shfl_up_sync(0xffffffffu, w, 1), wr = __shfl_down_sync(0xffffffffu, w, 1);
+                D = (unsigned)(sp == 0 ? pack_delta(wl, w, wr) : pack_delta(wr, w, wl));
+                m = lut_select((int)D);
+            }
+            if (m == 15) {
+                m = SCH == SCH_TENO5 ? 0 : 11;
+                if (face_out && j >= -2 && j <= n) latch_error(ctl, ERR_NONFINITE, A.ebase + j);
+            }
+            if constexpr (SCH == SCH_TENO5) {
+                v = poly5(s.coef + 5 * m, P[1], P[2], P[3], P[4], P[5]);
+            } else {
+                uint32_t bad = (uint32_t)m;
+#pragma unroll
+                for (int q = 0; q < 7; q++) bad |= mul_unranged(P[q]);
+                if (!__any_sync(0xffffffffu, bad != 0u))
+                    v = poly_f0_imul(P);
+                else
+                    v = poly7(s.coef + 7 * m, P[0], P[1], P[2], P[3], P[4], P[5], P[6]);
+            }
+            s.f[sp][k][lane] = v;
+            if (A.masks && face_out && j >= -1 && j <= n - 1)
+                A.masks[(size_t)(sp * 3 + k) * (n + 1) + (j + 1)] = (uint8_t)D;
+        }
+        __syncthreads();
+        // ---- back-projection, difference and RK stage: warp c, component c -------
+        if (warp < 3) {
+            const double f0 = s.f[0][0][lane] + s.f[1][0][lane], f1 = s.f[0][1][lane] + s.f[1][1][lane];
+            const double f2 = s.f[0][2][lane] + s.f[1][2][lane];
+            const double ut = s.ut[lane], cc = s.cc[lane];
+            double fh;
+            if (warp == 0) {
+                fh = __fma_rn(2.0, f1, f0) + f2;
+            } else if (warp == 1) {
+                fh = __fma_rn(2.0, ut * f1, (ut - cc) * f0) + (ut + cc) * f2;
+            } else {
+                const double w = ut * cc, Ht = s.Ht[lane];
+                fh = ((Ht - w) * f0 + s.X[lane] * f1) + (Ht + w) * f2;
+            }
+            const double fprev = __shfl_up_sync(0xffffffffu, fh, 1);
+            if (cell_out) {
+                const int ii = chk(ctl, j, 0, n);
+                double r = div64(fprev - fh, dx4);
+                if (!A.rhs_mode) {
+                    r = rk_combine_f64(A.stage, s.U[warp][lane + 3], A.dtT, r, u0);
+                    s.o[warp][lane] = r;
+                }
+                A.out[(size_t)warp * A.cso + ii] = r;
+            }
+        }
+        if (!A.rhs_mode) {
+            __syncthreads();
+            if (warp == 0 && cell_out) {
+                const double ov[3] = {s.o[0][lane], s.o[1][lane], s.o[2][lane]};
+                int wflag = 0;
+                wsmax = f64_max_pos(wsmax, wavespeed1d<double, SYS_EULER1D>(ov, gm1, A.gamma, A.a, &wflag));
+                if (wflag) latch_error(ctl, wflag, A.ebase + j);
+            }
+        }
+        if (tile + tstride < ntiles) __syncthreads();  // the next tile overwrites the staging rows
+    }
+    return wsmax;
+}
+
+// The scheme's FP64 coefficient table, by the whole CTA.
+template <int SCH>
+__device__ __forceinline__ void fill_coef64(double *s_coef) {
+    for (int q = threadIdx.x; q < (SCH == SCH_TENO5 ? 35 : 91); q += blockDim.x)
+        s_coef[q] = SCH == SCH_TENO5 ? coef5<double>(q) : coef<double>(q);
+}
+
 // ==========================================================================
 // Fused 1D stage kernel (grid-wide), SYS in {SYS_ADV, SYS_BURGERS, SYS_EULER1D}.
 // ==========================================================================
+// NF: fields projected together (see tiles1d); 0: one tile per CTA (tiles1d_split).
 template <typename T, int SYS, int SCH, bool PF = false, int NF = 1>
-__global__ void __launch_bounds__(WPB * 32, NF == 1 ? 2 : 1) stage1d_kernel(const Stage1D p) {
+__global__ void __launch_bounds__(WPB * 32, NF == 3 ? 1 : 2) stage1d_kernel(const Stage1D p) {
     constexpr int M = (SYS == SYS_EULER1D) ? 3 : 1;
-    constexpr int NP = (SYS == SYS_EULER1D) ? 3 : 1;
-    __shared__ T s_U[WPB][M][WC];
-    __shared__ T s_gp[WPB][M][WC];
-    __shared__ T s_gm[WPB][M][WC];
-    __shared__ T s_pr[WPB][NP][WC];
-    __shared__ T s_coef[WPB][92];
     __shared__ T s_red[PF ? 3 : 1][WPB];
 
     DevCtl *ctl = p.ctl;
     const bool fixed = p.dt_fixed > 0.0;
     if (!p.rhs_mode && !fixed && !ctl->active) return;  // uniform: the run has ended
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (SCH == SCH_TENO5) {
-        for (int q = lane; q < 35; q += 32) s_coef[warp][q] = coef5<T>(q);
-    } else {
-        for (int q = lane; q < 91; q += 32) s_coef[warp][q] = coef<T>(q);
-    }
 
     TileArgs<T> A;
     if constexpr (sizeof(T) == 8) {
@@ -847,14 +1038,27 @@ __global__ void __launch_bounds__(WPB * 32, NF == 1 ? 2 : 1) stage1d_kernel(cons
     A.ebase = 0;
     A.imul = NF == 1 && nw == WPB;
     A.ctl = ctl;
-    __syncwarp();
     constexpr int NA = PF ? 3 : 1;
     T ws[NA];
 #pragma unroll
     for (int q = 0; q < NA; q++) ws[q] = T(0);
-    const T w0 = tiles1d<T, SYS, SCH, PF, NF>(A, s_U[warp], s_gp[warp], s_gm[warp], s_pr[warp], s_coef[warp],
+    T w0;
+    if constexpr (NF == 0) {
+        __shared__ SplitSmem sm;
+        fill_coef64<SCH>(sm.coef);  // (ordered before its use by the tile's barriers)
+        w0 = tiles1d_split<SCH>(A, sm, blockIdx.x, gridDim.x);
+    } else {
+        __shared__ T s_U[WPB][M][WC];
+        __shared__ T s_gp[WPB][M][WC];
+        __shared__ T s_gm[WPB][M][WC];
+        __shared__ T s_pr[WPB][M][WC];
+        __shared__ T s_coef[92];
+        fill_coef64<SCH>(s_coef);
+        __syncthreads();
+        w0 = tiles1d<T, SYS, SCH, PF, NF>(A, s_U[warp], s_gp[warp], s_gm[warp], s_pr[warp], s_coef,
                                           p.tile_lo + blockIdx.x * nw + warp, gridDim.x * nw,
                                           p.tile_hi > 0 ? p.tile_hi : 0x7fffffff, ws);
+    }
     if constexpr (!PF) ws[0] = w0;
 
     if (!p.rhs_mode) {
@@ -2221,6 +2425,12 @@ inline P with_kt(P p) {
     return p;
 }
 
+// FP64 Euler problems of at most this many tiles per SM run one tile per CTA
+// (tiles1d_split) instead of one per warp.  64 steps, one tile per warp / per CTA:
+// 1600 cells (56 tiles) 3.99 / 2.08 ms, 8000 4.62 / 2.92, 16,000 4.71 / 4.55,
+// 24,000 (5.4 tiles per SM) 6.70 / 6.19, 30,000 (6.8) 6.79 / 7.53.
+constexpr int SPLIT_TILES = 6;
+
 inline int num_sms() {
     static int sms = 0;
     if (!sms) {
@@ -2373,6 +2583,13 @@ cudaError_t launch_stage1d(const Stage1D &p_, cudaStream_t st) {
         if (grid > resident) grid = resident;
         if (p.scheme != SCH_TENO7EXT && p.scheme != SCH_TENO5) return cudaErrorInvalidValue;
         const bool t5 = p.scheme == SCH_TENO5;
+        if (p.sys == SYS_EULER1D && !p.alpha_mode && p.tile_lo == 0 && p.tile_hi <= 0 &&
+            ntiles <= SPLIT_TILES * num_sms()) {
+            const int g = ntiles < 2 * num_sms() ? ntiles : 2 * num_sms();
+            if (t5) stage1d_kernel<T, SYS_EULER1D, SCH_TENO5, false, 0><<<g, WPB * 32, 0, st>>>(p);
+            else stage1d_kernel<T, SYS_EULER1D, SCH_TENO7EXT, false, 0><<<g, WPB * 32, 0, st>>>(p);
+            return cudaGetLastError();
+        }
         // Eight tiles per SM and more fill two CTAs per SM, for which one field at
         // a time leaves the registers and whose products go to the integer pipe
         // (Euler, 20 steps: 40,000 cells 4.3 -> 3.0 ms; 1M cells, 2 steps: 5.08 ->
@@ -2648,6 +2865,263 @@ cudaError_t launch_batch1d(const Batch1D &p, cudaStream_t st) {
     if (p.nbig < 0 || p.nbig > p.ntubes) return cudaErrorInvalidValue;
     batch1d_kernel<T><<<num_sms() * batch1d_per_sm<T>(), WPB * 32, 0, st>>>(with_kt(p));
     return cudaGetLastError();
+}
+
+}  // namespace t7
+
+// ==========================================================================
+// Small 1D problems: whole RK3 steps in one cooperative launch.
+//
+// At a few thousand cells a stage computes for a microsecond or two, and as a
+// launch of its own it also waits for the previous launch's end, its prologue's
+// loads and the last CTA's bookkeeping (three dependent L2 round trips).  Here
+// the CTAs stay, keep t, dt and alpha in registers (every CTA computes the same
+// values), and meet once per stage in grid_max or, where the grid is one cluster,
+// cluster_max, which is both the barrier between stages and the reduction of
+// alpha.  us per step, single launches in a graph -> here: Shu-Osher at 1600
+// cells FP32 19.8 -> 8.8 (12.1 without the cluster), FP64 71 -> 33; advection at
+// 200 cells FP64 19.7 -> 10.2.  Bound by the chain of one tile (some 2 us in FP32)
+// and the barrier (0.5 us in a cluster, 1.3 over the grid).
+// ==========================================================================
+namespace t7 {
+
+// Maximum over the grid of the threads' non-negative v (not NaN), and a barrier:
+// global writes before it are visible to every CTA after it.  Thread 0 publishes
+// the CTA's maximum, tagged, after a fence; every CTA's threads read all slots
+// until the tags match.  Two slot sets alternate: a CTA writes a set again only
+// after every CTA has published the stage between, hence read this one.  The
+// waiting is bounded; false (for the whole CTA) when it gave up.
+constexpr int RUN_SPIN_LIMIT = 1 << 21;
+__device__ __forceinline__ bool grid_max(RunSlot *slots, unsigned tag, double v, double &result, double (*s_red)[WPB]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    auto warp_pos = [](double x) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x = f64_max_pos(x, __shfl_xor_sync(0xffffffffu, x, o));
+        return x;
+    };
+    double (*red)[WPB] = s_red + 2 * (tag & 1u);
+    v = warp_pos(v);
+    if (lane == 0) red[0][warp] = v;
+    __syncthreads();
+    v = red[0][0];
+    for (int w = 1; w < nw; w++) v = f64_max_pos(v, red[0][w]);
+    if (gridDim.x == 1) {
+        result = v;
+        return true;
+    }
+    RunSlot *set = slots + (tag & 1u) * RUN_MAX_CTAS;
+    const unsigned long long want = (unsigned long long)tag << 32;
+    if (threadIdx.x == 0) {
+        const unsigned long long b = f64_bits(v);
+        __threadfence();
+        asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(&set[blockIdx.x]), "l"(want | (b >> 32)),
+                     "l"(want | (b & 0xffffffffull))
+                     : "memory");
+    }
+    bool failed = false;
+    for (int i = threadIdx.x; i < (int)gridDim.x && !failed; i += blockDim.x) {
+        unsigned long long a, b;
+        int spin = 0;
+        do {
+            asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(&set[i]) : "memory");
+            failed = ++spin > RUN_SPIN_LIMIT;
+        } while (!failed && (((a ^ want) | (b ^ want)) >> 32) != 0ull);
+        if (!failed) v = f64_max_pos(v, f64_of((a << 32) | (b & 0xffffffffull)));
+    }
+    __threadfence();
+    v = warp_pos(v);
+    if (lane == 0) red[1][warp] = v;
+    if (__syncthreads_or(failed)) return false;
+    v = red[1][0];
+    for (int w = 1; w < nw; w++) v = f64_max_pos(v, red[1][w]);
+    result = v;
+    return true;
+}
+
+// The same over a grid that is one thread-block cluster: every warp writes its
+// maximum into each CTA's shared memory, and the cluster's hardware barrier
+// orders those and the global writes.  s_cl [2][RUN_CLUSTER * WPB].
+constexpr int RUN_CLUSTER = 16;
+__device__ __forceinline__ double cluster_max(unsigned tag, double v, double (*s_cl)[RUN_CLUSTER * WPB]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, n = gridDim.x * nw;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = f64_max_pos(v, __shfl_xor_sync(0xffffffffu, v, o));
+    double *set = s_cl[tag & 1u];
+    const unsigned mine = (unsigned)__cvta_generic_to_shared(&set[blockIdx.x * nw + warp]);
+    if (lane < (int)gridDim.x) {
+        unsigned remote;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(mine), "r"(lane));
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote), "d"(v) : "memory");
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    double m = 0.0;
+    for (int i = lane; i < n; i += 32) m = f64_max_pos(m, set[i]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = f64_max_pos(m, __shfl_xor_sync(0xffffffffu, m, o));
+    return m;
+}
+
+// SPLIT (FP64 Euler): one tile per CTA (tiles1d_split).
+template <typename T, typename S, int SYS, int SCH, bool SPLIT>
+__global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 || SPLIT ? 2 : 1)) run1d_kernel(const Run1D q) {
+    constexpr int M = (SYS == SYS_EULER1D) ? 3 : 1;
+    constexpr bool F64 = sizeof(T) == 8;
+    constexpr int NWS = SPLIT ? 1 : WPB;
+    __shared__ T s_U[NWS][M][WC];
+    __shared__ T s_gp[NWS][M][WC];
+    __shared__ T s_gm[NWS][M][WC];
+    __shared__ T s_pr[NWS][M][WC];
+    __shared__ T s_coef[F64 ? 92 : 1];
+    __shared__ __align__(16) float s_cf[F64 ? 1 : 32][8];
+    __shared__ double s_red[4][WPB];
+    __shared__ double s_cl[2][RUN_CLUSTER * WPB];
+    const Stage1D &p = q.p;
+    DevCtl *ctl = p.ctl;
+    if (!ctl->active) return;  // uniform: the run has ended
+    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    if constexpr (F64)
+        fill_coef64<SCH>(s_coef);
+    else if constexpr (SCH == SCH_TENO5)
+        fill_delta_table5(s_cf);
+    else
+        fill_delta_table(s_cf);
+    __syncthreads();
+    double alpha = f64_of(ctl->amax[0][0]), t = ctl->t, dt = ctl->dt;
+    const double t_end = ctl->t_end, cfl_dx = ctl->cfl * ctl->dx;
+    int steps = ctl->steps;
+    const int max_steps = ctl->max_steps;
+    TileArgs<T> A;
+    A.masks = nullptr;
+    A.n = p.n;
+    A.cs = A.cso = (size_t)p.n;
+    A.bc_lo = p.bc_lo;
+    A.bc_hi = p.bc_hi;
+    A.dx = p.dx;
+    A.f_dx = p.f_dx;
+    A.gamma = pick<T>(p.gamma, p.f_gamma);
+    A.gm1 = pick<T>(p.gamma - 1.0, p.f_gm1);
+    A.a = pick<T>(p.a, p.f_a);
+    A.eps = pick<T>(p.eps, p.f_eps);
+    A.CT = pick<T>(p.CT, p.f_CT);
+    A.kt = pick<T>(p.kt, p.f_kt);
+    A.rhs_mode = 0;
+    A.ebase = 0;
+    A.imul = false;
+    A.halo = 0;
+    A.ctl = ctl;
+    A.U0 = static_cast<const T *>(q.U);
+    unsigned tag = q.tag;
+    bool ok = true, active = true;
+    for (int step = 0; step < q.nsteps && active && ok; step++) {
+        A.dtT = (T)dt;
+        A.dtD = dt;
+#pragma unroll 1
+        for (int k = 0; k < 3 && ok; k++) {
+            A.Us = static_cast<const T *>(k == 0 ? q.U : k == 1 ? q.U1 : q.U2);
+            A.out = static_cast<T *>(k == 0 ? q.U1 : k == 1 ? q.U2 : q.U);
+            A.stage = k;
+            A.alpha = (T)alpha;
+            T ws;
+            const int tile0 = blockIdx.x * nw + warp, stride = gridDim.x * nw;
+            if constexpr (SPLIT) {
+                __shared__ SplitSmem sm;
+                if (tag == q.tag) fill_coef64<SCH>(sm.coef);  // (ordered by the tile's barriers)
+                ws = tiles1d_split<SCH>(A, sm, blockIdx.x, gridDim.x);
+            } else if constexpr (F64)
+                ws = tiles1d<T, SYS, SCH, false, M>(A, s_U[warp], s_gp[warp], s_gm[warp], s_pr[warp], s_coef, tile0,
+                                                    stride);
+            else
+                ws = tiles1d_f32<SYS, SCH, S>(A, s_U[warp], s_gp[warp], s_gm[warp], s_pr[warp], s_cf, tile0, stride);
+            if (q.cluster)
+                alpha = cluster_max(tag, (double)ws, s_cl);
+            else
+                ok = grid_max(q.slots, tag, (double)ws, alpha, s_red);
+            tag++;
+        }
+        if (!ok) break;
+        t = t + dt;
+        steps++;
+        active = steps < max_steps && t < t_end;
+        dt = div64(cfl_dx, alpha);
+        if (t + dt > t_end) dt = t_end - t;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (!ok) latch_error(ctl, ERR_TIMEOUT, 0);
+        ctl->t = t;
+        ctl->dt = dt;
+        ctl->dt_f = (float)dt;
+        ctl->steps = steps;
+        ctl->active = active;
+        ctl->amax[0][0] = f64_bits(alpha);
+        ctl->alpha_f[0][0] = (float)alpha;
+        ctl->amax[1][0] = 0ull;  // as a step's last stage leaves it
+    }
+}
+
+template <typename T, typename S, int SYS, int SCH, bool SPLIT = false>
+cudaError_t launch_run1d_as(Run1D q, cudaStream_t st) {
+    const void *k = reinterpret_cast<const void *>(&run1d_kernel<T, S, SYS, SCH, SPLIT>);
+    const int ntiles = (q.p.n + WT - 1) / WT;
+    // FP32: up to 16 CTAs of 4 (then 8) warps, one tile a warp, as one cluster;
+    // FP64: one warp per SM while the tiles last (the warps of an SM share its
+    // FP64 pipe), except that a cluster's cheaper barrier outweighs that
+    const bool cluster = !SPLIT && ntiles <= RUN_CLUSTER * WPB && (sizeof(T) == 4 || SYS != SYS_EULER1D);
+    int nw = WPB;
+    if (cluster) {
+        if (sizeof(T) == 8 && ntiles <= RUN_CLUSTER) nw = 1;
+        else if (ntiles <= 4 * RUN_CLUSTER && (sizeof(T) == 8 || ntiles > WPB)) nw = 4;
+    } else if (sizeof(T) == 8 && !SPLIT) {
+        nw = warps_per_cta(ntiles, true);
+    }
+    int grid = SPLIT ? ntiles : (ntiles + nw - 1) / nw;
+    const int cap = num_sms() * resident_ctas(k, nw * 32);
+    if (grid > cap) grid = cap;
+    if (grid > RUN_MAX_CTAS) grid = RUN_MAX_CTAS;
+    q.p = with_kt(q.p);
+    q.cluster = cluster && grid > 1;
+    void *args[] = {&q};
+    if (!q.cluster) return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(nw * 32), args, 0, st);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = grid;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(nw * 32);
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(&cfg, k, args);
+}
+
+template <typename T, typename S>
+cudaError_t launch_run1d(const Run1D &q, cudaStream_t st) {
+    if (q.p.alpha_mode || (q.p.scheme != SCH_TENO7EXT && q.p.scheme != SCH_TENO5)) return cudaErrorNotSupported;
+    const bool t5 = q.p.scheme == SCH_TENO5;
+    // Beyond these sizes the launches of single stages are as fast or faster
+    // (scalar laws in FP64 past one cluster, in FP32 past two tiles per SM, Euler
+    // past eight).
+    const int ntiles = (q.p.n + WT - 1) / WT;
+    const int most = q.p.sys == SYS_EULER1D ? 8 * num_sms() : sizeof(T) == 8 ? RUN_CLUSTER * WPB : 2 * num_sms();
+    if (ntiles > most) return cudaErrorNotSupported;
+    switch (q.p.sys) {
+        case SYS_ADV:
+            return t5 ? launch_run1d_as<T, S, SYS_ADV, SCH_TENO5>(q, st)
+                      : launch_run1d_as<T, S, SYS_ADV, SCH_TENO7EXT>(q, st);
+        case SYS_BURGERS:
+            return t5 ? launch_run1d_as<T, S, SYS_BURGERS, SCH_TENO5>(q, st)
+                      : launch_run1d_as<T, S, SYS_BURGERS, SCH_TENO7EXT>(q, st);
+        case SYS_EULER1D:
+            if constexpr (sizeof(T) == 8)
+                if ((q.p.n + WT - 1) / WT <= SPLIT_TILES * num_sms())
+                    return t5 ? launch_run1d_as<T, S, SYS_EULER1D, SCH_TENO5, true>(q, st)
+                              : launch_run1d_as<T, S, SYS_EULER1D, SCH_TENO7EXT, true>(q, st);
+            return t5 ? launch_run1d_as<T, S, SYS_EULER1D, SCH_TENO5>(q, st)
+                      : launch_run1d_as<T, S, SYS_EULER1D, SCH_TENO7EXT>(q, st);
+        default: return cudaErrorNotSupported;
+    }
 }
 
 }  // namespace t7
