@@ -204,8 +204,8 @@ t7_status t7_run_host(t7_ctx *ctx, void *U_host, double cfl, double t_end, int m
  * fields) and the global Lax-Friedrichs alpha frozen at their values for U;
  * the Roe frame, the characteristic projection, the split fluxes and the flux
  * difference are differentiated exactly.  U, v, out: device [3][nx].  Async.
- * (FP32 contexts take the masks from a forward evaluation of U, so the
- * selection is the forward kernel's bit for bit.) */
+ * (The masks come from a forward evaluation of U, so the selection is the
+ * forward kernel's bit for bit.) */
 t7_status t7_euler_rhs_adjoint(t7_ctx *ctx, const void *U, const void *v, void *out);
 
 /* Adjoint of one SSP-RK3 step (Sec. 2.1) of size dt from the state U (the step's start,

@@ -10,14 +10,12 @@ struct Adjoint1D {
     const void *U;         // state [3][n]
     const void *v;         // adjoint input [3][n]
     void *out;             // accumulates scale (dL/dU)^T v, [3][n] (atomically)
-    const uint8_t *masks;  // nullable: forward Delta codes [2][3][n+1]; else recomputed
+    const uint8_t *masks;  // forward Delta codes [2][3][n+1]
     int n, bc_lo, bc_hi;
-    double dx, eps, CT, gamma;
+    double dx, gamma;
     DevCtl *ctl;
     int slot_in;               // alpha of U (frozen) ...
     const double *alpha_ptr;   // ... or, if not null, read from here
     double scale;              // out += scale (dL/dU)^T v
-    double kt;                 // keep_all_factor(CT), set by the launcher
-    float f_kt;
 };
 }  // namespace t7

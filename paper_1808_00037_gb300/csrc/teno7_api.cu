@@ -39,7 +39,7 @@ struct t7_ctx {
     int b_group;           // warps per tube chosen by t7_batch_autotune (0: not tuned)
     std::vector<double> b_cost;  // estimated cost (cells x estimated steps) of the tubes in processing order
     void *adj[3];          // adjoint work vectors (allocated on first use)
-    uint8_t *adj_masks[3]; // FP32: forward masks of the three stage states
+    uint8_t *adj_masks[3]; // forward masks of the three stage states
     t7::DevCtl *ctl_host;  // pinned mirror for status reads
     // CUDA graph of one chunk of RK3 steps of t7_run (small 1D problems, where
     // launch overhead dominates): captured on an internal stream for the
@@ -842,7 +842,7 @@ static t7_status adj_check(t7_ctx *c) {
             cudaGetLastError();
             return fail(c, T7_ENOMEM, "adjoint buffers");
         }
-        if (c->g.prec == T7_F32 && !c->adj_masks[k] && cudaMalloc((void **)&c->adj_masks[k], mbytes) != cudaSuccess) {
+        if (!c->adj_masks[k] && cudaMalloc((void **)&c->adj_masks[k], mbytes) != cudaSuccess) {
             cudaGetLastError();
             return fail(c, T7_ENOMEM, "adjoint mask buffers");
         }
@@ -850,7 +850,7 @@ static t7_status adj_check(t7_ctx *c) {
     return T7_OK;
 }
 
-// out = (dL/dU)^T v at U with alpha from `slot`, masks frozen (given or recomputed)
+// out = (dL/dU)^T v at U with alpha from `slot` and the given masks
 static cudaError_t adj_apply(t7_ctx *c, const void *U, int slot, const uint8_t *masks, const void *v, void *out) {
     cudaError_t e = cudaMemsetAsync(out, 0, c->ncell * c->m * c->esize, c->stream);
     if (e != cudaSuccess) return e;
@@ -864,8 +864,6 @@ static cudaError_t adj_apply(t7_ctx *c, const void *U, int slot, const uint8_t *
     a.bc_lo = c->g.bc[0];
     a.bc_hi = c->g.bc[1];
     a.dx = c->g.dx;
-    a.eps = eps_of(c->g.eps_x, c->g.dx);
-    a.CT = c->g.CT;
     a.gamma = c->g.gamma;
     a.ctl = c->ctl;
     a.slot_in = slot;
@@ -886,8 +884,6 @@ static cudaError_t adj_accumulate(t7_ctx *c, const void *U, const double *alpha,
     a.bc_lo = c->g.bc[0];
     a.bc_hi = c->g.bc[1];
     a.dx = c->g.dx;
-    a.eps = eps_of(c->g.eps_x, c->g.dx);
-    a.CT = c->g.CT;
     a.gamma = c->g.gamma;
     a.ctl = c->ctl;
     a.alpha_ptr = alpha;
@@ -928,7 +924,7 @@ static cudaError_t combine(t7_ctx *c, void *out, const void *x, const void *y, c
                                : t7::launch_combine_f32(out, x, y, z, c1, c2, c3, N, c->stream);
 }
 
-// FP32: masks of the forward stage kernel at state U (alpha in `slot`), so the
+// Masks of the forward stage kernel at state U (alpha in `slot`), so the
 // adjoint uses exactly the forward's selection
 static cudaError_t forward_masks(t7_ctx *c, const void *U, int slot, uint8_t *masks, void *scratch) {
     t7::Stage1D p = stage_params(c, U, nullptr, scratch);
@@ -944,12 +940,8 @@ t7_status t7_euler_rhs_adjoint(t7_ctx *c, const void *U, const void *v, void *ou
     if (st) return st;
     if (!U || !v || !out) return fail(c, T7_EINVAL, "t7_euler_rhs_adjoint: null array");
     cudaError_t e = alpha_init(c, U);
-    const uint8_t *masks = nullptr;
-    if (e == cudaSuccess && c->g.prec == T7_F32) {
-        e = forward_masks(c, U, 0, c->adj_masks[0], c->adj[0]);
-        masks = c->adj_masks[0];
-    }
-    if (e == cudaSuccess) e = adj_apply(c, U, 0, masks, v, out);
+    if (e == cudaSuccess) e = forward_masks(c, U, 0, c->adj_masks[0], c->adj[0]);
+    if (e == cudaSuccess) e = adj_apply(c, U, 0, c->adj_masks[0], v, out);
     if (e != cudaSuccess) return cuda_fail(c, e, "adjoint launch");
     return T7_OK;
 }
@@ -961,16 +953,14 @@ t7_status t7_rk3_step_adjoint(t7_ctx *c, const void *U, double dt, void *lambda)
     if (!U || !lambda || !(dt > 0.0)) return fail(c, T7_EINVAL, "t7_rk3_step_adjoint: bad argument");
     // Recompute the stage states U1, U2; slot k holds alpha of stage state k
     // while it is needed (the stage-1 launch clears slot 0, so alpha(U) is
-    // taken again before the last adjoint application).  FP32 records each
-    // state's forward masks as soon as its alpha is known.
+    // taken again before the last adjoint application).  Each state's forward
+    // masks are recorded as soon as its alpha is known.
     const void *Us[3] = {U, c->U1, c->U2};
     const uint8_t *mk[3] = {nullptr, nullptr, nullptr};
     cudaError_t e = alpha_init(c, U);
     for (int k = 0; k < 3 && e == cudaSuccess; k++) {
-        if (c->g.prec == T7_F32) {
-            e = forward_masks(c, Us[k], k, c->adj_masks[k], c->adj[0]);
-            mk[k] = c->adj_masks[k];
-        }
+        e = forward_masks(c, Us[k], k, c->adj_masks[k], c->adj[0]);
+        mk[k] = c->adj_masks[k];
         if (k == 2 || e != cudaSuccess) break;
         t7::Stage1D p = stage_params(c, Us[k], k == 0 ? nullptr : U, k == 0 ? c->U1 : c->U2);
         p.rhs_mode = 0;

@@ -303,6 +303,18 @@ __device__ __forceinline__ T pick(double d, float f) {
     }
 }
 
+// Entry t of Table co2's row 0, a constant where t is one.
+template <typename T>
+__device__ __forceinline__ constexpr T row0(int t) {
+    return t == 0   ? T(-1.0 / 140.0)
+           : t == 1 ? T(5.0 / 84.0)
+           : t == 2 ? T(-101.0 / 420.0)
+           : t == 3 ? T(319.0 / 420.0)
+           : t == 4 ? T(107.0 / 210.0)
+           : t == 5 ? T(-19.0 / 210.0)
+                    : T(1.0 / 105.0);
+}
+
 // Table co2 row 0 (the seventh-order polynomial) as immediates: the common
 // smooth case avoids the shared-memory coefficient table.  Same values and
 // summation order as the table path.
