@@ -173,7 +173,7 @@ cudaError_t stage2d(t7_ctx *c, const t7::Stage2D &p) {
     return c->g.prec == T7_F64 ? t7::launch_stage2d_f64(p, c->stream) : t7::launch_stage2d_f32(p, c->stream);
 }
 
-// alpha(U) (per direction in 2D) into slot 0, no slot cleared
+// alpha(U) (per direction in 2D) into slot 0
 cudaError_t alpha_launch(t7_ctx *c, const void *U) {
     if (c->g.sys == T7_EULER2D) {
         t7::Alpha2D a;
@@ -200,13 +200,11 @@ cudaError_t alpha_launch(t7_ctx *c, const void *U) {
     return c->g.prec != T7_F32 ? t7::launch_alpha1d_f64(a, c->stream) : t7::launch_alpha1d_f32(a, c->stream);
 }
 
-// alpha(U) into slot 0 after clearing all slots
-cudaError_t alpha_init(t7_ctx *c, const void *U) {
-    cudaError_t e = cudaMemsetAsync(c->ctl->amax, 0, sizeof(c->ctl->amax), c->stream);
-    if (e != cudaSuccess) return e;
-    return alpha_launch(c, U);
+// alpha(U) into slot 0 for a stage that follows; advection's is |a|, which its
+// stage kernels know
+cudaError_t alpha_for_stage(t7_ctx *c, const void *U) {
+    return c->g.sys == T7_SCALAR_ADVECTION ? cudaSuccess : alpha_launch(c, U);
 }
-
 
 // The last stage of a step (1D) in OUT_PARTS launches over consecutive
 // ranges of warp tiles; each finished range of cells is copied from U to the
@@ -460,7 +458,7 @@ t7_status t7_euler_rhs(t7_ctx *c, const void *U, void *dUdt, uint8_t *masks) {
     t7_status st = check_sys(c);
     if (st) return st;
     if (!U || !dUdt) return fail(c, T7_EINVAL, "t7_euler_rhs: null array");
-    cudaError_t e = alpha_init(c, U);
+    cudaError_t e = alpha_for_stage(c, U);
     if (e != cudaSuccess) return cuda_fail(c, e, "alpha");
     if (c->g.sys == T7_EULER2D) {
         t7::Stage2D p = stage2d_params(c, U, nullptr, dUdt, dUdt);
@@ -485,7 +483,7 @@ t7_status t7_cfl_dt(t7_ctx *c, const void *U, double cfl, double *dt_out) {
     t7_status st = check_sys(c);
     if (st) return st;
     if (!U || !dt_out || !(cfl > 0.0)) return fail(c, T7_EINVAL, "t7_cfl_dt: bad argument");
-    cudaError_t e = alpha_init(c, U);
+    cudaError_t e = alpha_launch(c, U);
     if (e != cudaSuccess) return cuda_fail(c, e, "alpha");
     if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return cuda_fail(c, e, "sync");
     if ((st = collect(c))) return st;
@@ -515,7 +513,7 @@ t7_status t7_rk3_step(t7_ctx *c, void *U, double dt) {
     t7_status st = check_sys(c);
     if (st) return st;
     if (!U || !(dt > 0.0)) return fail(c, T7_EINVAL, "t7_rk3_step: bad argument");
-    cudaError_t e = alpha_init(c, U);
+    cudaError_t e = alpha_for_stage(c, U);
     if (e != cudaSuccess) return cuda_fail(c, e, "alpha");
     if ((e = rk3(c, U, dt)) != cudaSuccess) return cuda_fail(c, e, "stage launch");
     return T7_OK;
@@ -568,8 +566,6 @@ static t7::Stage1D slab_params(t7_ctx *c, const void *Us, const void *U0, void *
 
 // alpha of the slab's cells (the padded array's interior) into *alpha_out
 static cudaError_t slab_alpha_launch(t7_ctx *c, const void *U, double *alpha_out) {
-    cudaError_t e = cudaMemsetAsync(&c->ctl->amax[0][0], 0, 2 * sizeof(unsigned long long), c->stream);
-    if (e != cudaSuccess) return e;
     if (c->g.sys == T7_EULER2D) {
         t7::Alpha2D a;
         memset(&a, 0, sizeof(a));
@@ -939,7 +935,7 @@ t7_status t7_euler_rhs_adjoint(t7_ctx *c, const void *U, const void *v, void *ou
     t7_status st = adj_check(c);
     if (st) return st;
     if (!U || !v || !out) return fail(c, T7_EINVAL, "t7_euler_rhs_adjoint: null array");
-    cudaError_t e = alpha_init(c, U);
+    cudaError_t e = alpha_launch(c, U);
     if (e == cudaSuccess) e = forward_masks(c, U, 0, c->adj_masks[0], c->adj[0]);
     if (e == cudaSuccess) e = adj_apply(c, U, 0, c->adj_masks[0], v, out);
     if (e != cudaSuccess) return cuda_fail(c, e, "adjoint launch");
@@ -957,7 +953,7 @@ t7_status t7_rk3_step_adjoint(t7_ctx *c, const void *U, double dt, void *lambda)
     // masks are recorded as soon as its alpha is known.
     const void *Us[3] = {U, c->U1, c->U2};
     const uint8_t *mk[3] = {nullptr, nullptr, nullptr};
-    cudaError_t e = alpha_init(c, U);
+    cudaError_t e = alpha_launch(c, U);
     for (int k = 0; k < 3 && e == cudaSuccess; k++) {
         e = forward_masks(c, Us[k], k, c->adj_masks[k], c->adj[0]);
         mk[k] = c->adj_masks[k];
@@ -1005,8 +1001,8 @@ t7_status t7_rk3_step_record(t7_ctx *c, const void *U_in, void *U_out, double dt
     double *alpha = reinterpret_cast<double *>(t + L.alpha);
     void *Ust[3] = {const_cast<void *>(U_in), t + L.u1, t + L.u2};
     void *Uo[3] = {t + L.u1, t + L.u2, U_out};
-    cudaError_t e = cudaMemsetAsync(c->ctl->amax, 0, sizeof(c->ctl->amax), c->stream);
-    if (e == cudaSuccess) {
+    cudaError_t e;
+    {
         t7::Alpha1D a;
         memset(&a, 0, sizeof(a));
         a.U = U_in;

@@ -22,6 +22,9 @@ struct DevCtl {
     // alphas of slots 0-2 as the bits of non-negative doubles: [slot][0] 1D
     // global, [slot][0..1] 2D (x, y), [slot][0..2] 1D per characteristic field
     unsigned long long amax[3][3];
+    // the alpha pass reduces here; its last CTA moves the maxima to its slot and
+    // leaves zeros, so that no launch has to clear anything before it
+    unsigned long long acc[3];
     double t, dt, t_end, cfl, dx, dy;
     float alpha_f[3][3];
     float dt_f, pad_f;

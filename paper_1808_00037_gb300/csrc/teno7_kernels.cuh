@@ -371,13 +371,16 @@ __device__ __forceinline__ T poly5(const T *__restrict__ c, const T v0, const T 
 //   plan_step    compute active and the CFL step dt for the next RK step from
 //                alpha(U^n) = amax[slot_out] (oracle's expression order)
 // --------------------------------------------------------------------------
+//   alpha_pass   the maxima are in acc: move them to amax[slot_out]
 __device__ __forceinline__ void finish_launch(DevCtl *ctl, int slot_out, int zero_slot, bool end_of_step,
                                               bool plan_step, bool two_d = false, double *alpha_rec = nullptr,
-                                              int nfield = 1) {
+                                              int nfield = 1, bool alpha_pass = false) {
     __threadfence();
     const unsigned prev = atomicAdd(&ctl->blocks_done, 1u);
     if (prev != gridDim.x * gridDim.y - 1) return;
     __threadfence();
+    if (alpha_pass)
+        for (int q = 0; q < 3; q++) atomicExch(&ctl->amax[slot_out][q], atomicExch(&ctl->acc[q], 0ull));
     const double a = __longlong_as_double((long long)atomicAdd(&ctl->amax[slot_out][0], 0ull));
     const double ay = (two_d || nfield > 1) ? __longlong_as_double((long long)atomicAdd(&ctl->amax[slot_out][1], 0ull))
                                             : 0.0;
@@ -1015,14 +1018,16 @@ __global__ void __launch_bounds__(WPB * 32, NF == 3 ? 1 : 2) stage1d_kernel(cons
 
     TileArgs<T> A;
     if constexpr (sizeof(T) == 8) {
-        A.alpha = p.alpha_in ? *p.alpha_in : __longlong_as_double((long long)ctl->amax[p.slot_in][0]);
+        A.alpha = p.alpha_in         ? *p.alpha_in
+                  : SYS == SYS_ADV ? fabs(p.a)  // (advection runs without an alpha pass)
+                                   : __longlong_as_double((long long)ctl->amax[p.slot_in][0]);
         A.dtT = fixed ? p.dt_fixed : ctl->dt;
         if constexpr (PF) {
 #pragma unroll
             for (int q = 0; q < 3; q++) A.alf[q] = __longlong_as_double((long long)ctl->amax[p.slot_in][q]);
         }
     } else {
-        A.alpha = p.alpha_in ? (float)*p.alpha_in : ctl->alpha_f[p.slot_in][0];
+        A.alpha = p.alpha_in ? (float)*p.alpha_in : SYS == SYS_ADV ? fabsf(p.f_a) : ctl->alpha_f[p.slot_in][0];
         A.dtT = fixed ? p.f_dt_fixed : ctl->dt_f;
     }
     // slab mode: cell 0 follows the padding (the RHS output dU/dt is unpadded)
@@ -1707,7 +1712,7 @@ __global__ void __launch_bounds__(WPB * 32, T7_F32_MINB) stage1d_f32_kernel(cons
     else
         fill_delta_table(s_cf);
     TileArgs<float> A;
-    A.alpha = p.alpha_in ? (float)*p.alpha_in : ctl->alpha_f[p.slot_in][0];
+    A.alpha = p.alpha_in ? (float)*p.alpha_in : SYS == SYS_ADV ? fabsf(p.f_a) : ctl->alpha_f[p.slot_in][0];
     A.dtT = fixed ? p.f_dt_fixed : ctl->dt_f;
     A.dtD = fixed ? p.dt_fixed : ctl->dt;
     // (the pointers stay untyped here: the state type S may be double)
@@ -2259,7 +2264,7 @@ __global__ void __launch_bounds__(WPB * 32, T7_F32_MINB) stage1d_f32fp_kernel(co
     else
         fill_delta_table(s_cf);
     TileArgs<float> A;
-    A.alpha = p.alpha_in ? (float)*p.alpha_in : ctl->alpha_f[p.slot_in][0];
+    A.alpha = p.alpha_in ? (float)*p.alpha_in : SYS == SYS_ADV ? fabsf(p.f_a) : ctl->alpha_f[p.slot_in][0];
     if constexpr (PF) {
 #pragma unroll
         for (int q = 0; q < 3; q++) A.alf[q] = ctl->alpha_f[p.slot_in][q];
@@ -2365,9 +2370,9 @@ __global__ void __launch_bounds__(256) alpha1d_kernel(const Alpha1D p) {
         for (int q = 0; q < NA; q++) {
             T v = s_red[q][0];
             for (int w = 1; w < 8; w++) v = fmax(v, s_red[q][w]);
-            atomicMax(&p.ctl->amax[p.slot][q], (unsigned long long)__double_as_longlong((double)v));
+            atomicMax(&p.ctl->acc[q], (unsigned long long)__double_as_longlong((double)v));
         }
-        finish_launch(p.ctl, p.slot, (p.slot + 1) % 3, false, true, false, p.alpha_rec, NA);
+        finish_launch(p.ctl, p.slot, (p.slot + 1) % 3, false, true, false, p.alpha_rec, NA, true);
     }
 }
 

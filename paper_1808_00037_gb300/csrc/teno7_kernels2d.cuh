@@ -564,9 +564,9 @@ __global__ void __launch_bounds__(256) alpha2d_kernel(const Alpha2D p) {
             vx = fmax(vx, s_red[0][w]);
             vy = fmax(vy, s_red[1][w]);
         }
-        atomicMax(&p.ctl->amax[p.slot][0], (unsigned long long)__double_as_longlong((double)vx));
-        atomicMax(&p.ctl->amax[p.slot][1], (unsigned long long)__double_as_longlong((double)vy));
-        finish_launch(p.ctl, p.slot, (p.slot + 1) % 3, false, true, true, HALO ? p.alpha_rec : nullptr);
+        atomicMax(&p.ctl->acc[0], (unsigned long long)__double_as_longlong((double)vx));
+        atomicMax(&p.ctl->acc[1], (unsigned long long)__double_as_longlong((double)vy));
+        finish_launch(p.ctl, p.slot, (p.slot + 1) % 3, false, true, true, HALO ? p.alpha_rec : nullptr, 1, true);
     }
 }
 
