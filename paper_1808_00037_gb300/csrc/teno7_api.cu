@@ -200,6 +200,46 @@ cudaError_t alpha_launch(t7_ctx *c, const void *U) {
     return c->g.prec != T7_F32 ? t7::launch_alpha1d_f64(a, c->stream) : t7::launch_alpha1d_f32(a, c->stream);
 }
 
+// Parameters of a launch of whole steps or of a right-hand side of a 1D problem:
+// from U through the context's stage buffers to out.
+t7::Run1D run_params(t7_ctx *c, int mode, const void *U, void *out) {
+    t7::Run1D q;
+    memset(&q, 0, sizeof(q));
+    q.p = stage_params(c, nullptr, nullptr, nullptr);
+    q.mode = mode;
+    q.in[0] = U;
+    q.in[1] = c->U1;
+    q.in[2] = c->U2;
+    q.out[0] = mode == t7::RUN_RHS ? out : c->U1;
+    q.out[1] = c->U2;
+    q.out[2] = out;
+    q.nsteps = 1;
+    return q;
+}
+
+// Enqueue it.  Returns false, with nothing enqueued, when the problem is not one
+// for a single launch, the stream is being captured into a graph (whose replays
+// would repeat the launch's tags), or the launch is refused.
+bool run_coop(t7_ctx *c, t7::Run1D &q) {
+    if (!is_1d(c->g.sys) || c->g.alpha_mode != T7_ALPHA_GLOBAL) return false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    q.slots = reinterpret_cast<t7::RunSlot *>(reinterpret_cast<char *>(c->ctl) + CTL_SLOTS);
+    q.tag = c->run_tag;
+    const cudaError_t e = c->g.prec == T7_MIXED ? t7::launch_run1d_mixed(q, c->stream)
+                          : c->g.prec == T7_F64 ? t7::launch_run1d_f64(q, c->stream)
+                                                : t7::launch_run1d_f32(q, c->stream);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    c->run_tag += 3u * (unsigned)q.nsteps + 1u;
+    return true;
+}
+
 // alpha(U) into slot 0 for a stage that follows; advection's is |a|, which its
 // stage kernels know
 cudaError_t alpha_for_stage(t7_ctx *c, const void *U) {
@@ -458,6 +498,9 @@ t7_status t7_euler_rhs(t7_ctx *c, const void *U, void *dUdt, uint8_t *masks) {
     t7_status st = check_sys(c);
     if (st) return st;
     if (!U || !dUdt) return fail(c, T7_EINVAL, "t7_euler_rhs: null array");
+    t7::Run1D q = run_params(c, t7::RUN_RHS, U, dUdt);
+    q.masks[0] = masks;
+    if (run_coop(c, q)) return T7_OK;
     cudaError_t e = alpha_for_stage(c, U);
     if (e != cudaSuccess) return cuda_fail(c, e, "alpha");
     if (c->g.sys == T7_EULER2D) {
@@ -513,6 +556,10 @@ t7_status t7_rk3_step(t7_ctx *c, void *U, double dt) {
     t7_status st = check_sys(c);
     if (st) return st;
     if (!U || !(dt > 0.0)) return fail(c, T7_EINVAL, "t7_rk3_step: bad argument");
+    t7::Run1D q = run_params(c, t7::RUN_STEP, U, U);
+    q.p.dt_fixed = dt;
+    q.p.f_dt_fixed = (float)dt;
+    if (run_coop(c, q)) return T7_OK;
     cudaError_t e = alpha_for_stage(c, U);
     if (e != cudaSuccess) return cuda_fail(c, e, "alpha");
     if ((e = rk3(c, U, dt)) != cudaSuccess) return cuda_fail(c, e, "stage launch");
@@ -719,27 +766,11 @@ static bool run_poll(t7_ctx *c, double t_end, cudaError_t *e) {
     return c->ctl_host->active && !c->ctl_host->err && c->ctl_host->t < t_end;
 }
 
-// k steps of U in one cooperative launch.  Returns false, with nothing enqueued,
-// when the problem is not one for it or the launch is refused.
+// k steps of U in one launch (see run_coop).
 static bool run_steps_coop(t7_ctx *c, void *U, int k) {
-    t7::Run1D q;
-    memset(&q, 0, sizeof(q));
-    q.p = stage_params(c, nullptr, nullptr, nullptr);
-    q.U = U;
-    q.U1 = c->U1;
-    q.U2 = c->U2;
+    t7::Run1D q = run_params(c, t7::RUN_MARCH, U, U);
     q.nsteps = k;
-    q.slots = reinterpret_cast<t7::RunSlot *>(reinterpret_cast<char *>(c->ctl) + CTL_SLOTS);
-    q.tag = c->run_tag;
-    cudaError_t e = c->g.prec == T7_MIXED ? t7::launch_run1d_mixed(q, c->stream)
-                    : c->g.prec == T7_F64 ? t7::launch_run1d_f64(q, c->stream)
-                                          : t7::launch_run1d_f32(q, c->stream);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    c->run_tag += 3u * (unsigned)k;
-    return true;
+    return run_coop(c, q);
 }
 
 // t7_run's loop; host_out (nullable, 1D, only with t_end = inf) receives a
@@ -753,13 +784,12 @@ static t7_status run_core(t7_ctx *c, void *U, double cfl, double t_end, int max_
     if (e != cudaSuccess) return cuda_fail(c, e, "alpha");
     // Steps are launched in chunks; between chunks the host polls whether the
     // device-side clock has reached t_end (a step past it is a no-op anyway).
-    const bool coop = is_1d(c->g.sys);
     const bool graphs = is_1d(c->g.sys) && c->ncell * c->m <= GRAPH_MAX_VALUES;
     int launched = 0;
     while (launched < max_steps) {
         int k = max_steps - launched < RUN_CHUNK ? max_steps - launched : RUN_CHUNK;
         const bool last_chunk = host_out && launched + k == max_steps;
-        if (coop && !last_chunk && run_steps_coop(c, U, k)) {
+        if (!last_chunk && run_steps_coop(c, U, k)) {
             launched += k;
             if (isfinite(t_end) && !run_poll(c, t_end, &e)) {
                 if (e != cudaSuccess) return cuda_fail(c, e, "poll");
@@ -1001,6 +1031,16 @@ t7_status t7_rk3_step_record(t7_ctx *c, const void *U_in, void *U_out, double dt
     double *alpha = reinterpret_cast<double *>(t + L.alpha);
     void *Ust[3] = {const_cast<void *>(U_in), t + L.u1, t + L.u2};
     void *Uo[3] = {t + L.u1, t + L.u2, U_out};
+    t7::Run1D q = run_params(c, t7::RUN_STEP, U_in, U_out);
+    q.p.dt_fixed = dt;
+    q.p.f_dt_fixed = (float)dt;
+    for (int k = 0; k < 3; k++) {
+        q.in[k] = Ust[k];
+        q.out[k] = Uo[k];
+        q.masks[k] = reinterpret_cast<uint8_t *>(t + L.masks[k]);
+    }
+    q.alpha_rec = alpha;
+    if (run_coop(c, q)) return T7_OK;
     cudaError_t e;
     {
         t7::Alpha1D a;

@@ -67,19 +67,26 @@ struct Stage1D {
     float f_kt;
 };
 
-// Several RK3 steps of a 1D problem in one cooperative launch (small problems).
-// Each CTA publishes its maximum of every stage's output in its own slot, tagged
-// with the stage's number, and waits for the others' (see grid_max).
+// A right-hand side or whole RK3 steps of a 1D problem in one launch (small
+// problems).  Each CTA publishes its maximum of every stage's output in its own
+// slot, tagged with the stage's number, and waits for the others' (grid_max).
 constexpr int RUN_MAX_CTAS = 512;
 struct RunSlot {
     unsigned long long w[2];  // tag << 32 | high, low half of the maximum's bits
 };
+enum { RUN_MARCH = 0, RUN_STEP = 1, RUN_RHS = 2 };
 struct Run1D {
-    Stage1D p;       // grid and parameters (Us, U0, out, stage, slot_in unused)
-    void *U, *U1, *U2;
+    Stage1D p;  // grid and parameters; RUN_STEP: dt_fixed (Us, U0, out, stage, slot_in unused)
+    int mode;   // RUN_MARCH: nsteps steps with the control block's clock and CFL step;
+                // RUN_STEP: one step of fixed size; RUN_RHS: out[0] = L(in[0]).
+                // The last two take alpha of in[0] themselves.
+    const void *in[3];  // stage inputs, in[0] = U^n
+    void *out[3];       // stage outputs
+    uint8_t *masks[3];  // nullable: Delta codes of the stages
+    double *alpha_rec;  // nullable: [3] alphas of the stage inputs
     int nsteps;
     RunSlot *slots;  // [2][RUN_MAX_CTAS]
-    unsigned tag;    // tag of the launch's first stage; 3 nsteps tags are used
+    unsigned tag;    // tag of the launch's first exchange; 3 nsteps + 1 tags are used at most
     int cluster;     // the grid is one thread-block cluster (set by the launcher)
 };
 

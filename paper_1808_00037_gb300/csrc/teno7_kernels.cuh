@@ -2978,23 +2978,32 @@ __device__ __forceinline__ double cluster_max(unsigned tag, double v, double (*s
     return m;
 }
 
-// SPLIT (FP64 Euler): one tile per CTA (tiles1d_split).
-template <typename T, typename S, int SYS, int SCH, bool SPLIT>
-__global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 || SPLIT ? 2 : 1)) run1d_kernel(const Run1D q) {
+// What a launch's tiles are: a warp's 29 cells; a CTA's (FP64 Euler); a warp's
+// 61 cells with paired faces (FP32 state).
+enum { FORM_WARP = 0, FORM_CTA = 1, FORM_PAIR = 2 };
+
+template <typename T, typename S, int SYS, int SCH, int FORM>
+__global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 || FORM == FORM_CTA ? 2 : 1)) run1d_kernel(const Run1D q) {
     constexpr int M = (SYS == SYS_EULER1D) ? 3 : 1;
     constexpr bool F64 = sizeof(T) == 8;
-    constexpr int NWS = SPLIT ? 1 : WPB;
+    constexpr int NWS = FORM == FORM_WARP ? WPB : 1, NWP = FORM == FORM_PAIR ? WPB : 1;
     __shared__ T s_U[NWS][M][WC];
     __shared__ T s_gp[NWS][M][WC];
     __shared__ T s_gm[NWS][M][WC];
     __shared__ T s_pr[NWS][M][WC];
+    __shared__ float2 s_U2[NWP][M][WP2];
+    __shared__ float2 s_gp2[NWP][M][WP2];
+    __shared__ float2 s_gm2[NWP][M][WP2];
+    __shared__ float2 s_pr2[NWP][M][WP2];
+    __shared__ float2 s_u02[NWP][M][32];
     __shared__ T s_coef[F64 ? 92 : 1];
     __shared__ __align__(16) float s_cf[F64 ? 1 : 32][8];
     __shared__ double s_red[4][WPB];
     __shared__ double s_cl[2][RUN_CLUSTER * WPB];
     const Stage1D &p = q.p;
     DevCtl *ctl = p.ctl;
-    if (!ctl->active) return;  // uniform: the run has ended
+    const bool march = q.mode == RUN_MARCH;
+    if (march && !ctl->active) return;  // uniform: the run has ended
     const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     if constexpr (F64)
         fill_coef64<SCH>(s_coef);
@@ -3002,13 +3011,7 @@ __global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 || SPLIT ? 2 : 1)) r
         fill_delta_table5(s_cf);
     else
         fill_delta_table(s_cf);
-    __syncthreads();
-    double alpha = f64_of(ctl->amax[0][0]), t = ctl->t, dt = ctl->dt;
-    const double t_end = ctl->t_end, cfl_dx = ctl->cfl * ctl->dx;
-    int steps = ctl->steps;
-    const int max_steps = ctl->max_steps;
     TileArgs<T> A;
-    A.masks = nullptr;
     A.n = p.n;
     A.cs = A.cso = (size_t)p.n;
     A.bc_lo = p.bc_lo;
@@ -3021,76 +3024,123 @@ __global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 || SPLIT ? 2 : 1)) r
     A.eps = pick<T>(p.eps, p.f_eps);
     A.CT = pick<T>(p.CT, p.f_CT);
     A.kt = pick<T>(p.kt, p.f_kt);
-    A.rhs_mode = 0;
+    A.rhs_mode = q.mode == RUN_RHS;
     A.ebase = 0;
     A.imul = false;
     A.halo = 0;
     A.ctl = ctl;
-    A.U0 = static_cast<const T *>(q.U);
+    A.U0 = static_cast<const T *>(q.in[0]);
+    double alpha = 0.0, t = 0.0, dt = p.dt_fixed, t_end = 0.0, cfl_dx = 0.0;
+    int steps = 0, max_steps = 0;
     unsigned tag = q.tag;
     bool ok = true, active = true;
-    for (int step = 0; step < q.nsteps && active && ok; step++) {
-        A.dtT = (T)dt;
+    auto exchange = [&](double v) {
+        if (q.cluster)
+            alpha = cluster_max(tag, v, s_cl);
+        else
+            ok = grid_max(q.slots, tag, v, alpha, s_red);
+        tag++;
+    };
+    __syncthreads();
+    if (march) {
+        alpha = f64_of(ctl->amax[0][0]);
+        t = ctl->t;
+        dt = ctl->dt;
+        t_end = ctl->t_end;
+        cfl_dx = ctl->cfl * ctl->dx;
+        steps = ctl->steps;
+        max_steps = ctl->max_steps;
+    } else if constexpr (SYS == SYS_ADV) {
+        alpha = (double)absval(A.a);
+    } else if constexpr (sizeof(T) == sizeof(S)) {
+        // the alpha pass of alpha1d_kernel
+        T m = T(0);
+        int flag = 0, first = 0x7fffffff;
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < p.n; i += gridDim.x * blockDim.x) {
+            T Uc[M];
+#pragma unroll
+            for (int k = 0; k < M; k++) Uc[k] = static_cast<const T *>(q.in[0])[(size_t)k * A.cs + chk(ctl, i, 0, p.n)];
+            int f = 0;
+            const T v = wavespeed1d<T, SYS>(Uc, A.gm1, A.gamma, A.a, &f);
+            if constexpr (F64) m = f64_max_pos(m, v);
+            else m = fmaxf(m, v);
+            if (f) {
+                flag |= f;
+                first = min(first, i);
+            }
+        }
+        if (flag) latch_error(ctl, flag, first);
+        exchange((double)m);
+    }
+    const bool first_thread = blockIdx.x == 0 && threadIdx.x == 0;
+    const int nsteps = march ? q.nsteps : 1, nstages = A.rhs_mode ? 1 : 3;
+    for (int step = 0; step < nsteps && active && ok; step++) {
+        A.dtT = march ? (T)dt : pick<T>(p.dt_fixed, p.f_dt_fixed);
         A.dtD = dt;
 #pragma unroll 1
-        for (int k = 0; k < 3 && ok; k++) {
-            A.Us = static_cast<const T *>(k == 0 ? q.U : k == 1 ? q.U1 : q.U2);
-            A.out = static_cast<T *>(k == 0 ? q.U1 : k == 1 ? q.U2 : q.U);
+        for (int k = 0; k < nstages && ok; k++) {
+            A.Us = static_cast<const T *>(q.in[k]);
+            A.out = static_cast<T *>(q.out[k]);
+            A.masks = q.masks[k];
             A.stage = k;
             A.alpha = (T)alpha;
+            if (q.alpha_rec && first_thread) q.alpha_rec[k] = alpha;
             T ws;
             const int tile0 = blockIdx.x * nw + warp, stride = gridDim.x * nw;
-            if constexpr (SPLIT) {
+            if constexpr (FORM == FORM_CTA) {
                 __shared__ SplitSmem sm;
-                if (tag == q.tag) fill_coef64<SCH>(sm.coef);  // (ordered by the tile's barriers)
+                if (step == 0 && k == 0) fill_coef64<SCH>(sm.coef);  // (ordered by the tile's barriers)
                 ws = tiles1d_split<SCH>(A, sm, blockIdx.x, gridDim.x);
-            } else if constexpr (F64)
+            } else if constexpr (FORM == FORM_PAIR) {
+                ws = tiles1d_f32_fp<SYS, SCH>(A, s_U2[warp], s_gp2[warp], s_gm2[warp], s_pr2[warp], s_u02[warp], s_cf,
+                                              tile0, stride, nullptr);
+            } else if constexpr (F64) {
                 ws = tiles1d<T, SYS, SCH, false, M>(A, s_U[warp], s_gp[warp], s_gm[warp], s_pr[warp], s_coef, tile0,
                                                     stride);
-            else
+            } else {
                 ws = tiles1d_f32<SYS, SCH, S>(A, s_U[warp], s_gp[warp], s_gm[warp], s_pr[warp], s_cf, tile0, stride);
-            if (q.cluster)
-                alpha = cluster_max(tag, (double)ws, s_cl);
-            else
-                ok = grid_max(q.slots, tag, (double)ws, alpha, s_red);
-            tag++;
+            }
+            if (march || k + 1 < nstages) exchange((double)ws);
         }
-        if (!ok) break;
+        if (!ok || !march) break;
         t = t + dt;
         steps++;
         active = steps < max_steps && t < t_end;
         dt = div64(cfl_dx, alpha);
         if (t + dt > t_end) dt = t_end - t;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (first_thread) {
         if (!ok) latch_error(ctl, ERR_TIMEOUT, 0);
-        ctl->t = t;
-        ctl->dt = dt;
-        ctl->dt_f = (float)dt;
-        ctl->steps = steps;
-        ctl->active = active;
-        ctl->amax[0][0] = f64_bits(alpha);
-        ctl->alpha_f[0][0] = (float)alpha;
-        ctl->amax[1][0] = 0ull;  // as a step's last stage leaves it
+        if (march) {
+            ctl->t = t;
+            ctl->dt = dt;
+            ctl->dt_f = (float)dt;
+            ctl->steps = steps;
+            ctl->active = active;
+            ctl->amax[0][0] = f64_bits(alpha);
+            ctl->alpha_f[0][0] = (float)alpha;
+            ctl->amax[1][0] = 0ull;  // as a step's last stage leaves it
+        }
     }
 }
 
-template <typename T, typename S, int SYS, int SCH, bool SPLIT = false>
+template <typename T, typename S, int SYS, int SCH, int FORM>
 cudaError_t launch_run1d_as(Run1D q, cudaStream_t st) {
-    const void *k = reinterpret_cast<const void *>(&run1d_kernel<T, S, SYS, SCH, SPLIT>);
-    const int ntiles = (q.p.n + WT - 1) / WT;
+    const void *k = reinterpret_cast<const void *>(&run1d_kernel<T, S, SYS, SCH, FORM>);
+    const int width = FORM == FORM_PAIR ? WT2 : WT, ntiles = (q.p.n + width - 1) / width;
     // FP32: up to 16 CTAs of 4 (then 8) warps, one tile a warp, as one cluster;
     // FP64: one warp per SM while the tiles last (the warps of an SM share its
     // FP64 pipe), except that a cluster's cheaper barrier outweighs that
-    const bool cluster = !SPLIT && ntiles <= RUN_CLUSTER * WPB && (sizeof(T) == 4 || SYS != SYS_EULER1D);
+    const bool cluster =
+        FORM == FORM_WARP && ntiles <= RUN_CLUSTER * WPB && (sizeof(T) == 4 || SYS != SYS_EULER1D);
     int nw = WPB;
     if (cluster) {
         if (sizeof(T) == 8 && ntiles <= RUN_CLUSTER) nw = 1;
         else if (ntiles <= 4 * RUN_CLUSTER && (sizeof(T) == 8 || ntiles > WPB)) nw = 4;
-    } else if (sizeof(T) == 8 && !SPLIT) {
+    } else if (sizeof(T) == 8 && FORM == FORM_WARP) {
         nw = warps_per_cta(ntiles, true);
     }
-    int grid = SPLIT ? ntiles : (ntiles + nw - 1) / nw;
+    int grid = FORM == FORM_CTA ? ntiles : (ntiles + nw - 1) / nw;
     const int cap = num_sms() * resident_ctas(k, nw * 32);
     if (grid > cap) grid = cap;
     if (grid > RUN_MAX_CTAS) grid = RUN_MAX_CTAS;
@@ -3113,30 +3163,54 @@ cudaError_t launch_run1d_as(Run1D q, cudaStream_t st) {
     return cudaLaunchKernelExC(&cfg, k, args);
 }
 
+// The form for a problem, or cudaErrorNotSupported where launches of single
+// stages are as fast or faster.  us per step of t7_run, single launches / one
+// launch:
+//   FP64 Euler, one tile per CTA (SPLIT_TILES), else per warp up to eight per SM:
+//     30,000 cells 113 / 106; a right-hand side or one step, whose CTAs would run
+//     several tiles, up to two tiles per SM (20,000 cells: 33 us / 35);
+//   FP64 scalar laws while one cluster holds them (200 cells 20 / 10, 8000 22 / 23);
+//   FP32 Euler, a warp's tiles up to eight per SM (24,000 cells 24 / 18), then
+//     paired faces up to 2^20 cells (50,000 24.2 / 22.7, 700,000 84 / 71, 1M 103 /
+//     92, 2M 159 / 157, 4M 281 / 298: there the tuned two-wave grid wins);
+//   FP32 scalar laws, a warp's tiles up to two per SM, then paired faces up to
+//     seven (Burgers 24,000 16.4 / 15.0, 50,000 16.1 / 16.1, 100,000 17.9 / 21.9);
+//   mixed Euler up to eight tiles per SM, scalar laws up to two.
+// Advection's right-hand side needs no alpha pass, and one plain launch is the
+// cheaper one for the host (8.4 / 10.5).
+template <typename T, typename S, int SYS, int SCH>
+cudaError_t launch_run1d_sys(const Run1D &q, cudaStream_t st) {
+    constexpr bool EULER = SYS == SYS_EULER1D, F64 = sizeof(T) == 8, F32 = sizeof(S) == 4;
+    const int ntiles = (q.p.n + WT - 1) / WT, sms = num_sms();
+    const bool march = q.mode == RUN_MARCH;
+    if (SYS == SYS_ADV && q.mode == RUN_RHS) return cudaErrorNotSupported;
+    if constexpr (F64 && EULER) {
+        if (ntiles <= (march ? SPLIT_TILES : 2) * sms) return launch_run1d_as<T, S, SYS, SCH, FORM_CTA>(q, st);
+        if (!march) return cudaErrorNotSupported;
+    }
+    if (ntiles <= (EULER ? 8 * sms : F64 ? RUN_CLUSTER * WPB : 2 * sms))
+        return launch_run1d_as<T, S, SYS, SCH, FORM_WARP>(q, st);
+    if constexpr (F32)
+        if ((EULER ? q.p.n <= 1 << 20 : ntiles <= 7 * sms) && (SYS != SYS_ADV || q.p.a > 0.0))
+            return launch_run1d_as<T, S, SYS, SCH, FORM_PAIR>(q, st);
+    return cudaErrorNotSupported;
+}
+
 template <typename T, typename S>
 cudaError_t launch_run1d(const Run1D &q, cudaStream_t st) {
     if (q.p.alpha_mode || (q.p.scheme != SCH_TENO7EXT && q.p.scheme != SCH_TENO5)) return cudaErrorNotSupported;
+    if (sizeof(T) != sizeof(S) && q.mode != RUN_MARCH) return cudaErrorNotSupported;  // (mixed: FP64 alpha pass)
     const bool t5 = q.p.scheme == SCH_TENO5;
-    // Beyond these sizes the launches of single stages are as fast or faster
-    // (scalar laws in FP64 past one cluster, in FP32 past two tiles per SM, Euler
-    // past eight).
-    const int ntiles = (q.p.n + WT - 1) / WT;
-    const int most = q.p.sys == SYS_EULER1D ? 8 * num_sms() : sizeof(T) == 8 ? RUN_CLUSTER * WPB : 2 * num_sms();
-    if (ntiles > most) return cudaErrorNotSupported;
     switch (q.p.sys) {
         case SYS_ADV:
-            return t5 ? launch_run1d_as<T, S, SYS_ADV, SCH_TENO5>(q, st)
-                      : launch_run1d_as<T, S, SYS_ADV, SCH_TENO7EXT>(q, st);
+            return t5 ? launch_run1d_sys<T, S, SYS_ADV, SCH_TENO5>(q, st)
+                      : launch_run1d_sys<T, S, SYS_ADV, SCH_TENO7EXT>(q, st);
         case SYS_BURGERS:
-            return t5 ? launch_run1d_as<T, S, SYS_BURGERS, SCH_TENO5>(q, st)
-                      : launch_run1d_as<T, S, SYS_BURGERS, SCH_TENO7EXT>(q, st);
+            return t5 ? launch_run1d_sys<T, S, SYS_BURGERS, SCH_TENO5>(q, st)
+                      : launch_run1d_sys<T, S, SYS_BURGERS, SCH_TENO7EXT>(q, st);
         case SYS_EULER1D:
-            if constexpr (sizeof(T) == 8)
-                if ((q.p.n + WT - 1) / WT <= SPLIT_TILES * num_sms())
-                    return t5 ? launch_run1d_as<T, S, SYS_EULER1D, SCH_TENO5, true>(q, st)
-                              : launch_run1d_as<T, S, SYS_EULER1D, SCH_TENO7EXT, true>(q, st);
-            return t5 ? launch_run1d_as<T, S, SYS_EULER1D, SCH_TENO5>(q, st)
-                      : launch_run1d_as<T, S, SYS_EULER1D, SCH_TENO7EXT>(q, st);
+            return t5 ? launch_run1d_sys<T, S, SYS_EULER1D, SCH_TENO5>(q, st)
+                      : launch_run1d_sys<T, S, SYS_EULER1D, SCH_TENO7EXT>(q, st);
         default: return cudaErrorNotSupported;
     }
 }

@@ -12,8 +12,10 @@ from paper_1808_00037_gb300 import inputs as I
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-# cells: one; a tile (29) and beside; 8, 16, 64 and 128 tiles and one cell more; 152 and 913 tiles
-SIZES = [1, 28, 29, 30, 232, 233, 464, 465, 1856, 1857, 3712, 3713, 29 * 152 + 1, 29 * 912 + 1]
+# cells: one; a tile (29) and beside; 8, 16, 64 and 128 tiles and one cell more; and past 152, 304, 912, 1064 and
+# 1216 tiles, where the form changes
+SIZES = [1, 28, 29, 30, 232, 233, 464, 465, 1856, 1857, 3712, 3713, 29 * 152 + 1, 29 * 304 + 1, 29 * 912 + 1,
+         29 * 1064 + 1, 29 * 1216 + 1]
 SYSTEMS = {"advection": (B.T7_SCALAR_ADVECTION, 0.2, 0), "burgers": (B.T7_BURGERS, 0.5, 0),
            "euler": (B.T7_EULER1D, 0.5, 1)}
 
@@ -94,3 +96,31 @@ def test_runs_on_several_streams_and_threads():
         th.join()
     for k in range(len(jobs)):
         assert torch.equal(want[k], got[k]), jobs[k]
+
+
+@pytest.mark.parametrize("prec", [B.T7_F64, B.T7_F32])
+@pytest.mark.parametrize("system", sorted(SYSTEMS))
+@pytest.mark.parametrize("n", [5, 29 * 16 + 7, 29 * 304, 29 * 304 + 1, 29 * 1216 + 1])
+def test_rhs_and_step_under_capture(system, n, prec):
+    """t7_euler_rhs and t7_rk3_step captured into a CUDA graph (where they are
+    launches of single stages) and replayed equal the plain calls, bit for bit."""
+    sys_, cfl, bc = SYSTEMS[system]
+    U, dx = state(system, n)
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        ctx = B.Context(sys_, n, dx, prec=prec, bc=(bc,) * 4, stream=s)
+        A = torch.tensor(U, dtype=ctx.dtype, device="cuda")
+        S, out, out_s = A.clone(), torch.empty_like(A), torch.empty_like(A)
+        dt = ctx.cfl_dt(A, cfl)
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            ctx.euler_rhs(A, out=out)
+            ctx.rk3_step(A, dt)
+        for _ in range(3):
+            g.replay()
+            ctx.euler_rhs(S, out=out_s)
+            ctx.rk3_step(S, dt)
+            ctx.sync()
+            assert torch.equal(out, out_s) and torch.equal(A, S)
+        ctx.close()
