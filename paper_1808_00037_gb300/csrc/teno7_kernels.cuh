@@ -563,8 +563,13 @@ __device__ __forceinline__ double rk_combine_f64(int stage, double us, double dt
 // projected together: one (128 registers, 16 warps per SM, products by mul64
 // where A.imul allows and the values are in its range; at 1M cells the FP64 pipe
 // is 69% busy, issue 41%) or all three (8 warps, FP64 products, the third shared).
-template <typename T, int SYS, int SCH = SCH_TENO7EXT, bool PF = false, int NF = 1>
-__device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)[WC], T (*sgm)[WC], T (*spr)[WC],
+//
+// LD, the length of a staging row: WC for a warp's own rows, or WCC, the rows of a
+// whole CTA: its WPB warps then take consecutive tiles, one each (no stride), and
+// stage their 242 cells together, each warp in one round instead of two.
+constexpr int WCC = WPB * WT + 16;  // (WPB WT + 10 cells)
+template <typename T, int SYS, int SCH = SCH_TENO7EXT, bool PF = false, int NF = 1, int LD = WC>
+__device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[LD], T (*sgp)[LD], T (*sgm)[LD], T (*spr)[LD],
                                      const T *scoef, int tile0, int tstride, int tile_end = 0x7fffffff,
                                      T *ws3 = nullptr) {
     static_assert(sizeof(T) == 8, "the FP64 tiles");
@@ -582,13 +587,15 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
     const Cut64 cut2 = cut64(4.0 * A.eps, A.CT, A.kt), cut4 = cut64(16.0 * A.eps, A.CT, A.kt);
     DevCtl *ctl = A.ctl;
     T wsmax = T(0);
-    for (int tile = tile0; tile < ntiles; tile += tstride) {
+    constexpr bool CTA = LD != WC;
+    for (int tile = tile0; CTA || tile < ntiles; tile += tstride) {
         const int c0 = tile * WT;
-        // ---- stage cells c0-5 .. c0+33 -----------------------------------
+        // ---- stage cells c0-5 .. c0+33 (CTA: of all its tiles) --------------
+        const int cfirst = CTA ? (tile - (int)(threadIdx.x >> 5)) * WT - 5 : c0 - 5;
         bool zero[2] = {M == 1 && A.kt > T(0), M == 1 && A.kt > T(0)};  // scalar laws: a split vanishes
         uint32_t unranged = 0u;  // a value mul64 does not take
-        for (int c = lane; c < WS; c += 32) {
-            int gi = c0 - 5 + c;
+        for (int c = CTA ? (int)threadIdx.x : lane; c < (CTA ? WPB * WT + 10 : WS); c += CTA ? WPB * 32 : 32) {
+            int gi = cfirst + c;
             if (gi < 0 || gi >= n) gi = ghost_or_halo(gi, n, A.bc_lo, A.bc_hi, A.halo);
             gi = chk(ctl, gi, A.halo ? -HALO_CELLS : 0, n + (A.halo ? HALO_CELLS : 0));
             T U[M], F[M];
@@ -620,7 +627,17 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
                 }
             }
         }
-        __syncwarp();
+        if constexpr (CTA) {
+            unranged = (uint32_t)__syncthreads_or(unranged != 0u);
+            if (tile >= ntiles) break;
+            const int off = c0 - 5 - cfirst;  // this warp's first cell in the rows
+            sU = reinterpret_cast<T (*)[LD]>(&sU[0][off]);
+            sgp = reinterpret_cast<T (*)[LD]>(&sgp[0][off]);
+            sgm = reinterpret_cast<T (*)[LD]>(&sgm[0][off]);
+            spr = reinterpret_cast<T (*)[LD]>(&spr[0][off]);
+        } else {
+            __syncwarp();
+        }
 
         // ---- face j+1/2: frame; then, split by split, projection, cutoff
         // bits, neighbours' bits, selection and polynomial ------------------
@@ -641,7 +658,7 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
 #pragma unroll 1
         for (int s = 0; s < 2; s++) {
             // taps in upwind order: '+' cells j-3+t, '-' cells j+4-t
-            T (*sg)[WC] = (PF || s == 0) ? sgp : sgm;
+            T (*sg)[LD] = (PF || s == 0) ? sgp : sgm;
             const int o = s == 0 ? lane : lane + 7, dir = s == 0 ? 1 : -1;
             // every window of the split zero: all stencils kept, flux +0
             const bool vanishes = M == 1 && !PF && __all_sync(0xffffffffu, s == 0 ? zero[0] : zero[1]);
@@ -795,6 +812,7 @@ __device__ __forceinline__ T tiles1d(const TileArgs<T> &A, T (*sU)[WC], T (*sgp)
                 if (wflag) latch_error(ctl, wflag, A.ebase + i);
             }
         }
+        if constexpr (CTA) break;
         __syncwarp();  // the next tile overwrites this warp's staging rows
     }
 
@@ -1065,16 +1083,19 @@ __global__ void __launch_bounds__(WPB * 32, NF == 3 ? 1 : 2) stage1d_kernel(cons
         fill_coef64<SCH>(sm.coef);  // (ordered before its use by the tile's barriers)
         w0 = tiles1d_split<SCH>(A, sm, blockIdx.x, gridDim.x);
     } else {
-        __shared__ T s_U[WPB][M][WC];
-        __shared__ T s_gp[WPB][M][WC];
-        __shared__ T s_gm[WPB][M][WC];
-        __shared__ T s_pr[WPB][M][WC];
+        constexpr bool CTA = NF == 1 && M == 3 && !PF;  // the CTA's tiles staged together
+        constexpr int LD = CTA ? WCC : WC, NW = CTA ? 1 : WPB;
+        __shared__ T s_U[NW][M][LD];
+        __shared__ T s_gp[NW][M][LD];
+        __shared__ T s_gm[NW][M][LD];
+        __shared__ T s_pr[NW][M][LD];
         __shared__ T s_coef[92];
         fill_coef64<SCH>(s_coef);
-        __syncthreads();
-        w0 = tiles1d<T, SYS, SCH, PF, NF>(A, s_U[warp], s_gp[warp], s_gm[warp], s_pr[warp], s_coef,
-                                          p.tile_lo + blockIdx.x * nw + warp, gridDim.x * nw,
-                                          p.tile_hi > 0 ? p.tile_hi : 0x7fffffff, ws);
+        if constexpr (!CTA) __syncthreads();
+        const int r = CTA ? 0 : warp;
+        w0 = tiles1d<T, SYS, SCH, PF, NF, LD>(A, s_U[r], s_gp[r], s_gm[r], s_pr[r], s_coef,
+                                              p.tile_lo + blockIdx.x * nw + warp, gridDim.x * nw,
+                                              p.tile_hi > 0 ? p.tile_hi : 0x7fffffff, ws);
     }
     if constexpr (!PF) ws[0] = w0;
 
@@ -2610,7 +2631,9 @@ cudaError_t launch_stage1d(const Stage1D &p_, cudaStream_t st) {
         // Eight tiles per SM and more fill two CTAs per SM, for which one field at
         // a time leaves the registers and whose products go to the integer pipe
         // (Euler, 20 steps: 40,000 cells 4.3 -> 3.0 ms; 1M cells, 2 steps: 5.08 ->
-        // 4.10 ms); below, few warps share an SM, each waits on its own chain, and
+        // 4.10 ms).  These run one tile a warp: as a grid of two or four waves with
+        // seven or eight tiles a warp, the last round was half empty (4.10 ms, 3.87
+        // one tile a warp).  Below, few warps share an SM, each waits on its own chain, and
         // all fields together with FP64 products are shorter (1600 cells, 256
         // steps: 18.0 against 20.2 ms).
         const bool many = ntiles >= 8 * num_sms();
@@ -2629,6 +2652,7 @@ cudaError_t launch_stage1d(const Stage1D &p_, cudaStream_t st) {
                 else stage1d_kernel<T, SYS_BURGERS, SCH_TENO7EXT><<<grid, nw * 32, 0, st>>>(p);
                 break;
             case SYS_EULER1D:
+                if (many) grid = (ntiles + WPB - 1) / WPB;
                 if (t5 && many) stage1d_kernel<T, SYS_EULER1D, SCH_TENO5><<<grid, nw * 32, 0, st>>>(p);
                 else if (t5) stage1d_kernel<T, SYS_EULER1D, SCH_TENO5, false, 3><<<grid, nw * 32, 0, st>>>(p);
                 else if (many) stage1d_kernel<T, SYS_EULER1D, SCH_TENO7EXT><<<grid, nw * 32, 0, st>>>(p);

@@ -299,12 +299,12 @@ __global__ void __launch_bounds__(WPB * 32, 2) xsweep2d_kernel(const Stage2D p) 
     __shared__ T s_gp[WPB][4][WC];
     __shared__ T s_gm[WPB][4][WC];
     __shared__ T s_pr[WPB][4][WC];
-    __shared__ T s_coef[WPB][92];
+    __shared__ T s_coef[92];
     DevCtl *ctl = p.ctl;
     const bool fixed = p.dt_fixed > 0.0;
     if (!p.rhs_mode && !fixed && !ctl->active) return;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int q = lane; q < 91; q += 32) s_coef[warp][q] = coef<T>(q);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    fill_coef64<SCH_TENO7EXT>(s_coef);
     const T alpha = alpha2d_in<T, HALO>(p, ctl, 0);
     const T gm1 = pick<T>(p.gamma - 1.0, p.f_gm1);
     const Cut64 cut2 = cut64(4.0 * p.eps_x, p.CT, p.kt), cut4 = cut64(16.0 * p.eps_x, p.CT, p.kt);
@@ -319,8 +319,8 @@ __global__ void __launch_bounds__(WPB * 32, 2) xsweep2d_kernel(const Stage2D p) 
     T (*sgp)[WC] = s_gp[warp];
     T (*sgm)[WC] = s_gm[warp];
     T (*spr)[WC] = s_pr[warp];
-    __syncwarp();
-    for (long tile = (long)blockIdx.x * WPB + warp; tile < ntiles; tile += (long)gridDim.x * WPB) {
+    __syncthreads();
+    for (long tile = (long)blockIdx.x * nw + warp; tile < ntiles; tile += (long)gridDim.x * nw) {
         const int y = (int)(tile / ntx);
         const int c0 = (int)(tile % ntx) * WT;
         const T *row = Us + (size_t)y * nx;
@@ -352,7 +352,7 @@ __global__ void __launch_bounds__(WPB * 32, 2) xsweep2d_kernel(const Stage2D p) 
             [&](int s, int k, int D) {
                 if (masks) p.masks[((size_t)(4 * s + k) * ny + y) * (nx + 1) + (j + 1)] = (uint8_t)D;
             },
-            gm1, cut2, cut4, !__any_sync(0xffffffffu, unranged != 0u), s_coef[warp], fh);
+            gm1, cut2, cut4, !__any_sync(0xffffffffu, unranged != 0u), s_coef, fh);
         if (flag && face_out && j >= -2 && j <= nx)
             latch_error(ctl, (flag & (ERR_NONPHYSICAL | ERR_NONFINITE)) | ((flag & ERR_NOEXIST) ? ERR_NONFINITE : 0),
                         flat_cell(y, j, nx));
@@ -371,29 +371,32 @@ __global__ void __launch_bounds__(WPB * 32, 2) xsweep2d_kernel(const Stage2D p) 
 }
 
 // --------------------------------------------------------------------------
-// y sweep + RK stage.  Block (bx, by): columns 32 bx .. 32 bx + 31, cells of
-// rows 29 by .. 29 by + 28.  Dynamic shared memory (T):
-//   gp, gm, pr  [4][39][33] each; ry [4][29][33]; coef [92]; reductions.
+// FP64 y sweep + RK stage.  Block (bx, by): COLS columns, cells of rows 29 by ..
+// 29 by + 28, COLS / 2 warps (two columns each) and 32 / COLS CTAs per SM, so that
+// one CTA's staging and epilogue run beside another's faces and the last round of
+// blocks is a short one.  16 columns; fewer where those would not fill the SMs
+// (launch_stage2d).  Dynamic shared memory (T):
+//   gp, gm, pr  [4][39][COLS+1] each; ry [4][29][COLS+1]; coef [92]; reductions.
 // --------------------------------------------------------------------------
 constexpr int YB_COLS = 32, YB_ROWS = WT, YB_STAGE = WS, YB_LD = 33;
-constexpr int YW64 = 16;  // warps of an FP64 y-sweep CTA (its shared memory allows one CTA per SM)
 
-template <typename T>
+template <typename T, int COLS>
 constexpr size_t ysweep_smem_bytes() {
-    return sizeof(T) * (3 * 4 * YB_STAGE * YB_LD + 4 * YB_ROWS * YB_LD + 92) + 2 * YW64 * sizeof(T);
+    return sizeof(T) * (3 * 4 * YB_STAGE * (COLS + 1) + 4 * YB_ROWS * (COLS + 1) + 92) + COLS * sizeof(T);
 }
 
-template <typename T, bool HALO>
-__global__ void __launch_bounds__(YW64 * 32, 1) ysweep2d_kernel(const Stage2D p) {
+template <typename T, bool HALO, int COLS>
+__global__ void __launch_bounds__(COLS * 16, 32 / COLS) ysweep2d_kernel(const Stage2D p) {
+    constexpr int LD = COLS + 1, NW = COLS / 2;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *sm = reinterpret_cast<T *>(smem_raw);
-    T *s_gp = sm;                                 // [4][39][33]
-    T *s_gm = s_gp + 4 * YB_STAGE * YB_LD;        // [4][39][33]
-    T *s_pr = s_gm + 4 * YB_STAGE * YB_LD;        // [4][39][33]
-    T *s_ry = s_pr + 4 * YB_STAGE * YB_LD;        // [4][29][33]
-    T *s_coef = s_ry + 4 * YB_ROWS * YB_LD;       // [92]
-    T *s_red = s_coef + 92;                       // [2][YW64]
-    auto at = [](T *base, int c, int r, int col) -> T & { return base[(c * YB_STAGE + r) * YB_LD + col]; };
+    T *s_gp = sm;                                 // [4][39][LD]
+    T *s_gm = s_gp + 4 * YB_STAGE * LD;        // [4][39][LD]
+    T *s_pr = s_gm + 4 * YB_STAGE * LD;        // [4][39][LD]
+    T *s_ry = s_pr + 4 * YB_STAGE * LD;        // [4][29][LD]
+    T *s_coef = s_ry + 4 * YB_ROWS * LD;       // [92]
+    T *s_red = s_coef + 92;                       // [2][NW]
+    auto at = [](T *base, int c, int r, int col) -> T & { return base[(c * YB_STAGE + r) * LD + col]; };
 
     DevCtl *ctl = p.ctl;
     const bool fixed = p.dt_fixed > 0.0;
@@ -402,18 +405,18 @@ __global__ void __launch_bounds__(YW64 * 32, 1) ysweep2d_kernel(const Stage2D p)
     const int nx = p.nx, ny = p.ny;
     const size_t N = (size_t)nx * ny;
     const size_t sv = HALO ? p.sv : N, svo = HALO ? p.svo : N;
-    const int x0 = blockIdx.x * YB_COLS, r0 = blockIdx.y * YB_ROWS;
+    const int x0 = blockIdx.x * COLS, r0 = blockIdx.y * YB_ROWS;
     const T alpha = alpha2d_in<T, HALO>(p, ctl, 1);
     const T gamma = pick<T>(p.gamma, p.f_gamma), gm1 = pick<T>(p.gamma - 1.0, p.f_gm1);
     const Cut64 cut2 = cut64(4.0 * p.eps_y, p.CT, p.kt), cut4 = cut64(16.0 * p.eps_y, p.CT, p.kt);
     const T dy4 = FLUX_SCALE_EULER * p.dy;
     const T *Us = static_cast<const T *>(p.Us);
-    for (int q = tid; q < 91; q += blockDim.x) s_coef[q] = coef<T>(q);
+    fill_coef64<SCH_TENO7EXT>(s_coef);
 
-    // ---- stage rows r0-5 .. r0+33 of columns x0 .. x0+31 (coalesced along x)
+    // ---- stage rows r0-5 .. r0+33 of columns x0 .. x0 + COLS - 1 (coalesced along x)
     uint32_t any_unranged = 0u;
-    for (int idx = tid; idx < YB_STAGE * YB_COLS; idx += blockDim.x) {
-        const int r = idx / YB_COLS, col = idx % YB_COLS, x = x0 + col;
+    for (int idx = tid; idx < YB_STAGE * COLS; idx += blockDim.x) {
+        const int r = idx / COLS, col = idx % COLS, x = x0 + col;
         if (x >= nx) continue;
         int y = r0 - 5 + r;
         y = y_row<HALO>(y, p);
@@ -433,8 +436,8 @@ __global__ void __launch_bounds__(YW64 * 32, 1) ysweep2d_kernel(const Stage2D p)
     }
     const bool imul = !__syncthreads_or(any_unranged != 0u);
 
-    // ---- faces down the columns: warp w takes columns w and w+16
-    for (int col = warp; col < YB_COLS; col += YW64) {
+    // ---- faces down the columns: warp w takes columns w and w + NW
+    for (int col = warp; col < COLS; col += NW) {
         const int x = x0 + col;
         if (x >= nx) break;
         const int j = r0 - 2 + lane;  // face j+1/2 along y
@@ -460,7 +463,7 @@ __global__ void __launch_bounds__(YW64 * 32, 1) ysweep2d_kernel(const Stage2D p)
 #pragma unroll
             for (int k = 0; k < 4; k++) {
                 const T r = div64(fprev[k] - fh[k], dy4);
-                s_ry[(k * YB_ROWS + (lane - 2)) * YB_LD + col] = r;
+                s_ry[(k * YB_ROWS + (lane - 2)) * LD + col] = r;
             }
         }
     }
@@ -479,14 +482,14 @@ __global__ void __launch_bounds__(YW64 * 32, 1) ysweep2d_kernel(const Stage2D p)
         }
     }
     T mx = T(0), my = T(0);
-    for (int idx = tid; idx < YB_ROWS * YB_COLS; idx += blockDim.x) {
-        const int r = idx / YB_COLS, col = idx % YB_COLS, x = x0 + col, y = r0 + r;
+    for (int idx = tid; idx < YB_ROWS * COLS; idx += blockDim.x) {
+        const int r = idx / COLS, col = idx % COLS, x = x0 + col, y = r0 + r;
         if (x >= nx || y >= ny) continue;
         const size_t g = (size_t)chk(p.ctl, y, 0, p.ny) * nx + chk(p.ctl, x, 0, p.nx);
         T o[4];
 #pragma unroll
         for (int k = 0; k < 4; k++) {
-            const T rr = R[(size_t)k * N + g] + s_ry[(k * YB_ROWS + r) * YB_LD + col];
+            const T rr = R[(size_t)k * N + g] + s_ry[(k * YB_ROWS + r) * LD + col];
             if (p.rhs_mode) {
                 out[(size_t)k * svo + g] = rr;
                 continue;
@@ -509,14 +512,14 @@ __global__ void __launch_bounds__(YW64 * 32, 1) ysweep2d_kernel(const Stage2D p)
         my = warp_max(my);
         if (lane == 0) {
             s_red[warp] = mx;
-            s_red[YW64 + warp] = my;
+            s_red[NW + warp] = my;
         }
         __syncthreads();
         if (tid == 0) {
-            T vx = s_red[0], vy = s_red[YW64];
-            for (int w = 1; w < YW64; w++) {
+            T vx = s_red[0], vy = s_red[NW];
+            for (int w = 1; w < NW; w++) {
                 vx = fmax(vx, s_red[w]);
-                vy = fmax(vy, s_red[YW64 + w]);
+                vy = fmax(vy, s_red[NW + w]);
             }
             const int so = (p.stage + 1) % 3;
             atomicMax(&ctl->amax[so][0], (unsigned long long)__double_as_longlong((double)vx));
@@ -1594,26 +1597,37 @@ cudaError_t launch_stage2d_paired(const Stage2D &p_, cudaStream_t st) {
     }
 }
 
+template <typename T, bool HALO, int COLS>
+cudaError_t launch_ysweep2d(const Stage2D &p, cudaStream_t st) {
+    const size_t smem = ysweep_smem_bytes<T, COLS>();
+    cudaError_t e = cudaFuncSetAttribute(ysweep2d_kernel<T, HALO, COLS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
+    if (e != cudaSuccess) return e;
+    dim3 grid((p.nx + COLS - 1) / COLS, (p.ny + YB_ROWS - 1) / YB_ROWS);
+    ysweep2d_kernel<T, HALO, COLS><<<grid, COLS * 16, smem, st>>>(p);
+    return cudaGetLastError();
+}
+
 template <typename T, bool HALO = false>
 cudaError_t launch_stage2d(const Stage2D &p_, cudaStream_t st) {
     if constexpr (sizeof(T) == 4) {
         return launch_stage2d_paired<float, HALO>(p_, st);
     } else {
-    const Stage2D p = with_kt(p_);
-    const int ntx = (p.nx + WT - 1) / WT;
-    long ntiles = (long)ntx * p.ny;
-    long gx = (ntiles + WPB - 1) / WPB;
-    const long cap = (long)num_sms() * 4;
-    if (gx > cap) gx = cap;
-    xsweep2d_kernel<T, HALO><<<(int)gx, WPB * 32, 0, st>>>(p);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    const size_t smem = ysweep_smem_bytes<T>();
-    e = cudaFuncSetAttribute(ysweep2d_kernel<T, HALO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid((p.nx + YB_COLS - 1) / YB_COLS, (p.ny + YB_ROWS - 1) / YB_ROWS);
-    ysweep2d_kernel<T, HALO><<<grid, YW64 * 32, smem, st>>>(p);
-    return cudaGetLastError();
+        const Stage2D p = with_kt(p_);
+        // x sweep: one tile a warp (a grid of four waves left its last round partly
+        // empty: 700 x 650 cells, a step 2.90 -> 2.77 ms), fewer warps per CTA where
+        // that fills more SMs
+        const long ntiles = (long)((p.nx + WT - 1) / WT) * p.ny;
+        const int nw = warps_per_cta(ntiles < (1 << 20) ? (int)ntiles : 1 << 20, true);
+        xsweep2d_kernel<T, HALO><<<(unsigned)((ntiles + nw - 1) / nw), nw * 32, 0, st>>>(p);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        // y sweep: blocks of 16 columns from four per SM on, else of 4 (ms per step
+        // with 32 / 16 / 8 / 4 columns: 700 x 650 2.90 / 2.66 / 2.74 / -, 300 x 290
+        // 0.77 / - / 0.65 / 0.63, 200 x 170 0.59 / - / 0.40 / 0.39)
+        const long rows = (p.ny + YB_ROWS - 1) / YB_ROWS;
+        return rows * ((p.nx + 15) / 16) >= 4 * num_sms() ? launch_ysweep2d<T, HALO, 16>(p, st)
+                                                         : launch_ysweep2d<T, HALO, 4>(p, st);
     }
 }
 
