@@ -627,6 +627,16 @@ __device__ __forceinline__ void cell2d_f32(const float U[4], float gm1, float al
 // back-projection to the physical face flux fh[4].  pr(q, i), gp(c, i),
 // gm(c, i) read staged index i (face j+1/2 <-> cells j-3+t at index lane+t).
 // codes_p / codes_m receive the four fields' Delta codes (5 bits each).
+__device__ __forceinline__ float2 poly_f0_pair(const float2 P[7]) {
+    float2 v = __fmul2_rn(f2(-1.f / 140.f), P[0]);
+    v = __ffma2_rn(f2(5.f / 84.f), P[1], v);
+    v = __ffma2_rn(f2(-101.f / 420.f), P[2], v);
+    v = __ffma2_rn(f2(319.f / 420.f), P[3], v);
+    v = __ffma2_rn(f2(107.f / 210.f), P[4], v);
+    v = __ffma2_rn(f2(-19.f / 210.f), P[5], v);
+    return __ffma2_rn(f2(1.f / 105.f), P[6], v);
+}
+
 template <int DIR, typename PR, typename GP, typename GM>
 __device__ __forceinline__ void face2d_f32(float fh[4], unsigned &codes_p, unsigned &codes_m, int &flag, PR pr,
                                            GP gp, GM gm, const float (*s_cf)[8], float eps4, float CT, float kt,
@@ -678,6 +688,15 @@ __device__ __forceinline__ void face2d_f32(float fh[4], unsigned &codes_p, unsig
         }
         unsigned cp, cm;
         cutoff2(P[1], P[2], P[3], P[4], P[5], eps4, CT, kt, cp, cm);
+        float2 s;
+        if (__all_sync(0xffffffffu, (cp & cm) == 7u)) {
+            // the whole warp keeps every stencil: no codes to exchange or look up
+            codes_p |= 31u << (5 * k);
+            codes_m |= 31u << (5 * k);
+            s = poly_f0_pair(P);
+            f[k] = __fadd_rn(s.x, s.y);
+            continue;
+        }
         const unsigned word = (cp << 1) | (cm << 6);
         const unsigned wl = __shfl_up_sync(0xffffffffu, word, 1);
         const unsigned wr = __shfl_down_sync(0xffffffffu, word, 1);
@@ -685,7 +704,6 @@ __device__ __forceinline__ void face2d_f32(float fh[4], unsigned &codes_p, unsig
         const unsigned dm = (((wr << 1) & 0x200u) | (word & 0x1C0u) | ((wl >> 1) & 0x20u)) >> 5;
         codes_p |= dp << (5 * k);
         codes_m |= dm << (5 * k);
-        float2 s;
         if (dp == 31u && dm == 31u) {
             s = __fmul2_rn(f2(-1.f / 140.f), P[0]);
             s = __ffma2_rn(f2(5.f / 84.f), P[1], s);
@@ -1159,6 +1177,16 @@ __device__ __forceinline__ void face2d_pair(float2 fh[4], unsigned (&D)[2][2], i
                 const float2 tau = tau_pair(P[k][1], P[k][2], P[k][3], P[k][4], P[k][5]);
                 keep_all = keep_all && tau.x < kt * eps4 && tau.y < kt * eps4;
             }
+            if (__all_sync(0xffffffffu, keep_all)) {
+                // the whole warp keeps every stencil: no codes to exchange or look up
+                D[s][0] = 0x3fffffffu;
+#pragma unroll
+                for (int k = 0; k < 3; k++) {
+                    const float2 v = poly_f0_pair(P[k]);
+                    const int fk = k == 2 ? 3 : k;
+                    f[fk] = s == 0 ? v : __fadd2_rn(f[fk], v);
+                }
+            } else {
             unsigned word = 0;
             if (keep_all) {
                 word = (7u << 1) | (7u << 6) | (7u << 11) | (7u << 16) | (7u << 21) | (7u << 26);
@@ -1178,6 +1206,7 @@ __device__ __forceinline__ void face2d_pair(float2 fh[4], unsigned (&D)[2][2], i
                 const int fk = k == 2 ? 3 : k;
                 f[fk] = s == 0 ? v : __fadd2_rn(f[fk], v);
             }
+            }
         }
         // ---- field 2 (shear)
         {
@@ -1189,9 +1218,15 @@ __device__ __forceinline__ void face2d_pair(float2 fh[4], unsigned (&D)[2][2], i
             }
             unsigned cA, cB;
             cutoff2(P[1], P[2], P[3], P[4], P[5], eps4, CT, kt, cA, cB);
-            const unsigned Dw = pair_delta<1>((cA << 1) | (cB << 6), s, lane, WRAP);
-            D[s][1] = Dw;
-            const float2 v = pair_poly(P, Dw & 31u, (Dw >> 5) & 31u, s_cf);
+            float2 v;
+            if (__all_sync(0xffffffffu, (cA & cB) == 7u)) {
+                D[s][1] = 0x3ffu;
+                v = poly_f0_pair(P);
+            } else {
+                const unsigned Dw = pair_delta<1>((cA << 1) | (cB << 6), s, lane, WRAP);
+                D[s][1] = Dw;
+                v = pair_poly(P, Dw & 31u, (Dw >> 5) & 31u, s_cf);
+            }
             f[2] = s == 0 ? v : __fadd2_rn(f[2], v);
         }
     }
@@ -1221,7 +1256,7 @@ __device__ __forceinline__ unsigned pair_code(const unsigned (&D)[2][2], int s, 
 // 71 cells c0-5 .. c0+65 are staged as pairs (cell i, cell i + 32), one tile
 // ahead in registers.  FP32 state only.
 // --------------------------------------------------------------------------
-template <bool HALO>
+template <bool HALO, bool CODES>  // CODES: a right-hand side that may want its codes
 __global__ void __launch_bounds__(WPB * 32, 2) xsweep2d_f32fp_kernel(const Stage2D p) {
     __shared__ float2 s_pr[WPB][4][WP2];
     __shared__ float2 s_gp[WPB][4][WP2];
@@ -1322,7 +1357,7 @@ __global__ void __launch_bounds__(WPB * 32, 2) xsweep2d_f32fp_kernel(const Stage
             fh, D, flagA, flagB, [&](int q, int i) { return spr[q][i]; },
             [&](int s, int cc, int i) { return s == 0 ? sgp[cc][i] : sgm[cc][i]; }, s_cf, eps4, CT, kt, gm1, lane);
         const int jA = c0 - 2 + lane, jB = c0 + 30 + lane;  // faces, and the cells they update
-        if (p.rhs_mode && p.masks) {
+        if (CODES && p.rhs_mode && p.masks) {
 #pragma unroll
             for (int h = 0; h < 2; h++) {
                 const int j = h == 0 ? jA : jB;
@@ -1365,8 +1400,12 @@ inline constexpr size_t ysweep_f32p_smem_bytes() {
                             2 * WPB);
 }
 
-template <typename S, bool HALO>  // S = float (the FP32 state) only
+// S = float (the FP32 state) only.  MODE 0, 1, 2: RK stage MODE without codes;
+// -1: as p says.
+template <typename S, bool HALO, int MODE>
 __global__ void __launch_bounds__(WPB * 32, 2) ysweep2d_f32p_kernel(const Stage2D p) {
+    const bool rhs_mode = MODE < 0 && p.rhs_mode;
+    const int stage = MODE < 0 ? p.stage : MODE;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float *s_ry = reinterpret_cast<float *>(smem_raw);  // [4][29][33]
     float *s_gp = s_ry + 4 * YB_ROWS * YB_LD;            // [4][39][33]
@@ -1381,7 +1420,7 @@ __global__ void __launch_bounds__(WPB * 32, 2) ysweep2d_f32p_kernel(const Stage2
 
     DevCtl *ctl = p.ctl;
     const bool fixed = p.dt_fixed > 0.0;
-    if (!p.rhs_mode && !fixed && !ctl->active) return;
+    if (!rhs_mode && !fixed && !ctl->active) return;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nx = p.nx, ny = p.ny;
     const size_t N = (size_t)nx * ny;
@@ -1395,8 +1434,8 @@ __global__ void __launch_bounds__(WPB * 32, 2) ysweep2d_f32p_kernel(const Stage2
     const float *U0 = static_cast<const float *>(p.U0);
     float *out = static_cast<float *>(p.out);
     const float idy = 1.f / p.f_dy;
-    const float dtF = p.rhs_mode ? 0.f : (fixed ? p.f_dt_fixed : ctl->dt_f);
-    const bool use_u0 = !p.rhs_mode && p.stage > 0;
+    const float dtF = rhs_mode ? 0.f : (fixed ? p.f_dt_fixed : ctl->dt_f);
+    const bool use_u0 = !rhs_mode && stage > 0;
     fill_delta_table(s_cf);
     // running max(|u|+c), max(|v|+c) of the CTA's output cells, as the bit
     // patterns of non-negative floats (ordered like the values)
@@ -1459,7 +1498,7 @@ __global__ void __launch_bounds__(WPB * 32, 2) ysweep2d_f32p_kernel(const Stage2
                 [&](int cc, int i) { return at(s_gp, cc, i, col); },
                 [&](int cc, int i) { return at(s_gm, cc, i, col); }, s_cf, eps4, CT, kt, gm1, lane);
             const bool face_out = lane >= 1 && lane <= 30;
-            if (p.rhs_mode && p.masks && face_out && j >= -1 && j <= ny - 1) {
+            if (MODE < 0 && rhs_mode && p.masks && face_out && j >= -1 && j <= ny - 1) {
                 uint8_t *ym = p.masks + (size_t)8 * ny * (nx + 1);
 #pragma unroll
                 for (int k = 0; k < 4; k++) {
@@ -1492,7 +1531,7 @@ __global__ void __launch_bounds__(WPB * 32, 2) ysweep2d_f32p_kernel(const Stage2
 #pragma unroll
                     for (int k = 0; k < 4; k++) {
                         Rv[e][k] = R[(size_t)k * N + gi];
-                        Uv[e][k] = p.rhs_mode ? 0.f : Us[(size_t)k * sv + gi];
+                        Uv[e][k] = rhs_mode ? 0.f : Us[(size_t)k * sv + gi];
                         U0v[e][k] = use_u0 ? U0[(size_t)k * sv + gi] : 0.f;
                     }
                 }
@@ -1507,15 +1546,15 @@ __global__ void __launch_bounds__(WPB * 32, 2) ysweep2d_f32p_kernel(const Stage2
 #pragma unroll
                 for (int k = 0; k < 4; k++) {
                     const float rr = Rv[e][k] + s_ry[(k * YB_ROWS + r) * YB_LD + col];
-                    if (p.rhs_mode) {
+                    if (rhs_mode) {
                         out[(size_t)k * svo + gi] = rr;
                         continue;
                     }
                     float o;
                     const float v = fmaf(dtF, rr, Uv[e][k]);
-                    if (p.stage == 0) {
+                    if (stage == 0) {
                         o = v;
-                    } else if (p.stage == 1) {
+                    } else if (stage == 1) {
                         o = fmaf(0.75f, U0v[e][k], 0.25f * v);
                     } else {
                         const float u0 = U0v[e][k];
@@ -1524,7 +1563,7 @@ __global__ void __launch_bounds__(WPB * 32, 2) ysweep2d_f32p_kernel(const Stage2
                     out[(size_t)k * svo + gi] = o;
                     of[k] = o;
                 }
-                if (!p.rhs_mode) {
+                if (!rhs_mode) {
                     int wflag = 0;
                     float sx, sy;
                     wavespeed2d<float>(of, gm1, gamma, sx, sy, &wflag);
@@ -1534,7 +1573,7 @@ __global__ void __launch_bounds__(WPB * 32, 2) ysweep2d_f32p_kernel(const Stage2
                 }
             }
         }
-        if (!p.rhs_mode) {
+        if (!rhs_mode) {
             mx = warp_max(mx);
             my = warp_max(my);
             if (lane == 0) {
@@ -1544,14 +1583,14 @@ __global__ void __launch_bounds__(WPB * 32, 2) ysweep2d_f32p_kernel(const Stage2
         }
         __syncthreads();  // s_ry and the staged arrays are rewritten by the next block
     }
-    if (!p.rhs_mode) {
+    if (!rhs_mode) {
         __syncthreads();
         if (tid == 0) {
             const float vx = __int_as_float(s_amax[0]), vy = __int_as_float(s_amax[1]);
-            const int so = (p.stage + 1) % 3;
+            const int so = (stage + 1) % 3;
             atomicMax(&ctl->amax[so][0], (unsigned long long)__double_as_longlong((double)vx));
             atomicMax(&ctl->amax[so][1], (unsigned long long)__double_as_longlong((double)vy));
-            finish_launch(ctl, so, (p.stage + 2) % 3, p.stage == 2 && !fixed, p.stage == 2 && !fixed, true,
+            finish_launch(ctl, so, (stage + 2) % 3, stage == 2 && !fixed, stage == 2 && !fixed, true,
                           HALO ? p.alpha_rec : nullptr);
         }
     }
@@ -1570,21 +1609,30 @@ cudaError_t launch_stage2d_paired(const Stage2D &p_, cudaStream_t st) {
     if constexpr (sizeof(S) == 4) {
         // FP32 state: paired faces, 61-cell tiles
         const long gx2 = ((long)((p.nx + WT2 - 1) / WT2) * p.ny + WPB - 1) / WPB;
-        xsweep2d_f32fp_kernel<HALO><<<(int)(gx2 < cap ? gx2 : cap), WPB * 32, 0, st>>>(p);
+        const int g = (int)(gx2 < cap ? gx2 : cap);
+        if (p.rhs_mode) xsweep2d_f32fp_kernel<HALO, true><<<g, WPB * 32, 0, st>>>(p);
+        else xsweep2d_f32fp_kernel<HALO, false><<<g, WPB * 32, 0, st>>>(p);
     } else {
         xsweep2d_f32_kernel<S, HALO><<<(int)gx, WPB * 32, 0, st>>>(p);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     if constexpr (sizeof(S) == 4) {
-        // FP32 state: persistent CTAs (two per SM) with the next block prefetched
-        const size_t smem = ysweep_f32p_smem_bytes();
-        e = cudaFuncSetAttribute(ysweep2d_f32p_kernel<S, HALO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-        const long nb = (long)((p.nx + YB_COLS - 1) / YB_COLS) * ((p.ny + YB_ROWS - 1) / YB_ROWS);
-        const long cap = (long)num_sms() * 2;
-        ysweep2d_f32p_kernel<S, HALO><<<(int)(nb < cap ? nb : cap), WPB * 32, smem, st>>>(p);
-        return cudaGetLastError();
+        // FP32 state: persistent CTAs (two per SM) with the next block prefetched;
+        // each stage its own instantiation
+        auto launch = [&](auto kernel) {
+            const size_t smem = ysweep_f32p_smem_bytes();
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+            const long nb = (long)((p.nx + YB_COLS - 1) / YB_COLS) * ((p.ny + YB_ROWS - 1) / YB_ROWS);
+            const long most = (long)num_sms() * 2;
+            kernel<<<(int)(nb < most ? nb : most), WPB * 32, smem, st>>>(p);
+            return cudaGetLastError();
+        };
+        if (p.rhs_mode) return launch(ysweep2d_f32p_kernel<S, HALO, -1>);
+        return p.stage == 0   ? launch(ysweep2d_f32p_kernel<S, HALO, 0>)
+               : p.stage == 1 ? launch(ysweep2d_f32p_kernel<S, HALO, 1>)
+                              : launch(ysweep2d_f32p_kernel<S, HALO, 2>);
     } else {
         // mixed precision (FP64 state): one block per CTA
         const size_t smem = ysweep_f32_smem_bytes<S>();
