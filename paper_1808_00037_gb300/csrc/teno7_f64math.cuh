@@ -323,9 +323,9 @@ T7_HD void split_f32(double x, float &h, float &l) {
 // within 2.2e-6 of itself plus A = 2^-60 max|w|^2 (1e-36 covers underflow).
 //   kept     tau + 1e-5 (beta_0 + beta_2) + A < kt (0.9999 (beta_min + eps) - A)
 //            implies tau < kt (beta_min + eps): all bits set (keep_all_factor).
-//   decided  where tau > 0.01 (beta_0 + beta_2) and A is below 1e-5 of the
-//            smallest beta + eps, g_k is known within 2.5e-4 and chi_k / C_T
-//            within 1%: the FP32 comparison holds unless chi_k is within 3% of
+//   decided  where tau > 0.003 (beta_0 + beta_2) and A is below 1e-5 of the
+//            smallest beta + eps, g_k is known within 7.5e-4 and chi_k / C_T
+//            within 2%: the FP32 comparison holds unless chi_k is within 3% of
 //            C_T.
 // Everything else, and what FP32 cannot hold, goes to the FP64 evaluation.
 T7_HD unsigned cutoff_bits(double w0, double w1, double w2, double w3, double w4, const Cut64 &K) {
@@ -346,7 +346,7 @@ T7_HD unsigned cutoff_bits(double w0, double w1, double w2, double w3, double w4
     const float A = fmaf(W * W, 8.673617379884035e-19f, 1e-36f);
     const float sum = b0 + b2, tau = fabsf(b0 - b2), bm = fminf(fminf(b0, b1), b2) + K.e4;
     if (fmaf(1e-5f, sum, tau) + A < K.ktf * fmaf(0.9999f, bm, -A)) return 7u;
-    if (K.ctf > 0.f && tau > 0.01f * sum && A < 1e-5f * bm) {
+    if (K.ctf > 0.f && tau > 0.003f * sum && A < 1e-5f * bm) {
         const float g0 = fmaf(tau, f32_rcp(b0 + K.e4), 1.f), g1 = fmaf(tau, f32_rcp(b1 + K.e4), 1.f);
         const float g2 = fmaf(tau, f32_rcp(b2 + K.e4), 1.f);
         const float gm = fmaxf(fmaxf(g0, g1), g2), rg = f32_rcp(gm);
