@@ -3014,41 +3014,30 @@ cudaError_t launch_batch1d(const Batch1D &p, cudaStream_t st) {
 // ==========================================================================
 namespace t7 {
 
-// Maximum over the grid of the threads' non-negative v (not NaN), and a barrier:
-// global writes before it are visible to every CTA after it.  Thread 0 publishes
-// the CTA's maximum, tagged, after a fence; every CTA's threads read all slots
-// until the tags match.  Two slot sets alternate: a CTA writes a set again only
-// after every CTA has published the stage between, hence read this one.  The
-// waiting is bounded; false (for the whole CTA) when it gave up.
+// Maximum over a warp of non-negative values (not NaN), ordered like their bits.
+__device__ __forceinline__ double warp_max_pos(double v) {
+    const unsigned long long b = f64_bits(v);
+    const unsigned hi = (unsigned)(b >> 32), m = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned l = __reduce_max_sync(0xffffffffu, hi == m ? (unsigned)b : 0u);
+    return f64_of((unsigned long long)m << 32 | l);
+}
+
+// A CTA's slot of the exchange `tag`, and the read of all slots by one warp: waits
+// (bounded) until every slot carries the tag and returns the maximum; false when
+// it gave up.
 constexpr int RUN_SPIN_LIMIT = 1 << 21;
-__device__ __forceinline__ bool grid_max(RunSlot *slots, unsigned tag, double v, double &result, double (*s_red)[WPB]) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    auto warp_pos = [](double x) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x = f64_max_pos(x, __shfl_xor_sync(0xffffffffu, x, o));
-        return x;
-    };
-    double (*red)[WPB] = s_red + 2 * (tag & 1u);
-    v = warp_pos(v);
-    if (lane == 0) red[0][warp] = v;
-    __syncthreads();
-    v = red[0][0];
-    for (int w = 1; w < nw; w++) v = f64_max_pos(v, red[0][w]);
-    if (gridDim.x == 1) {
-        result = v;
-        return true;
-    }
-    RunSlot *set = slots + (tag & 1u) * RUN_MAX_CTAS;
+__device__ __forceinline__ void publish_max(RunSlot *slots, unsigned tag, double v) {
+    const unsigned long long b = f64_bits(v), t = (unsigned long long)tag << 32;
+    asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(
+                     &slots[(tag & 1u) * RUN_MAX_CTAS + blockIdx.x]),
+                 "l"(t | (b >> 32)), "l"(t | (b & 0xffffffffull))
+                 : "memory");
+}
+__device__ __forceinline__ bool read_slots(const RunSlot *slots, unsigned tag, int first, int stride, double &v) {
+    const RunSlot *set = slots + (tag & 1u) * RUN_MAX_CTAS;
     const unsigned long long want = (unsigned long long)tag << 32;
-    if (threadIdx.x == 0) {
-        const unsigned long long b = f64_bits(v);
-        __threadfence();
-        asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(&set[blockIdx.x]), "l"(want | (b >> 32)),
-                     "l"(want | (b & 0xffffffffull))
-                     : "memory");
-    }
     bool failed = false;
-    for (int i = threadIdx.x; i < (int)gridDim.x && !failed; i += blockDim.x) {
+    for (int i = first; i < (int)gridDim.x && !failed; i += stride) {
         unsigned long long a, b;
         int spin = 0;
         do {
@@ -3057,13 +3046,36 @@ __device__ __forceinline__ bool grid_max(RunSlot *slots, unsigned tag, double v,
         } while (!failed && (((a ^ want) | (b ^ want)) >> 32) != 0ull);
         if (!failed) v = f64_max_pos(v, f64_of((a << 32) | (b & 0xffffffffull)));
     }
+    return !failed;
+}
+
+// Maximum over the grid of the threads' non-negative v (not NaN), and a barrier:
+// global writes before it are visible to every CTA after it.  Thread 0 publishes
+// the CTA's maximum, tagged, after a fence; every CTA's threads read all slots
+// until the tags match.  Two slot sets alternate: a CTA writes a set again only
+// after every CTA has published the stage between, hence read this one.  The
+// waiting is bounded; false (for the whole CTA) when it gave up.
+__device__ __forceinline__ bool grid_max(RunSlot *slots, unsigned tag, double v, double &result, double (*s_red)[WPB]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    double (*red)[WPB] = s_red + 2 * (tag & 1u);
+    v = warp_max_pos(v);
+    if (lane == 0) red[0][warp] = v;
+    __syncthreads();
+    v = warp_max_pos(lane < nw ? red[0][lane] : 0.0);
+    if (gridDim.x == 1) {
+        result = v;
+        return true;
+    }
+    if (threadIdx.x == 0) {
+        __threadfence();
+        publish_max(slots, tag, v);
+    }
+    const bool failed = !read_slots(slots, tag, threadIdx.x, blockDim.x, v);
     __threadfence();
-    v = warp_pos(v);
+    v = warp_max_pos(v);
     if (lane == 0) red[1][warp] = v;
     if (__syncthreads_or(failed)) return false;
-    v = red[1][0];
-    for (int w = 1; w < nw; w++) v = f64_max_pos(v, red[1][w]);
-    result = v;
+    result = warp_max_pos(lane < nw ? red[1][lane] : 0.0);
     return true;
 }
 
@@ -3073,8 +3085,7 @@ __device__ __forceinline__ bool grid_max(RunSlot *slots, unsigned tag, double v,
 constexpr int RUN_CLUSTER = 16;
 __device__ __forceinline__ double cluster_max(unsigned tag, double v, double (*s_cl)[RUN_CLUSTER * WPB]) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, n = gridDim.x * nw;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = f64_max_pos(v, __shfl_xor_sync(0xffffffffu, v, o));
+    v = warp_max_pos(v);
     double *set = s_cl[tag & 1u];
     const unsigned mine = (unsigned)__cvta_generic_to_shared(&set[blockIdx.x * nw + warp]);
     if (lane < (int)gridDim.x) {
@@ -3085,9 +3096,7 @@ __device__ __forceinline__ double cluster_max(unsigned tag, double v, double (*s
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     double m = 0.0;
     for (int i = lane; i < n; i += 32) m = f64_max_pos(m, set[i]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = f64_max_pos(m, __shfl_xor_sync(0xffffffffu, m, o));
-    return m;
+    return warp_max_pos(m);
 }
 
 // What a launch's tiles are: a warp's 29 cells; a CTA's (FP64 Euler); a warp's
