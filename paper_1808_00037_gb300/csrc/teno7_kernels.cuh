@@ -229,12 +229,21 @@ __device__ __forceinline__ int chk(DevCtl *ctl, int i, int lo, int hi) {
     return i;
 }
 
-template <typename T>
-__device__ __forceinline__ T warp_max(T v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
+// Maximum over a warp of non-negative values (not NaN), ordered like their bits.
+__device__ __forceinline__ double warp_max_pos(double v) {
+    const unsigned long long b = f64_bits(v);
+    const unsigned hi = (unsigned)(b >> 32), m = __reduce_max_sync(0xffffffffu, hi);
+    const unsigned l = __reduce_max_sync(0xffffffffu, hi == m ? (unsigned)b : 0u);
+    return f64_of((unsigned long long)m << 32 | l);
 }
+
+// Maximum over a warp of wave speeds (non-negative, not NaN).
+__device__ __forceinline__ double warp_max(double v) { return warp_max_pos(v); }
+__device__ __forceinline__ float warp_max(float v) {
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+}
+__device__ __forceinline__ double speed_max(double x, double y) { return f64_max_pos(x, y); }
+__device__ __forceinline__ float speed_max(float x, float y) { return fmaxf(x, y); }
 
 // Largest characteristic speed of one cell (1D systems) and its validity.
 // FP64 follows the oracle's expression order; FP32 uses fast reciprocals.
@@ -1153,7 +1162,7 @@ __global__ void __launch_bounds__(WPB * 32, NF == 3 ? 1 : 2) stage1d_kernel(cons
 #pragma unroll
             for (int q = 0; q < NA; q++) {
                 T v = s_red[q][0];
-                for (int w = 1; w < nw; w++) v = fmax(v, s_red[q][w]);
+                for (int w = 1; w < nw; w++) v = speed_max(v, s_red[q][w]);
                 atomicMax(&ctl->amax[so][q], (unsigned long long)__double_as_longlong((double)v));
             }
             finish_launch(ctl, so, (p.stage + 2) % 3, p.stage == 2 && !fixed && !p.partial,
@@ -2451,9 +2460,9 @@ __global__ void __launch_bounds__(256) alpha1d_kernel(const Alpha1D p) {
             T w[3];
             wavespeeds1d<T>(Uc, gm1, gamma, w, &f);
 #pragma unroll
-            for (int q = 0; q < 3; q++) m[q] = fmax(m[q], w[q]);
+            for (int q = 0; q < 3; q++) m[q] = speed_max(m[q], w[q]);
         } else {
-            m[0] = fmax(m[0], wavespeed1d<T, SYS>(Uc, gm1, gamma, a, &f));
+            m[0] = speed_max(m[0], wavespeed1d<T, SYS>(Uc, gm1, gamma, a, &f));
         }
         if (f) {
             flag |= f;
@@ -2471,7 +2480,7 @@ __global__ void __launch_bounds__(256) alpha1d_kernel(const Alpha1D p) {
 #pragma unroll
         for (int q = 0; q < NA; q++) {
             T v = s_red[q][0];
-            for (int w = 1; w < 8; w++) v = fmax(v, s_red[q][w]);
+            for (int w = 1; w < 8; w++) v = speed_max(v, s_red[q][w]);
             atomicMax(&p.ctl->acc[q], (unsigned long long)__double_as_longlong((double)v));
         }
         finish_launch(p.ctl, p.slot, (p.slot + 1) % 3, false, true, false, p.alpha_rec, NA, true);
@@ -2830,7 +2839,7 @@ __global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 ? 2 : 1)) batch1d_ke
         if (lane == 0) s_red[warp] = v;
         group_sync(group, G);
         T m = s_red[group * G];
-        for (int w = 1; w < G; w++) m = fmax(m, s_red[group * G + w]);
+        for (int w = 1; w < G; w++) m = speed_max(m, s_red[group * G + w]);
         group_sync(group, G);
         return m;
     };
@@ -2846,7 +2855,7 @@ __global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 ? 2 : 1)) batch1d_ke
         for (int i = wg * 32 + lane; i < n; i += G * 32) {
             T Uc[3] = {U[off + i], U[cs + off + i], U[2 * cs + off + i]};
             int f = 0;
-            a0 = fmax(a0, wavespeed1d<T, SYS_EULER1D>(Uc, gm1, gamma, T(0), &f));
+            a0 = speed_max(a0, wavespeed1d<T, SYS_EULER1D>(Uc, gm1, gamma, T(0), &f));
             if (f) {
                 flag |= f;
                 first = min(first, i);
@@ -2950,14 +2959,14 @@ __global__ void __launch_bounds__(256) batch1d_alpha_kernel(const Batch1D p, dou
             T Uc[3] = {U[off + i], U[cs + off + i], U[2 * cs + off + i]};
             int f = 0;
             const T w = wavespeed1d<T, SYS_EULER1D>(Uc, gm1, gamma, T(0), &f);
-            if (!f) a = fmax(a, w);
+            if (!f) a = speed_max(a, w);
         }
         a = warp_max(a);
         if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = a;
         __syncthreads();
         if (threadIdx.x == 0) {
             T m = s_red[0];
-            for (int w = 1; w < 8; w++) m = fmax(m, s_red[w]);
+            for (int w = 1; w < 8; w++) m = speed_max(m, s_red[w]);
             alpha_out[tube] = (double)m;
         }
         __syncthreads();
@@ -3013,14 +3022,6 @@ cudaError_t launch_batch1d(const Batch1D &p, cudaStream_t st) {
 // and the barrier (0.5 us in a cluster, 1.3 over the grid).
 // ==========================================================================
 namespace t7 {
-
-// Maximum over a warp of non-negative values (not NaN), ordered like their bits.
-__device__ __forceinline__ double warp_max_pos(double v) {
-    const unsigned long long b = f64_bits(v);
-    const unsigned hi = (unsigned)(b >> 32), m = __reduce_max_sync(0xffffffffu, hi);
-    const unsigned l = __reduce_max_sync(0xffffffffu, hi == m ? (unsigned)b : 0u);
-    return f64_of((unsigned long long)m << 32 | l);
-}
 
 // A CTA's slot of the exchange `tag`, and the read of all slots by one warp: waits
 // (bounded) until every slot carries the tag and returns the maximum; false when

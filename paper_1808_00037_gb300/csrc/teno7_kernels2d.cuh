@@ -518,8 +518,8 @@ __global__ void __launch_bounds__(COLS * 16, 32 / COLS) ysweep2d_kernel(const St
         if (tid == 0) {
             T vx = s_red[0], vy = s_red[NW];
             for (int w = 1; w < NW; w++) {
-                vx = fmax(vx, s_red[w]);
-                vy = fmax(vy, s_red[NW + w]);
+                vx = speed_max(vx, s_red[w]);
+                vy = speed_max(vy, s_red[NW + w]);
             }
             const int so = (p.stage + 1) % 3;
             atomicMax(&ctl->amax[so][0], (unsigned long long)__double_as_longlong((double)vx));
@@ -550,8 +550,8 @@ __global__ void __launch_bounds__(256) alpha2d_kernel(const Alpha2D p) {
             flag |= f;
             first = min(first, (int)i);
         }
-        mx = fmax(mx, sx);
-        my = fmax(my, sy);
+        mx = speed_max(mx, sx);
+        my = speed_max(my, sy);
     }
     if (flag) latch_error(p.ctl, flag, first);
     mx = warp_max(mx);
@@ -564,8 +564,8 @@ __global__ void __launch_bounds__(256) alpha2d_kernel(const Alpha2D p) {
     if (threadIdx.x == 0) {
         T vx = s_red[0][0], vy = s_red[1][0];
         for (int w = 1; w < 8; w++) {
-            vx = fmax(vx, s_red[0][w]);
-            vy = fmax(vy, s_red[1][w]);
+            vx = speed_max(vx, s_red[0][w]);
+            vy = speed_max(vy, s_red[1][w]);
         }
         atomicMax(&p.ctl->acc[0], (unsigned long long)__double_as_longlong((double)vx));
         atomicMax(&p.ctl->acc[1], (unsigned long long)__double_as_longlong((double)vy));
