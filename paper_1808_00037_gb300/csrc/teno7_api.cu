@@ -84,7 +84,7 @@ t7_status cuda_fail(t7_ctx *c, cudaError_t e, const char *what) {
 
 int nvars(int sys) { return sys == T7_EULER1D ? 3 : (sys == T7_EULER2D ? 4 : 1); }
 
-// The control block, and after it the slots of the cooperative run kernels.
+// The control block, and after it the slots of the one-launch runs.
 constexpr size_t CTL_SLOTS = (sizeof(t7::DevCtl) + 255) / 256 * 256;
 constexpr size_t CTL_BYTES = CTL_SLOTS + 2 * t7::RUN_MAX_CTAS * sizeof(t7::RunSlot);
 

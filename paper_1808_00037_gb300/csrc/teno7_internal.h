@@ -207,9 +207,6 @@ cudaError_t launch_combine2_f64(void *out1, void *out2, const void *x, const voi
 cudaError_t launch_combine2_f32(void *out1, void *out2, const void *x, const void *y, double a1, double b1,
                                 double a2, double b2, size_t N, cudaStream_t s);
 
-// Finalization done by the last CTA of a launch (see DevCtl).
-enum { FIN_NONE = 0, FIN_ALPHA = 1, FIN_STEP = 2 };
-
 struct Recon {
     const void *v;  // n + 8 values
     void *fhat;     // n + 1

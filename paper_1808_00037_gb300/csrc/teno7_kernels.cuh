@@ -3,8 +3,11 @@
 // precision:
 //   teno7_f64.cu  compiled with -fmad=false: every FP64 expression below is
 //                 evaluated one IEEE operation at a time in the written order
-//                 (the same order in which the CPU oracle states the method),
-//                 so FP64 results and stencil masks are reproducible bit for bit;
+//                 (the same order in which the CPU oracle states the method; an
+//                 FMA is written where its product is exact), so FP64 results
+//                 and stencil masks are reproducible bit for bit.  Quotients,
+//                 roots, many products and the cutoff decision give the FP64
+//                 operation's bits from other pipes (teno7_f64math.cuh);
 //   teno7_f32.cu  FMA contraction on; the cutoff test uses an overflow-safe
 //                 rescaled form (g_k / g_max)^6 because gamma_k = (1 + r)^6
 //                 overflows FP32 near strong jumps.
@@ -15,7 +18,9 @@
 // reach are staged in warp-private shared memory (conserved variables, the
 // global Lax-Friedrichs split fluxes G+- = (F +- alpha U)/2 and, for the Euler
 // system, u, H and sqrt(rho) for the Roe average), so no CTA-wide barrier is
-// needed inside the loop; warps stride over tiles.  Each lane then
+// needed inside the loop; warps stride over tiles.  (Large FP64 Euler launches
+// stage the eight tiles of a CTA together and run one tile a warp; small ones put
+// one tile on a whole CTA, tiles1d_split.)  Each lane then
 //   1. builds its face's Roe frame (L, R) and projects the cells it needs into
 //      characteristic fields (q+ on cells j-3 .. j+3, q- on j-2 .. j+4);
 //   2. computes the three cutoff bits of both splits of every field (Eqs.
@@ -33,7 +38,8 @@
 // mixed precision form, the batch tubes and parted launches); stage1d_f32fp_kernel
 // pairs two faces of a 61-cell tile (lane l: faces c0-2+l and c0+30+l) and runs
 // the splits one after the other (whole-domain and slab launches of the FP32
-// state).  Both give the same bits.
+// state).  Both give the same bits.  Small problems run whole steps, or a right-hand
+// side with its alpha, in one launch of the same tiles (run1d_kernel).
 // Grids cover whole waves of each kernel's resident CTAs (stage_grid); the
 // loads of a tile take the boundary map only where a staged cell lies outside
 // the grid; every index formed for a global access passes through chk(),
@@ -172,19 +178,6 @@ __device__ __forceinline__ T poly7(const T *__restrict__ c, const T v0, const T 
     return s;
 }
 
-template <typename T>
-__device__ __forceinline__ T dv(T a, T b);
-template <>
-__device__ __forceinline__ double dv<double>(double a, double b) {
-    return a / b;
-}
-template <>
-__device__ __forceinline__ float dv<float>(float a, float b) {
-    return __fdividef(a, b);
-}
-
-__device__ __forceinline__ double sq_root(double x) { return sqrt(x); }
-__device__ __forceinline__ float sq_root(float x) { return sqrtf(x); }
 __device__ __forceinline__ double absval(double x) { return fabs(x); }
 __device__ __forceinline__ float absval(float x) { return fabsf(x); }
 
@@ -2597,7 +2590,7 @@ inline int resident_ctas(const void *kernel, int threads, size_t smem = 0) {
     return ctas;
 }
 
-// Warps per CTA of the 1D stage and adjoint kernels: WPB, or -- for the
+// Warps per CTA of the stage kernels: WPB, or -- for the
 // FP64-pipe-bound kernels (spread = true) -- halved while that would leave SMs
 // without a CTA, so small problems run one warp tile per SM instead of eight
 // tiles on a few SMs (GB300's FP64 rate per SM is low; FP32 stage kernels at
