@@ -228,6 +228,14 @@ bool run_coop(t7_ctx *c, t7::Run1D &q) {
         return false;
     }
     q.slots = reinterpret_cast<t7::RunSlot *>(reinterpret_cast<char *>(c->ctl) + CTL_SLOTS);
+    const unsigned tags = 3u * (unsigned)q.nsteps + 1u;
+    if (c->run_tag > 0xffffffffu - tags) {  // out of tags: begin again over cleared slots
+        if (cudaMemsetAsync(q.slots, 0, CTL_BYTES - CTL_SLOTS, c->stream) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        c->run_tag = 1;
+    }
     q.tag = c->run_tag;
     const cudaError_t e = c->g.prec == T7_MIXED ? t7::launch_run1d_mixed(q, c->stream)
                           : c->g.prec == T7_F64 ? t7::launch_run1d_f64(q, c->stream)
@@ -236,7 +244,7 @@ bool run_coop(t7_ctx *c, t7::Run1D &q) {
         cudaGetLastError();
         return false;
     }
-    c->run_tag += 3u * (unsigned)q.nsteps + 1u;
+    c->run_tag += tags;
     return true;
 }
 
