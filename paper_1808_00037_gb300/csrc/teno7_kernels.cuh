@@ -3157,6 +3157,9 @@ __global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 || FORM == FORM_CTA 
         tag++;
     };
     __syncthreads();
+    // before any CTA writes into another's shared memory, all of them have begun
+    if (q.cluster)
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
     if (march) {
         alpha = f64_of(ctl->amax[0][0]);
         t = ctl->t;
