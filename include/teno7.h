@@ -253,6 +253,8 @@ t7_status t7_rk3_step_adjoint_recorded(t7_ctx *ctx, const void *U_in, const void
  *                (with -8 there is nothing to split off);
  *                0: as -G with G chosen by t7_batch_autotune (8 if never
  *                tuned).  Any other value: T7_EINVAL.
+ *                With G = 8 (a whole CTA per tube) a batch of fewer tubes than
+ *                the GPU holds CTAs gives each tube a cluster of 2, 4 or 8.
  *                The results do not depend on this argument: every tube's
  *                arithmetic is the same for every group size.
  *   steps_out, t_out  host or NULL, per tube

@@ -1197,8 +1197,25 @@ static int batch_nbig(t7_ctx *c, int ntubes, int group) {
     return nbig;
 }
 
+// CTAs per tube (8 warps each) of a batch that would leave SMs idle at one: doubled while the
+// clusters of all tubes still fit on the chip half full, up to 8, and while the longest
+// tube has tiles for them (a warp each).  20 steps, 1 / 2 / 4 / 8 CTAs per tube, ms:
+// FP32 (256 to 8192 cells, 304 CTAs resident) 25 tubes 2.56 / 1.05 / 0.64 / 0.50, 70 2.95 /
+// 1.09 / 0.89 / 0.80, 150 3.02 / 1.62 / 1.18 / 1.52, 300 3.09 / 1.92 / 2.21 / 2.86, 700 3.86 /
+// 4.06 / 4.82 / 6.35; FP64 (256 to 2048, 152) 20 tubes 14.3 / 7.9 / 4.7 / 3.8, 60 14.8 /
+// 8.4 / 6.7 / 9.0, 110 14.6 / 8.6 / 10.7 / 15.8, 200 14.7 / 14.7 / 17.7 / 27.8.
+static int batch_cluster(t7_ctx *c, const int64_t *offsets, int ntubes) {
+    const int room = c->g.prec == T7_F64 ? t7::batch1d_groups_f64(8) : t7::batch1d_groups_f32(8);
+    int64_t longest = 0;
+    for (int t = 0; t < ntubes; t++) longest = std::max(longest, offsets[t + 1] - offsets[t]);
+    const int64_t tiles = (longest + 28) / 29;
+    int ctas = 1;
+    while (ctas < 8 && (int64_t)ntubes * ctas < room && 8 * ctas < tiles) ctas *= 2;
+    return ctas;
+}
+
 static cudaError_t batch_launch(t7_ctx *c, void *U, int ntubes, double t_end, double cfl, int max_steps,
-                                int group, bool whole_cta_phase) {
+                                int group, bool whole_cta_phase, int cluster) {
     cudaError_t e = cudaMemsetAsync(c->b_queue, 0, 2 * sizeof(int), c->stream);
     if (e != cudaSuccess) return e;
     t7::Batch1D p;
@@ -1219,6 +1236,7 @@ static cudaError_t batch_launch(t7_ctx *c, void *U, int ntubes, double t_end, do
     p.CT = c->g.CT;
     p.max_steps = max_steps;
     p.group_warps = group;
+    p.cluster = cluster;
     p.nbig = whole_cta_phase ? batch_nbig(c, ntubes, group) : 0;
     p.queue = c->b_queue;
     p.steps_out = c->b_steps;
@@ -1254,7 +1272,8 @@ t7_status t7_batch_run(t7_ctx *c, void *U, const int64_t *offsets, const double 
     if (group != 1 && group != 2 && group != 4 && group != 8)
         return fail(c, T7_EINVAL, "t7_batch_run: group_warps must be 0, +-1, +-2, +-4 or +-8");
     if ((st = batch_prepare(c, U, offsets, dx, ntubes, t_end, cfl, max_steps))) return st;
-    cudaError_t e = batch_launch(c, U, ntubes, t_end, cfl, max_steps, group, group_warps <= 0);
+    cudaError_t e = batch_launch(c, U, ntubes, t_end, cfl, max_steps, group, group_warps <= 0,
+                                 group == 8 ? batch_cluster(c, offsets, ntubes) : 1);
     if (e != cudaSuccess) return cuda_fail(c, e, "batch launch");
     if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return cuda_fail(c, e, "sync");
     if (steps_out && (e = cudaMemcpy(steps_out, c->b_steps, sizeof(int) * ntubes, cudaMemcpyDeviceToHost)) !=
@@ -1283,7 +1302,8 @@ t7_status t7_batch_autotune(t7_ctx *c, const void *U, const int64_t *offsets, co
         // every candidate advances the same copy of the state by trial_steps steps
         cudaError_t e = cudaMemcpyAsync(c->Uhost, U, bytes, cudaMemcpyDeviceToDevice, c->stream);
         if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
-        if (e == cudaSuccess) e = batch_launch(c, c->Uhost, ntubes, INFINITY, cfl, trial_steps, groups[gi], false);
+        if (e == cudaSuccess) e = batch_launch(c, c->Uhost, ntubes, INFINITY, cfl, trial_steps, groups[gi], false,
+                                              groups[gi] == 8 ? batch_cluster(c, offsets, ntubes) : 1);
         if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(e1);
         float ms = 0.f;

@@ -174,6 +174,7 @@ struct Batch1D {
     double t_end, cfl, gamma, CT;
     int max_steps;
     int group_warps;           // warps per tube (1, 2, 4 or 8)
+    int cluster;               // > 1: every tube on a cluster of that many CTAs (group_warps and nbig unused)
     int nbig;                  // the first nbig tubes of `order` run on whole CTAs (all 8 warps)
     int *queue;                // device work counters [2] (whole-CTA, then group tubes), zero before the launch
     int *steps_out;            // device, per tube

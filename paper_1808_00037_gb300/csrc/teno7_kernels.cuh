@@ -2779,6 +2779,34 @@ cudaError_t launch_recon(const Recon &p, cudaStream_t st) {
 
 }  // namespace t7
 
+namespace t7 {
+
+// Maximum over a thread-block cluster of the threads' non-negative v (not NaN), and
+// a barrier: global writes before it are visible to every CTA of the cluster after
+// it.  Every warp writes its maximum into each CTA's shared memory, and the
+// cluster's hardware barrier orders those and the global writes.  rank, ctas: this
+// CTA's and their number (<= RUN_CLUSTER); s_cl [2][RUN_CLUSTER * WPB], the two used
+// in turn (tag).
+constexpr int RUN_CLUSTER = 16;
+__device__ __forceinline__ double cluster_max(unsigned tag, double v, double (*s_cl)[RUN_CLUSTER * WPB], int rank,
+                                              int ctas) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, n = ctas * nw;
+    v = warp_max_pos(v);
+    double *set = s_cl[tag & 1u];
+    const unsigned mine = (unsigned)__cvta_generic_to_shared(&set[rank * nw + warp]);
+    if (lane < ctas) {
+        unsigned remote;
+        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(mine), "r"(lane));
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote), "d"(v) : "memory");
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    double m = 0.0;
+    for (int i = lane; i < n; i += 32) m = f64_max_pos(m, set[i]);
+    return warp_max_pos(m);
+}
+
+}  // namespace t7
+
 // ==========================================================================
 // Persistent ragged-batch kernel (1D Euler).  The CTA's warps form groups of
 // G = p.group_warps warps; each group's leader takes the next tube from an
@@ -2786,7 +2814,8 @@ cudaError_t launch_recon(const Recon &p, cudaStream_t st) {
 // tube's whole SSP-RK3 loop to t_end: alpha of U^n and the CFL step (the
 // oracle's expressions), then three stages, each a warp-tile sweep over the
 // tube followed by a group reduction of the new state's max(|u| + c), which is
-// the next stage's alpha.  Group barriers are named barriers (id = group + 1).
+// the next stage's alpha.  Group barriers are named barriers (id = group + 1); in
+// the cluster form the group is a cluster of CTAs and its barrier the cluster's.
 // Tubes are independent, so groups never wait on each other.
 // ==========================================================================
 namespace t7 {
@@ -2799,7 +2828,10 @@ __device__ __forceinline__ void group_sync(int group, int G) {
     }
 }
 
-template <typename T>
+// CLUSTER: a batch of fewer tubes than CTAs fit (batch_cluster).  A cluster of CTAs
+// takes the place of a group: the longest tube's stages set the time, and one CTA
+// takes 36 rounds of tiles for 8192 cells (25 tubes, 20 steps: 2.56 -> 0.50 ms).
+template <typename T, bool CLUSTER = false>
 __global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 ? 2 : 1)) batch1d_kernel(const Batch1D p) {
     __shared__ T s_U[WPB][3][WC];
     __shared__ T s_gp[WPB][3][WC];
@@ -2825,9 +2857,18 @@ __global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 ? 2 : 1)) batch1d_ke
     // the whole CTA as one group, so that no single tube outlasts the rest of
     // the batch on a small group.
     int G = WPB, group = 0, wg = warp;
+    __shared__ double s_cl[CLUSTER ? 2 : 1][CLUSTER ? RUN_CLUSTER * WPB : 1];
+    unsigned rank = 0, ctas = 1, tag = 0;
+    if constexpr (CLUSTER) {
+        asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+        asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(ctas));
+        G = WPB * ctas;
+        wg = rank * WPB + warp;
+    }
 
     // group max over its G warps; every lane of the group gets the result
     auto group_max = [&](T v) -> T {
+        if constexpr (CLUSTER) return (T)cluster_max(tag++, (double)v, s_cl, rank, ctas);
         v = warp_max(v);
         if (lane == 0) s_red[warp] = v;
         group_sync(group, G);
@@ -2912,26 +2953,50 @@ __global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 ? 2 : 1)) batch1d_ke
         }
     };
 
-    // phase 1: whole-CTA groups over order[0 .. nbig)
-    for (;;) {
-        if (warp == 0 && lane == 0) s_tube[0] = atomicAdd(p.queue + 1, 1);
-        __syncthreads();
-        const int q = s_tube[0];
-        __syncthreads();
-        if (q >= p.nbig) break;
-        run_tube(p.order[q]);
-    }
-    // phase 2: groups of p.group_warps warps over order[nbig .. ntubes)
-    G = p.group_warps;
-    group = warp / G;
-    wg = warp % G;
-    for (;;) {
-        if (wg == 0 && lane == 0) s_tube[group] = p.nbig + atomicAdd(p.queue, 1);
-        group_sync(group, G);
-        const int q = s_tube[group];
-        group_sync(group, G);
-        if (q >= p.ntubes) break;
-        run_tube(p.order[q]);
+    if constexpr (CLUSTER) {
+        // (all CTAs have begun before any writes into another's shared memory)
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+        // the first CTA takes a tube for its cluster (every tube's exchanges lie
+        // between a read of s_tube and its next write; after the last barrier no
+        // CTA touches another's shared memory)
+        for (;;) {
+            if (rank == 0 && threadIdx.x == 0) {
+                const int q = atomicAdd(p.queue, 1);
+                const unsigned mine = (unsigned)__cvta_generic_to_shared(&s_tube[0]);
+                for (unsigned r = 0; r < ctas; r++) {
+                    unsigned remote;
+                    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(mine), "r"(r));
+                    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(remote), "r"(q) : "memory");
+                }
+            }
+            __syncwarp();
+            asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+            const int q = s_tube[0];
+            if (q >= p.ntubes) return;
+            run_tube(p.order[q]);
+        }
+    } else {
+        // phase 1: whole-CTA groups over order[0 .. nbig)
+        for (;;) {
+            if (warp == 0 && lane == 0) s_tube[0] = atomicAdd(p.queue + 1, 1);
+            __syncthreads();
+            const int q = s_tube[0];
+            __syncthreads();
+            if (q >= p.nbig) break;
+            run_tube(p.order[q]);
+        }
+        // phase 2: groups of p.group_warps warps over order[nbig .. ntubes)
+        G = p.group_warps;
+        group = warp / G;
+        wg = warp % G;
+        for (;;) {
+            if (wg == 0 && lane == 0) s_tube[group] = p.nbig + atomicAdd(p.queue, 1);
+            group_sync(group, G);
+            const int q = s_tube[group];
+            group_sync(group, G);
+            if (q >= p.ntubes) break;
+            run_tube(p.order[q]);
+        }
     }
 }
 
@@ -2994,6 +3059,24 @@ cudaError_t launch_batch1d(const Batch1D &p, cudaStream_t st) {
     if (p.group_warps != 1 && p.group_warps != 2 && p.group_warps != 4 && p.group_warps != 8)
         return cudaErrorInvalidValue;
     if (p.nbig < 0 || p.nbig > p.ntubes) return cudaErrorInvalidValue;
+    if (p.cluster > 1) {
+        const void *k = reinterpret_cast<const void *>(&batch1d_kernel<T, true>);
+        Batch1D q = with_kt(p);
+        const int room = num_sms() * batch1d_per_sm<T>() / p.cluster;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = p.cluster;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((p.ntubes < room ? p.ntubes : room) * p.cluster);
+        cfg.blockDim = dim3(WPB * 32);
+        cfg.stream = st;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        void *args[] = {&q};
+        if (cudaLaunchKernelExC(&cfg, k, args) == cudaSuccess) return cudaSuccess;
+        cudaGetLastError();  // no room for such a cluster: one CTA per tube
+    }
     batch1d_kernel<T><<<num_sms() * batch1d_per_sm<T>(), WPB * 32, 0, st>>>(with_kt(p));
     return cudaGetLastError();
 }
@@ -3073,26 +3156,6 @@ __device__ __forceinline__ bool grid_max(RunSlot *slots, unsigned tag, double v,
     return true;
 }
 
-// The same over a grid that is one thread-block cluster: every warp writes its
-// maximum into each CTA's shared memory, and the cluster's hardware barrier
-// orders those and the global writes.  s_cl [2][RUN_CLUSTER * WPB].
-constexpr int RUN_CLUSTER = 16;
-__device__ __forceinline__ double cluster_max(unsigned tag, double v, double (*s_cl)[RUN_CLUSTER * WPB]) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, n = gridDim.x * nw;
-    v = warp_max_pos(v);
-    double *set = s_cl[tag & 1u];
-    const unsigned mine = (unsigned)__cvta_generic_to_shared(&set[blockIdx.x * nw + warp]);
-    if (lane < (int)gridDim.x) {
-        unsigned remote;
-        asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(mine), "r"(lane));
-        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote), "d"(v) : "memory");
-    }
-    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-    double m = 0.0;
-    for (int i = lane; i < n; i += 32) m = f64_max_pos(m, set[i]);
-    return warp_max_pos(m);
-}
-
 // What a launch's tiles are: a warp's 29 cells; a CTA's (FP64 Euler); a warp's
 // 61 cells with paired faces (FP32 state).
 enum { FORM_WARP = 0, FORM_CTA = 1, FORM_PAIR = 2 };
@@ -3151,7 +3214,7 @@ __global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 || FORM == FORM_CTA 
     bool ok = true, active = true;
     auto exchange = [&](double v) {
         if (q.cluster)
-            alpha = cluster_max(tag, v, s_cl);
+            alpha = cluster_max(tag, v, s_cl, blockIdx.x, gridDim.x);
         else
             ok = grid_max(q.slots, tag, v, alpha, s_red);
         tag++;
