@@ -50,7 +50,9 @@ __device__ __forceinline__ float fmaT(float a, float b, float c) { return __fmaf
 // frame in reverse instead of as dual numbers took a launch at 4096 cells from 69
 // to 15 us.  A tile is 32 faces and the AT = 25 cells that all eight of their
 // faces belong to, among the n + 8 cells with their ghosts; a ghost cell's share
-// goes to the cell it stands for, atomically, as do the cells near the ends.
+// goes to the cell it stands for, atomically, as do the cells near the ends.  The RK
+// step's vector sums ride along (e1, e2, aux): four launches a recorded step instead of
+// six, the gradient of 100 steps at 4096 cells FP32 6.77 -> 6.49 ms, FP64 13.25 -> 13.06.
 constexpr int AT = 25, AWPB = 4;  // cells per tile, warps per CTA
 
 template <typename T>
@@ -250,6 +252,18 @@ __global__ void __launch_bounds__(AWPB * 32, 2) rhs_adjoint1d_kernel(const Adjoi
             o[1] = fmaT(ir, fmaT(-gm1 * u, lHs, lus), o[1]);
             o[2] = fmaT(ir, gam * lHs, o[2]);
             const int cell = chk(p.ctl, ghost_map(l, n, p.bc_lo, p.bc_hi), 0, n);
+            if (l >= 0 && l < n) {  // the cell itself, not a ghost of it
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    const size_t i = (size_t)c * n + cell;
+                    if (p.e1) o[c] = fmaT(T(p.c1), static_cast<const T *>(p.e1)[i], o[c]);
+                    if (p.e2) o[c] = fmaT(T(p.c2), static_cast<const T *>(p.e2)[i], o[c]);
+                    if (p.aux) {
+                        T *x = static_cast<T *>(p.aux) + i;
+                        *x = p.aux_c != 0.0 ? T(p.aux_c) * *x : T(0);
+                    }
+                }
+            }
 #pragma unroll
             for (int c = 0; c < 3; c++) {
                 T *dst = &out[(size_t)c * n + cell];
@@ -268,28 +282,6 @@ __global__ void combine_kernel(T *out, const T *x, const T *y, const T *z, T c1,
         const T a = x ? c1 * x[i] : T(0);
         out[i] = a + c2 * (y[i] + c3 * z[i]);
     }
-}
-
-// out1 = a1 x + b1 y; out2 = a2 x + b2 y (if out2); x may be null.  out1 may
-// alias x or y (each element is read before it is written).
-template <typename T>
-__global__ void combine2_kernel(T *out1, T *out2, const T *x, const T *y, T a1, T b1, T a2, T b2, size_t N) {
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (size_t)gridDim.x * blockDim.x) {
-        const T xv = x ? x[i] : T(0), yv = y[i];
-        out1[i] = a1 * xv + b1 * yv;
-        if (out2) out2[i] = a2 * xv + b2 * yv;
-    }
-}
-
-template <typename T>
-cudaError_t launch_combine2(void *out1, void *out2, const void *x, const void *y, double a1, double b1, double a2,
-                            double b2, size_t N, cudaStream_t st) {
-    int grid = (int)((N + 255) / 256);
-    if (grid > num_sms() * 8) grid = num_sms() * 8;
-    combine2_kernel<T><<<grid, 256, 0, st>>>(static_cast<T *>(out1), static_cast<T *>(out2),
-                                             static_cast<const T *>(x), static_cast<const T *>(y), T(a1), T(b1),
-                                             T(a2), T(b2), N);
-    return cudaGetLastError();
 }
 
 template <typename T>

@@ -16,6 +16,10 @@ struct Adjoint1D {
     DevCtl *ctl;
     int slot_in;               // alpha of U (frozen) ...
     const double *alpha_ptr;   // ... or, if not null, read from here
-    double scale;              // out += scale (dL/dU)^T v
+    double scale;              // out += scale (dL/dU)^T v + c1 e1 + c2 e2
+    const void *e1, *e2;       // nullable, [3][n], not out
+    double c1, c2;
+    void *aux;                 // nullable, [3][n], none of the others: aux = aux_c aux (0: cleared)
+    double aux_c;
 };
 }  // namespace t7

@@ -905,11 +905,10 @@ static cudaError_t adj_apply(t7_ctx *c, const void *U, int slot, const uint8_t *
     return c->g.prec == T7_F64 ? t7::launch_rhs_adjoint1d_f64(a, c->stream) : t7::launch_rhs_adjoint1d_f32(a, c->stream);
 }
 
-// out += scale (dL/dU)^T v at U with recorded alpha and masks (no zeroing)
-static cudaError_t adj_accumulate(t7_ctx *c, const void *U, const double *alpha, const uint8_t *masks, const void *v,
-                                  void *out, double scale) {
-    t7::Adjoint1D a;
-    memset(&a, 0, sizeof(a));
+// out += scale (dL/dU)^T v + c1 e1 + c2 e2 at U with recorded alpha and masks, and
+// aux = aux_c aux (e1, e2, c1, c2, aux, aux_c from `a`)
+static cudaError_t adj_accumulate(t7_ctx *c, t7::Adjoint1D a, const void *U, const double *alpha,
+                                  const uint8_t *masks, const void *v, void *out, double scale) {
     a.U = U;
     a.v = v;
     a.out = out;
@@ -923,13 +922,6 @@ static cudaError_t adj_accumulate(t7_ctx *c, const void *U, const double *alpha,
     a.alpha_ptr = alpha;
     a.scale = scale;
     return c->g.prec == T7_F64 ? t7::launch_rhs_adjoint1d_f64(a, c->stream) : t7::launch_rhs_adjoint1d_f32(a, c->stream);
-}
-
-static cudaError_t combine2(t7_ctx *c, void *out1, void *out2, const void *x, const void *y, double a1, double b1,
-                            double a2, double b2) {
-    const size_t N = c->ncell * c->m;
-    return c->g.prec == T7_F64 ? t7::launch_combine2_f64(out1, out2, x, y, a1, b1, a2, b2, N, c->stream)
-                               : t7::launch_combine2_f32(out1, out2, x, y, a1, b1, a2, b2, N, c->stream);
 }
 
 // Layout of one tape entry: U1, U2 (state-sized), the forward Delta codes of
@@ -1090,16 +1082,27 @@ t7_status t7_rk3_step_adjoint_recorded(t7_ctx *c, const void *U_in, const void *
     const void *Us[3] = {U_in, t + L.u1, t + L.u2};
     const uint8_t *mk[3];
     for (int k = 0; k < 3; k++) mk[k] = t + L.masks[k];
-    void *A = c->adj[0], *W = c->adj[1], *T = c->adj[2];
-    // U3 = U/3 + 2/3 (U2 + dt L(U2)):  W = 2/3 lam + 2/3 dt L2^T lam,  A = lam/3
-    cudaError_t e = combine2(c, W, A, nullptr, lambda, 0.0, 2.0 / 3.0, 0.0, 1.0 / 3.0);
-    if (e == cudaSuccess) e = adj_accumulate(c, Us[2], alpha + 2, mk[2], lambda, W, (2.0 / 3.0) * dt);
-    // U2 = 3/4 U + 1/4 (U1 + dt L(U1)):  A += 3/4 W,  T = W/4 + dt/4 L1^T W
-    if (e == cudaSuccess) e = combine2(c, A, T, A, W, 1.0, 0.75, 0.0, 0.25);
-    if (e == cudaSuccess) e = adj_accumulate(c, Us[1], alpha + 1, mk[1], W, T, 0.25 * dt);
-    // U1 = U + dt L(U):  lam = A + T + dt L0^T T
-    if (e == cudaSuccess) e = combine2(c, lambda, nullptr, A, T, 1.0, 1.0, 0.0, 0.0);
-    if (e == cudaSuccess) e = adj_accumulate(c, Us[0], alpha, mk[0], T, lambda, dt);
+    void *W = c->adj[0], *T = c->adj[1];
+    t7::Adjoint1D a[3];
+    memset(a, 0, sizeof(a));
+    cudaError_t e = cudaMemsetAsync(W, 0, c->ncell * c->m * c->esize, c->stream);
+    // U3 = U/3 + 2/3 (U2 + dt L(U2)):  W = 2/3 lam + 2/3 dt L2^T lam  (T = 0)
+    a[2].e1 = lambda;
+    a[2].c1 = 2.0 / 3.0;
+    a[2].aux = T;
+    if (e == cudaSuccess) e = adj_accumulate(c, a[2], Us[2], alpha + 2, mk[2], lambda, W, (2.0 / 3.0) * dt);
+    // U2 = 3/4 U + 1/4 (U1 + dt L(U1)):  T = W/4 + dt/4 L1^T W  (lam = lam/3)
+    a[1].e1 = W;
+    a[1].c1 = 0.25;
+    a[1].aux = lambda;
+    a[1].aux_c = 1.0 / 3.0;
+    if (e == cudaSuccess) e = adj_accumulate(c, a[1], Us[1], alpha + 1, mk[1], W, T, 0.25 * dt);
+    // U1 = U + dt L(U):  lam = lam/3 + 3/4 W + T + dt L0^T T
+    a[0].e1 = T;
+    a[0].c1 = 1.0;
+    a[0].e2 = W;
+    a[0].c2 = 0.75;
+    if (e == cudaSuccess) e = adj_accumulate(c, a[0], Us[0], alpha, mk[0], T, lambda, dt);
     if (e != cudaSuccess) return cuda_fail(c, e, "adjoint of a recorded step");
     return T7_OK;
 }

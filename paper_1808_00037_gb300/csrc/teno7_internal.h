@@ -203,10 +203,6 @@ cudaError_t launch_combine_f64(void *out, const void *x, const void *y, const vo
 cudaError_t launch_combine_f32(void *out, const void *x, const void *y, const void *z, double c1, double c2,
                                double c3, size_t N, cudaStream_t s);
 // out1 = a1 x + b1 y; out2 (nullable) = a2 x + b2 y; x may be null
-cudaError_t launch_combine2_f64(void *out1, void *out2, const void *x, const void *y, double a1, double b1,
-                                double a2, double b2, size_t N, cudaStream_t s);
-cudaError_t launch_combine2_f32(void *out1, void *out2, const void *x, const void *y, double a1, double b1,
-                                double a2, double b2, size_t N, cudaStream_t s);
 
 struct Recon {
     const void *v;  // n + 8 values
