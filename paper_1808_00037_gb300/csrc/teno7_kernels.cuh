@@ -2922,10 +2922,13 @@ __global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 ? 2 : 1)) batch1d_ke
         T *ins[3] = {U + off, W1 + off, W2 + off};
         T *outs[3] = {W1 + off, W2 + off, U + off};
 
+        const double cfl_dx = p.cfl * dx;
         double t = 0.0;
         int steps = 0;
         while (steps < p.max_steps && t < p.t_end) {
-            double dt = (p.cfl * dx) / (double)alpha;
+            // (FP32: 21.01 -> 20.82 ms for 20 steps of 4096 tubes with the FP64 division's
+            // 142 cycles a warp off the SM's pipe)
+            double dt = div64(cfl_dx, (double)alpha);
             if (t + dt > p.t_end) dt = p.t_end - t;
             A.dtT = T(dt);
 // (FP32: each stage its own code, 23.7 -> 21.0 ms for 20 steps of 4096 tubes;
