@@ -52,11 +52,13 @@ FP64_NOMINAL_TFLOPS = 1.25
 #   FP64: 30 per-cell staging + 718 per face + 28 update = 776 (no FMA)
 FLOPS_PER_CELL_STAGE = {"f32": 808.0, "f64": 776.0}
 # Executed floating-point operations per cell per stage launch, from ncu's
-# per-opcode thread counters of one launch on the same workload (FMA = 2,
+# per-opcode thread counters of launches on the same workload (FMA = 2,
 # packed f32x2 FMA = 4, packed add/mul = 2, scalar add/mul = 1; the keep-all
-# shortcut skips most of the cutoff, so this is below the algorithmic count);
+# shortcut skips most of the cutoff, so this is below the algorithmic count; f64:
+# operations of the FP64 pipe only, products, quotients and roots being formed on
+# the integer and FP32 pipes), mean of the three stages on 2M (f64: 1M) cells of it;
 # None when not captured for the current kernel.
-EXEC_FLOPS_PER_CELL_STAGE = {"f32": 584.4, "f64": 812.0}
+EXEC_FLOPS_PER_CELL_STAGE = {"f32": 588.1, "f64": 231.9}
 # DRAM bytes per stage launch per cell measured by ncu (dram__bytes_read.sum +
 # dram__bytes_write.sum, averaged over the three stage launches of one RK3
 # step at N = 16,777,600) for the current kernels; None when not captured.

@@ -3096,8 +3096,8 @@ cudaError_t launch_batch1d(const Batch1D &p, cudaStream_t st) {
 // values), and meet once per stage in grid_max or, where the grid is one cluster,
 // cluster_max, which is both the barrier between stages and the reduction of
 // alpha.  us per step, single launches in a graph -> here: Shu-Osher at 1600
-// cells FP32 19.8 -> 8.8 (12.1 without the cluster), FP64 71 -> 33; advection at
-// 200 cells FP64 19.7 -> 10.2.  Bound by the chain of one tile (some 2 us in FP32)
+// cells FP32 19.8 -> 8.5 (12.1 without the cluster), FP64 71 -> 29.5; advection at
+// 200 cells FP64 19.7 -> 9.1.  Bound by the chain of one tile (some 2 us in FP32)
 // and the barrier (0.5 us in a cluster, 1.3 over the grid).
 // ==========================================================================
 namespace t7 {
