@@ -254,7 +254,7 @@ cudaError_t alpha_for_stage(t7_ctx *c, const void *U) {
     return c->g.sys == T7_SCALAR_ADVECTION ? cudaSuccess : alpha_launch(c, U);
 }
 
-// The last stage of a step (1D) in OUT_PARTS launches over consecutive
+// The last stage of a step (1D) in up to OUT_PARTS launches over consecutive
 // ranges of warp tiles; each finished range of cells is copied from U to the
 // host array host_out ([m][nx], pageable or page-locked) on the copy stream
 // while the next range computes, so the result leaves the device at the
