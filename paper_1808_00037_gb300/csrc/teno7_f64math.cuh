@@ -68,18 +68,20 @@ T7_HD int f32_to_int(float x) {  // nearest integer, |x| < 2^31
     return (int)lrintf(x);
 #endif
 }
-// Approximate reciprocal, within 2 ulp.  (T7_HOST_ERR: a host check may scale the
+// Approximate reciprocal, within 2 ulp; subnormal arguments and results (those of
+// arguments above 2^126) count as zero.  (T7_HOST_ERR: a host check may scale the
 // approximations by their error bound.)
 #ifndef T7_HOST_ERR
 #define T7_HOST_ERR
 #endif
+T7_HD float f32_flush(float x) { return fabsf(x) < 1.17549435e-38f ? copysignf(0.f, x) : x; }
 T7_HD float f32_rcp(float x) {
 #ifdef __CUDA_ARCH__
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 #else
-    return (1.0f / x) T7_HOST_ERR;
+    return f32_flush((1.0f / f32_flush(x)) T7_HOST_ERR);
 #endif
 }
 
@@ -89,7 +91,7 @@ T7_HD float f32_rsqrt(float x) {  // approximate 1/sqrt, within 2^-22
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 #else
-    return (float)(1.0 / sqrt((double)x)) T7_HOST_ERR;
+    return (float)(1.0 / sqrt((double)f32_flush(x))) T7_HOST_ERR;
 #endif
 }
 
@@ -323,10 +325,11 @@ T7_HD void split_f32(double x, float &h, float &l) {
 // within 2.2e-6 of itself plus A = 2^-60 max|w|^2 (1e-36 covers underflow).
 //   kept     tau + 1e-5 (beta_0 + beta_2) + A < kt (0.9999 (beta_min + eps) - A)
 //            implies tau < kt (beta_min + eps): all bits set (keep_all_factor).
-//   decided  where tau > 0.003 (beta_0 + beta_2) and A is below 1e-5 of the
-//            smallest beta + eps, g_k is known within 7.5e-4 and chi_k / C_T
-//            within 2%: the FP32 comparison holds unless chi_k is within 3% of
-//            C_T.
+//   decided  where tau > 0.003 (beta_0 + beta_2), A is below 1e-5 of the
+//            smallest beta + eps, and the largest beta + eps below 2^125 (above
+//            2^126 its reciprocal would vanish), g_k is known within 7.5e-4 and
+//            chi_k / C_T within 2%: the FP32 comparison holds unless chi_k is
+//            within 3% of C_T.
 // Everything else, and what FP32 cannot hold, goes to the FP64 evaluation.
 T7_HD unsigned cutoff_bits(double w0, double w1, double w2, double w3, double w4, const Cut64 &K) {
     float h0, h1, h2, h3, h4, l0, l1, l2, l3, l4;
@@ -346,7 +349,7 @@ T7_HD unsigned cutoff_bits(double w0, double w1, double w2, double w3, double w4
     const float A = fmaf(W * W, 8.673617379884035e-19f, 1e-36f);
     const float sum = b0 + b2, tau = fabsf(b0 - b2), bm = fminf(fminf(b0, b1), b2) + K.e4;
     if (fmaf(1e-5f, sum, tau) + A < K.ktf * fmaf(0.9999f, bm, -A)) return 7u;
-    if (K.ctf > 0.f && tau > 0.003f * sum && A < 1e-5f * bm) {
+    if (K.ctf > 0.f && tau > 0.003f * sum && A < 1e-5f * bm && fmaxf(fmaxf(b0, b1), b2) + K.e4 < 4e37f) {
         const float g0 = fmaf(tau, f32_rcp(b0 + K.e4), 1.f), g1 = fmaf(tau, f32_rcp(b1 + K.e4), 1.f);
         const float g2 = fmaf(tau, f32_rcp(b2 + K.e4), 1.f);
         const float gm = fmaxf(fmaxf(g0, g1), g2), rg = f32_rcp(gm);
