@@ -41,6 +41,12 @@
  *     array, and the next synchronising call returns T7_EINDEX (before any
  *     other status) with the lowest failing index in t7_last_error().  The
  *     release build never returns T7_EINDEX.
+ *   - t7_run, t7_run_host, t7_rk3_step, t7_rk3_step_record and t7_euler_rhs of a
+ *     small 1D problem may be one launch whose blocks wait for one another
+ *     between stages.  Every wait is bounded (a second or two); one that ran out
+ *     is latched, and that call, or for an asynchronous one the next
+ *     synchronising call, returns T7_ETIMEOUT.  The output is then incomplete
+ *     (the state of a run or step partly advanced); the context stays usable.
  *   - A call never aborts the process; it returns a t7_status and, on
  *     failure, t7_last_error() describes the cause.
  */

@@ -1,7 +1,8 @@
 /*
  * teno7_probe.h -- measured arithmetic peaks of the current CUDA device, the
  * denominators of the ALU roofline that the TENO7-ext stage kernels are
- * reported against; and a self-test of the checked build's index check.  The paper has no counterpart: it reports no
+ * reported against; a self-test of the checked build's index check; and a switch
+ * for tests of the one-launch runs' waits.  The paper has no counterpart: it reports no
  * performance figures.  Part of libteno7 (links against teno7.h's status
  * codes).
  */
@@ -42,6 +43,20 @@ t7_status t7_probe_fma(int kind, int iters, int repeats, void *stream, double *t
  * T7_EINVAL for a null pointer or lo >= hi, T7_ENOMEM / T7_ECUDA if a CUDA
  * call fails. */
 t7_status t7_probe_index_check(int i, int lo, int hi, int *index_out, int *flagged_out, int *checked_build_out);
+
+/* Makes the waits of this context's next one-launch run, step or right-hand side
+ * (teno7.h: T7_ETIMEOUT) run out (checked build only: the release build's kernels
+ * carry no such switch, which cost its small runs 0.5 to 1%), or sets its
+ * exchange tags, so that tests reach these paths (no counterpart in the paper).  One-launch forms whose blocks
+ * do not wait for one another (a single block or cluster) are not affected.
+ *   block  the block that gives up at its first wait; -1: none
+ *   polls  after which the other blocks give up, 1 .. 2^21 (the default)
+ *   tag    next exchange tag, not below the context's present one (exchanges of
+ *          later calls count on from it and restart from 1 after 2^32 - 1); 0:
+ *          unchanged
+ * block and polls hold for one launch; the release build takes -1 and 2^21 only.
+ * T7_EINVAL for a bad argument. */
+t7_status t7_probe_run_waits(t7_ctx *ctx, int block, int polls, unsigned tag);
 
 #ifdef __cplusplus
 }

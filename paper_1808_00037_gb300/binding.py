@@ -82,6 +82,7 @@ def load(path: Path | str | None = None) -> ctypes.CDLL:
         "t7_batch_autotune": ([vp, vp, vp, vp, i, d, i, ctypes.POINTER(i), vp], i),
         "t7_probe_fma": ([i, i, i, vp, ctypes.POINTER(d), ctypes.POINTER(ctypes.c_float)], i),
         "t7_probe_index_check": ([i, i, i, ctypes.POINTER(i), ctypes.POINTER(i), ctypes.POINTER(i)], i),
+        "t7_probe_run_waits": ([vp, i, i, ctypes.c_uint], i),
         "t7_slab_alpha": ([vp, vp, vp], i),
         "t7_slab_rhs": ([vp, vp, vp, vp, u8p], i),
         "t7_slab_stage": ([vp, i, vp, vp, vp, vp, d, vp], i),
@@ -342,6 +343,10 @@ class Context:
                                                off.size - 1, cfl, trial_steps, ctypes.byref(g), ms.ctypes.data),
                     "t7_batch_autotune")
         return g.value, ms
+
+    def probe_run_waits(self, block: int = -1, polls: int = 1 << 21, tag: int = 0):
+        """Make the next one-launch call's waits run out (see t7_probe_run_waits)."""
+        self._check(self.lib.t7_probe_run_waits(self.h, block, polls, tag), "t7_probe_run_waits")
 
     def sync(self):
         self._check(self.lib.t7_sync(self.h), "t7_sync")

@@ -17,6 +17,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "teno7.h"
+#include "teno7_probe.h"
 #include "teno7_internal.h"
 #include "teno7_adjoint_params.h"
 
@@ -49,6 +50,9 @@ struct t7_ctx {
     cudaGraphExec_t gexec;
     void *g_U;
     unsigned run_tag;      // next stage tag of the cooperative run kernels
+#if T7_CHECKED
+    int probe_block, probe_limit;  // t7_probe_run_waits: the next one's give_up and spin_limit
+#endif
     // t7_run_host with a known step count: the last stage is launched in parts
     // and each finished part is copied to the host array on cstream
     cudaStream_t cstream;
@@ -237,6 +241,10 @@ bool run_coop(t7_ctx *c, t7::Run1D &q) {
         c->run_tag = 1;
     }
     q.tag = c->run_tag;
+#if T7_CHECKED
+    q.give_up = c->probe_block;
+    q.spin_limit = c->probe_limit;
+#endif
     const cudaError_t e = c->g.prec == T7_MIXED ? t7::launch_run1d_mixed(q, c->stream)
                           : c->g.prec == T7_F64 ? t7::launch_run1d_f64(q, c->stream)
                                                 : t7::launch_run1d_f32(q, c->stream);
@@ -245,6 +253,10 @@ bool run_coop(t7_ctx *c, t7::Run1D &q) {
         return false;
     }
     c->run_tag += tags;
+#if T7_CHECKED
+    c->probe_block = -1;
+    c->probe_limit = t7::RUN_SPIN_LIMIT;
+#endif
     return true;
 }
 
@@ -402,6 +414,10 @@ t7_status t7_create(const t7_grid *g, void *stream, t7_ctx **out) {
     c->ncell = (size_t)g->nx * g->ny;
     c->stream = (cudaStream_t)stream;
     c->run_tag = 1;  // the slots start at zero
+#if T7_CHECKED
+    c->probe_block = -1;
+    c->probe_limit = t7::RUN_SPIN_LIMIT;
+#endif
     cudaGetDevice(&c->device);
     size_t bytes = c->ncell * c->m * c->esize;
     if (cudaMalloc(&c->U1, bytes) != cudaSuccess || cudaMalloc(&c->U2, bytes) != cudaSuccess ||
@@ -866,6 +882,21 @@ t7_status t7_run_host(t7_ctx *c, void *U_host, double cfl, double t_end, int max
     if (e != cudaSuccess) return cuda_fail(c, e, "D2H copy");
     if ((e = cudaStreamSynchronize(c->stream)) != cudaSuccess) return cuda_fail(c, e, "sync");
     return st;
+}
+
+t7_status t7_probe_run_waits(t7_ctx *c, int block, int polls, unsigned tag) {
+    if (!c) return T7_EINVAL;
+    if (block < -1 || polls < 1 || polls > t7::RUN_SPIN_LIMIT || (tag != 0 && tag < c->run_tag))
+        return fail(c, T7_EINVAL, "t7_probe_run_waits: bad argument");
+#if T7_CHECKED
+    c->probe_block = block;
+    c->probe_limit = polls;
+#else
+    if (block != -1 || polls != t7::RUN_SPIN_LIMIT)
+        return fail(c, T7_EINVAL, "t7_probe_run_waits: only the checked build's waits can be made to run out");
+#endif
+    if (tag != 0) c->run_tag = tag;
+    return T7_OK;
 }
 
 // -------------------------------------------------------------- adjoint ----

@@ -4,6 +4,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#ifndef T7_CHECKED
+#define T7_CHECKED 0  // 1: the checked build (teno7.h)
+#endif
+
 namespace t7 {
 
 enum { SYS_ADV = 0, SYS_EULER1D = 1, SYS_EULER2D = 2, SYS_BURGERS = 3 };
@@ -71,6 +75,7 @@ struct Stage1D {
 // problems).  Each CTA publishes its maximum of every stage's output in its own
 // slot, tagged with the stage's number, and waits for the others' (grid_max).
 constexpr int RUN_MAX_CTAS = 512;
+constexpr int RUN_SPIN_LIMIT = 1 << 21;  // polls of a block's wait, a second or two
 struct RunSlot {
     unsigned long long w[2];  // tag << 32 | high, low half of the maximum's bits
 };
@@ -88,6 +93,10 @@ struct Run1D {
     RunSlot *slots;  // [2][RUN_MAX_CTAS]
     unsigned tag;    // tag of the launch's first exchange; 3 nsteps + 1 tags are used at most
     int cluster;     // the grid is one thread-block cluster (set by the launcher)
+#if T7_CHECKED
+    int spin_limit;  // polls after which a block gives up waiting for another's slot
+    int give_up;     // block that gives up at its first wait, or -1
+#endif
 };
 
 // Ghost cells per side of a slab (the stencil reach of the scheme, Eq. app:

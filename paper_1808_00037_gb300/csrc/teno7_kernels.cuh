@@ -205,9 +205,6 @@ __device__ __forceinline__ void latch_error(DevCtl *ctl, int flag, int index) {
 // and replaced by lo, so that the access stays inside the buffer and the
 // launch completes; the host reports T7_EINDEX.  In the release build
 // (T7_CHECKED=0) chk is the identity and adds no instruction.
-#ifndef T7_CHECKED
-#define T7_CHECKED 0
-#endif
 __device__ __forceinline__ int chk(DevCtl *ctl, int i, int lo, int hi) {
 #if T7_CHECKED
     if (i < lo || i >= hi) {
@@ -3102,10 +3099,9 @@ cudaError_t launch_batch1d(const Batch1D &p, cudaStream_t st) {
 // ==========================================================================
 namespace t7 {
 
-// A CTA's slot of the exchange `tag`, and the read of all slots by one warp: waits
-// (bounded) until every slot carries the tag and returns the maximum; false when
-// it gave up.
-constexpr int RUN_SPIN_LIMIT = 1 << 21;
+// A CTA's slot of the exchange `tag`, and the read of the slots by its threads: waits
+// until every slot carries the tag and returns the maximum; false when it gave up
+// (after `limit` polls of one slot; at once with 0).
 __device__ __forceinline__ void publish_max(RunSlot *slots, unsigned tag, double v) {
     const unsigned long long b = f64_bits(v), t = (unsigned long long)tag << 32;
     asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(
@@ -3113,7 +3109,8 @@ __device__ __forceinline__ void publish_max(RunSlot *slots, unsigned tag, double
                  "l"(t | (b >> 32)), "l"(t | (b & 0xffffffffull))
                  : "memory");
 }
-__device__ __forceinline__ bool read_slots(const RunSlot *slots, unsigned tag, int first, int stride, double &v) {
+__device__ __forceinline__ bool read_slots(const RunSlot *slots, unsigned tag, int first, int stride, int limit,
+                                           double &v) {
     const RunSlot *set = slots + (tag & 1u) * RUN_MAX_CTAS;
     const unsigned long long want = (unsigned long long)tag << 32;
     bool failed = false;
@@ -3122,7 +3119,7 @@ __device__ __forceinline__ bool read_slots(const RunSlot *slots, unsigned tag, i
         int spin = 0;
         do {
             asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(&set[i]) : "memory");
-            failed = ++spin > RUN_SPIN_LIMIT;
+            failed = ++spin > limit;
         } while (!failed && (((a ^ want) | (b ^ want)) >> 32) != 0ull);
         if (!failed) v = f64_max_pos(v, f64_of((a << 32) | (b & 0xffffffffull)));
     }
@@ -3135,7 +3132,8 @@ __device__ __forceinline__ bool read_slots(const RunSlot *slots, unsigned tag, i
 // until the tags match.  Two slot sets alternate: a CTA writes a set again only
 // after every CTA has published the stage between, hence read this one.  The
 // waiting is bounded; false (for the whole CTA) when it gave up.
-__device__ __forceinline__ bool grid_max(RunSlot *slots, unsigned tag, double v, double &result, double (*s_red)[WPB]) {
+__device__ __forceinline__ bool grid_max(RunSlot *slots, unsigned tag, int limit, double v, double &result,
+                                         double (*s_red)[WPB]) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     double (*red)[WPB] = s_red + 2 * (tag & 1u);
     v = warp_max_pos(v);
@@ -3150,7 +3148,7 @@ __device__ __forceinline__ bool grid_max(RunSlot *slots, unsigned tag, double v,
         __threadfence();
         publish_max(slots, tag, v);
     }
-    const bool failed = !read_slots(slots, tag, threadIdx.x, blockDim.x, v);
+    const bool failed = !read_slots(slots, tag, threadIdx.x, blockDim.x, limit, v);
     __threadfence();
     v = warp_max_pos(v);
     if (lane == 0) red[1][warp] = v;
@@ -3219,7 +3217,11 @@ __global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 || FORM == FORM_CTA 
         if (q.cluster)
             alpha = cluster_max(tag, v, s_cl, blockIdx.x, gridDim.x);
         else
-            ok = grid_max(q.slots, tag, v, alpha, s_red);
+#if T7_CHECKED
+            ok = grid_max(q.slots, tag, (int)blockIdx.x == q.give_up ? 0 : q.spin_limit, v, alpha, s_red);
+#else
+            ok = grid_max(q.slots, tag, RUN_SPIN_LIMIT, v, alpha, s_red);
+#endif
         tag++;
     };
     __syncthreads();
@@ -3296,14 +3298,17 @@ __global__ void __launch_bounds__(WPB * 32, (sizeof(T) == 4 || FORM == FORM_CTA 
         dt = div64(cfl_dx, alpha);
         if (t + dt > t_end) dt = t_end - t;
     }
+    // A CTA that gave up leaves its part of what follows undone, which no other need
+    // notice (a right-hand side exchanges once, a step's last stage ends without an
+    // exchange): each latches.
+    if (!ok && threadIdx.x == 0) latch_error(ctl, ERR_TIMEOUT, 0);
     if (first_thread) {
-        if (!ok) latch_error(ctl, ERR_TIMEOUT, 0);
         if (march) {
             ctl->t = t;
             ctl->dt = dt;
             ctl->dt_f = (float)dt;
             ctl->steps = steps;
-            ctl->active = active;
+            ctl->active = active && ok;  // (the run's later launches return at once)
             ctl->amax[0][0] = f64_bits(alpha);
             ctl->alpha_f[0][0] = (float)alpha;
             ctl->amax[1][0] = 0ull;  // as a step's last stage leaves it
