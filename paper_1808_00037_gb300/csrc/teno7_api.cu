@@ -9,7 +9,9 @@
 #include <string.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
+#include <mutex>
 #include <new>
 #include <numeric>
 #include <vector>
@@ -58,6 +60,9 @@ struct t7_ctx {
     cudaStream_t cstream;
     cudaEvent_t c_ev[8], c_done;
     cudaEvent_t sw_ev;     // t7_set_stream: orders the new stream after the old one
+    cudaEvent_t r_ev[2];   // ends of t7_run's last two chunks (run_ahead)
+    t7_ctx *use_prev, *use_next;  // the device's live contexts (DeviceUse) ...
+    cudaStream_t use_stream;      // ... and the stream this one is listed with
     char err[512];
 };
 
@@ -221,6 +226,61 @@ t7::Run1D run_params(t7_ctx *c, int mode, const void *U, void *out) {
     return q;
 }
 
+// What else a device is used for.  The CTAs of a one-launch grid have to be resident
+// together, so that grids which fill much of the chip run one after another, where
+// stage launches of several streams fill each other's gaps.  us per step and context,
+// t7_run of FP32 Euler on 1 / 2 / 4 / 16 threads and streams:
+//                           one launch                   stage launches
+//   10,000 cells   14.4 /  7.6 /  4.7 /  3.0    23.8 / 12.6 /  6.1 / 3.9
+//   20,000         17.1 /  9.6 /  6.8 /  6.2    20.7 / 11.3 /  6.6 / 4.0
+//   34,000         17.0 / 10.8 / 10.9 / 10.0    23.9 / 12.6 /  6.7 / 4.7
+//   100,003        25.8 / 26.5 / 25.8 / 25.5    25.8 / 14.0 / 10.4 / 9.9
+// (FP64 8000 43.5 / 42.0 / 41.4 / 40.6 and 45.5 / 28.8 / 27.0 / 26.6), and us per
+// right-hand side from 1 / 2 / 4 / 16 streams: 50,000 cells 10.5 / 6.4 / 4.2 / 4.1 and
+// 15.5 / 8.3 / 5.4 / 5.4, 100,003 14.2 / 9.8 / 9.6 / 9.7 and 16.4 / 8.3 / 5.4 / 5.3; per
+// step of 20,000 20.5 / 10.7 / 6.4 / 6.4 and 32 / 17 / 9.9 / 9.2, 50,000 23.6 / 14.3 /
+// 11.8 / 11.8 and 33 / 19.6 / 10.4 / 9.0.  So, where contexts are on several streams, a
+// run takes one launch while as many grids as there are runs in progress, and two, fit
+// the chip, and a call whose overlap the library cannot see (it returns before the GPU ends) where
+// two of a right-hand side's or three of a step's grids fit.  The results are the same
+// bit for bit.
+struct DeviceUse {
+    std::mutex mu;
+    t7_ctx *first = nullptr;           // the live contexts
+    std::atomic<bool> streams{false};  // they are on more than one stream
+    std::atomic<int> runs{0};          // t7_run and t7_run_host calls in progress
+};
+DeviceUse g_use[64];
+DeviceUse &use_of(const t7_ctx *c) { return g_use[c->device & 63]; }
+
+// Enters a context into its device's list (again, after a change of its stream), or
+// removes it.
+void use_list(t7_ctx *c, bool live) {
+    DeviceUse &use = use_of(c);
+    std::lock_guard<std::mutex> lock(use.mu);
+    if (c->use_prev) c->use_prev->use_next = c->use_next;
+    else if (use.first == c) use.first = c->use_next;
+    if (c->use_next) c->use_next->use_prev = c->use_prev;
+    c->use_prev = c->use_next = nullptr;
+    if (live) {
+        c->use_stream = c->stream;
+        c->use_next = use.first;
+        if (use.first) use.first->use_prev = c;
+        use.first = c;
+    }
+    bool several = false;
+    for (const t7_ctx *q = use.first; q && !several; q = q->use_next) several = q->use_stream != use.first->use_stream;
+    use.streams = several;
+}
+
+struct RunInProgress {
+    explicit RunInProgress(t7_ctx *c) : use(use_of(c)) { use.runs++; }
+    ~RunInProgress() { use.runs--; }
+    RunInProgress(const RunInProgress &) = delete;
+    RunInProgress &operator=(const RunInProgress &) = delete;
+    DeviceUse &use;
+};
+
 // Enqueue it.  Returns false, with nothing enqueued, when the problem is not one
 // for a single launch, the stream is being captured into a graph (whose replays
 // would repeat the launch's tags), or the launch is refused.
@@ -241,6 +301,11 @@ bool run_coop(t7_ctx *c, t7::Run1D &q) {
         c->run_tag = 1;
     }
     q.tag = c->run_tag;
+    const DeviceUse &use = use_of(c);
+    q.share = !use.streams                ? 1
+              : q.mode == t7::RUN_MARCH ? std::max(2, use.runs.load())
+              : q.mode == t7::RUN_RHS   ? 2
+                                        : 3;
 #if T7_CHECKED
     q.give_up = c->probe_block;
     q.spin_limit = c->probe_limit;
@@ -440,12 +505,14 @@ t7_status t7_create(const t7_grid *g, void *stream, t7_ctx **out) {
         return T7_ECUDA;
     }
     snprintf(c->err, sizeof(c->err), "no error");
+    use_list(c, true);
     *out = c;
     return T7_OK;
 }
 
 t7_status t7_destroy(t7_ctx *c) {
     if (!c) return T7_EINVAL;
+    use_list(c, false);
     if (c->U1) cudaFree(c->U1);
     if (c->U2) cudaFree(c->U2);
     if (c->Uhost) cudaFree(c->Uhost);
@@ -471,6 +538,8 @@ t7_status t7_destroy(t7_ctx *c) {
     if (c->c_done) cudaEventDestroy(c->c_done);
     if (c->cstream) cudaStreamDestroy(c->cstream);
     if (c->sw_ev) cudaEventDestroy(c->sw_ev);
+    for (int k = 0; k < 2; k++)
+        if (c->r_ev[k]) cudaEventDestroy(c->r_ev[k]);
     delete c;
     return T7_OK;
 }
@@ -487,6 +556,7 @@ t7_status t7_set_stream(t7_ctx *c, void *stream) {
     if (e == cudaSuccess) e = cudaStreamWaitEvent(s, c->sw_ev, 0);
     if (e != cudaSuccess) return cuda_fail(c, e, "t7_set_stream: ordering the new stream after the old one");
     c->stream = s;
+    use_list(c, true);
     return T7_OK;
 }
 
@@ -796,6 +866,19 @@ static bool run_poll(t7_ctx *c, double t_end, cudaError_t *e) {
     return c->ctl_host->active && !c->ctl_host->err && c->ctl_host->t < t_end;
 }
 
+// Called after chunk `chunk` (from 0) of a run was queued: with contexts on several
+// streams, waits for the chunk before it, so that the run's later chunks take the form
+// that the runs in progress by then call for, and the GPU still has one in hand.
+static cudaError_t run_ahead(t7_ctx *c, int chunk) {
+    if (!is_1d(c->g.sys) || !use_of(c).streams) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < 2 && e == cudaSuccess; k++)
+        if (!c->r_ev[k]) e = cudaEventCreateWithFlags(&c->r_ev[k], cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(c->r_ev[chunk & 1], c->stream);
+    if (e == cudaSuccess) e = cudaEventSynchronize(c->r_ev[~chunk & 1]);  // (never recorded or an earlier run's: done)
+    return e;
+}
+
 // k steps of U in one launch (see run_coop).
 static bool run_steps_coop(t7_ctx *c, void *U, int k) {
     t7::Run1D q = run_params(c, t7::RUN_MARCH, U, U);
@@ -808,6 +891,7 @@ static bool run_steps_coop(t7_ctx *c, void *U, int k) {
 static t7_status run_core(t7_ctx *c, void *U, double cfl, double t_end, int max_steps, int *steps_out, double *t_out,
                           void *host_out) {
     t7_status st;
+    RunInProgress in_progress(c);
     cudaError_t e = t7::launch_ctl_begin(c->ctl, t_end, cfl, c->g.dx, c->g.dy, max_steps, c->stream);
     if (e != cudaSuccess) return cuda_fail(c, e, "ctl");
     e = alpha_launch(c, U);
@@ -815,8 +899,10 @@ static t7_status run_core(t7_ctx *c, void *U, double cfl, double t_end, int max_
     // Steps are launched in chunks; between chunks the host polls whether the
     // device-side clock has reached t_end (a step past it is a no-op anyway).
     const bool graphs = is_1d(c->g.sys) && c->ncell * c->m <= GRAPH_MAX_VALUES;
-    int launched = 0;
+    int launched = 0, chunk = 0;
     while (launched < max_steps) {
+        if (launched > 0 && !isfinite(t_end) && (e = run_ahead(c, chunk++)) != cudaSuccess)
+            return cuda_fail(c, e, "waiting for the chunk before last");
         int k = max_steps - launched < RUN_CHUNK ? max_steps - launched : RUN_CHUNK;
         const bool last_chunk = host_out && launched + k == max_steps;
         if (!last_chunk && run_steps_coop(c, U, k)) {

@@ -93,6 +93,7 @@ struct Run1D {
     RunSlot *slots;  // [2][RUN_MAX_CTAS]
     unsigned tag;    // tag of the launch's first exchange; 3 nsteps + 1 tags are used at most
     int cluster;     // the grid is one thread-block cluster (set by the launcher)
+    int share;       // so many such grids have to be resident at once (else it is not launched)
 #if T7_CHECKED
     int spin_limit;  // polls after which a block gives up waiting for another's slot
     int give_up;     // block that gives up at its first wait, or -1

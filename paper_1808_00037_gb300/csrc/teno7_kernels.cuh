@@ -3338,6 +3338,7 @@ cudaError_t launch_run1d_as(Run1D q, cudaStream_t st) {
     if (grid > RUN_MAX_CTAS) grid = RUN_MAX_CTAS;
     q.p = with_kt(q.p);
     q.cluster = cluster && grid > 1;
+    if (!q.cluster && grid > 1 && (long long)q.share * grid > cap) return cudaErrorNotSupported;
     void *args[] = {&q};
     if (!q.cluster) return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(nw * 32), args, 0, st);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
