@@ -271,7 +271,9 @@ t7_status t7_batch_run(t7_ctx *ctx, void *U, const int64_t *offsets, const doubl
 /* Autotuner of the batch tile shape (no counterpart in the paper; the
  * scheme is t7_batch_run's): times trial_steps steps of every tube
  * for group_warps = 1, 2, 4, 8 on a device copy of U (U is not modified),
- * keeps the fastest in the context for later t7_batch_run calls, and returns
+ * keeps one in the context for later t7_batch_run calls -- the largest whose
+ * time is below 1.02 times the shortest: fewer tubes in flight stay in L2
+ * and the longest ends sooner, which a trial does not show -- and returns
  * it in *group_out (nullable); ms_out (nullable, 4 floats) receives the trial
  * times.  Synchronises.  Trials of 10 or more steps are needed for the
  * ranking to hold over a whole run: smaller groups run more tubes at once,

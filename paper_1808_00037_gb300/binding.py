@@ -333,7 +333,8 @@ class Context:
         return steps, t
 
     def batch_autotune(self, U, offsets, dx, cfl: float, trial_steps: int = 20):
-        """Pick group_warps (warps per tube) by timing trial steps; U is not modified.
+        """Pick group_warps (warps per tube) by timing trial steps (the largest within
+        2% of the fastest); U is not modified.
         Returns (group_warps, trial milliseconds for 1, 2, 4, 8)."""
         off = np.ascontiguousarray(offsets, dtype=np.int64)
         dxa = np.ascontiguousarray(dx, dtype=np.float64)
