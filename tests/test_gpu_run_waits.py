@@ -78,6 +78,8 @@ def test_wait_that_runs_out(checked, prec, n, call, block):
     want = call(fresh, U)
     fresh.sync()
     assert torch.equal(got, want)
+    c.close()
+    fresh.close()
 
 
 @pytest.mark.parametrize("prec,n", FORMS)
@@ -87,6 +89,7 @@ def test_run_ends_where_a_wait_ran_out(checked, prec, n):
     c.probe_run_waits(1, polls=1 << 12)
     steps, t = ctypes.c_int(-1), ctypes.c_double(-1.0)
     st = c.lib.t7_run(c.h, U.data_ptr(), 0.5, math.inf, 192, ctypes.byref(steps), ctypes.byref(t))
+    c.close()
     assert (st, steps.value, t.value) == (B.T7_ETIMEOUT, 0, 0.0)
 
 

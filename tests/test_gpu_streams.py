@@ -3,6 +3,7 @@ chip beside the others' give way to launches of single stages (they would run on
 another), and the results stay the same bit for bit.  Which form a call takes shows in
 the checked build, where the waits of a one-launch form can be made to run out
 (t7_probe_run_waits) and stage launches have none."""
+import gc
 import threading
 import time
 
@@ -39,6 +40,7 @@ def waits(c, call):
 
 @pytest.fixture
 def checked(monkeypatch):
+    gc.collect()  # no context of an earlier test is left on a stream of its own
     monkeypatch.setattr(B, "_lib", B.load(build.build(checked=True)))
 
 
