@@ -54,14 +54,20 @@ FLOPS_PER_CELL_STAGE = {"f32": 808.0, "f64": 776.0}
 # Executed floating-point operations per cell per stage launch, from ncu's
 # per-opcode thread counters of launches on the same workload (FMA = 2,
 # packed f32x2 FMA = 4, packed add/mul = 2, scalar add/mul = 1; the keep-all
-# shortcut skips most of the cutoff, so this is below the algorithmic count; f64:
-# operations of the FP64 pipe only, products, quotients and roots being formed on
-# the integer and FP32 pipes), mean of the three stages on 2M (f64: 1M) cells of it;
-# None when not captured for the current kernel.
+# shortcut skips most of the cutoff, so this is below the algorithmic count), mean
+# of the three stages on 2M (f64: 1M) cells of it; None when not captured for the
+# current kernel.  The two do not count the same: f64 has the operations of the FP64
+# pipe only (EXEC_KIND).
 EXEC_FLOPS_PER_CELL_STAGE = {"f32": 588.1, "f64": 231.9}
+EXEC_KIND = {"f32": "all FP32 operations", "f64": "operations of the FP64 pipe only; products, quotients, roots and "
+             "cutoff decisions run on the integer and FP32 pipes"}
+# f64: the algorithmic rate over the FP64-pipe peak, which passes 1
+ROOFLINE_NOTE = {"f32": None, "f64": "algorithmic FLOP over the FP64-pipe peak; part of them run on other pipes, so "
+                 "frac can pass 1 and is not the distance to a limit"}
 # DRAM bytes per stage launch per cell measured by ncu (dram__bytes_read.sum +
 # dram__bytes_write.sum, averaged over the three stage launches of one RK3
-# step at N = 16,777,600) for the current kernels; None when not captured.
+# step at N = 16,777,600) for the current kernels, an instantiation per stage (f32:
+# 356.1, 572.0 and 556.5 MB); None when not captured.
 TRAFFIC_PER_CELL_LAUNCH = {"f32": 29.50, "f64": None}
 
 
@@ -798,8 +804,9 @@ def main():
                          "frac": tflops / peak_alu, "traffic": None if tr is None else tr * n,
                          "flops_per_cell_stage": FLOPS_PER_CELL_STAGE[name],
                          "flops_kind": "algorithmic (cutoff counted in full)",
-                         "executed": {"flops_per_cell_stage": ex, "achieved": ex_tflops,
+                         "executed": {"flops_per_cell_stage": ex, "kind": EXEC_KIND[name], "achieved": ex_tflops,
                                       "frac": None if ex is None else ex_tflops / peak_alu},
+                         **({"note": ROOFLINE_NOTE[name]} if ROOFLINE_NOTE[name] else {}),
                          "peak_kind": alu["kind"],
                          "nominal_peak": FP32_NOMINAL_TFLOPS if name == "f32" else FP64_NOMINAL_TFLOPS},
             "hbm": {"achieved": achieved, "peak": hbm_peak, "unit": "GB/s", "frac": achieved / hbm_peak,

@@ -212,7 +212,6 @@ cudaError_t launch_combine_f64(void *out, const void *x, const void *y, const vo
                                double c3, size_t N, cudaStream_t s);
 cudaError_t launch_combine_f32(void *out, const void *x, const void *y, const void *z, double c1, double c2,
                                double c3, size_t N, cudaStream_t s);
-// out1 = a1 x + b1 y; out2 (nullable) = a2 x + b2 y; x may be null
 
 struct Recon {
     const void *v;  // n + 8 values

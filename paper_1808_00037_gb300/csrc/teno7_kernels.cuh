@@ -125,9 +125,9 @@ __device__ __forceinline__ T coef(int idx) {
 }
 
 // keep_all_factor of the FP32 1D tiles, evaluated in the kernel: with kt taken
-// from the launch parameters instead, the compiler if-converts the cutoff's slow
-// path and the 16.8M-cell stage executes 29% more instructions (1.06 -> 1.34 ms
-// per step); the powf costs a launch about a microsecond.
+// from the launch parameters instead, the 16.8M-cell stage executes 29% more
+// instructions (ncu; 1.06 -> 1.34 ms per step), for a reason not established; the
+// powf costs a launch about a microsecond.
 __device__ __forceinline__ float keep_all_factor_device(float CT) {
     return (CT > 0.f && CT < 1.f / 3.f) ? 0.9f * powf(3.f * CT, -1.f / 6.f) - 1.f : 0.f;
 }
@@ -3358,17 +3358,21 @@ cudaError_t launch_run1d_as(Run1D q, cudaStream_t st) {
 
 // The form for a problem, or cudaErrorNotSupported where launches of single
 // stages are as fast or faster.  us per step of t7_run, single launches / one
-// launch:
+// launch (one stream; several: DeviceUse, teno7_api.cu):
 //   FP64 Euler, one tile per CTA (SPLIT_TILES), else per warp up to eight per SM:
-//     30,000 cells 113 / 106; a right-hand side or one step, whose CTAs would run
-//     several tiles, up to two tiles per SM (20,000 cells: 33 us / 35);
-//   FP64 scalar laws while one cluster holds them (200 cells 20 / 10, 8000 22 / 23);
-//   FP32 Euler, a warp's tiles up to eight per SM (24,000 cells 24 / 18), then
-//     paired faces up to 2^20 cells (50,000 24.2 / 22.7, 700,000 84 / 71, 1M 103 /
-//     92, 2M 159 / 157, 4M 281 / 298: there the tuned two-wave grid wins);
+//     1600 cells 38.0 / 31.2, 8000 45.5 / 40.4, 24,000 88.3 / 83.4, 30,000 114.4 /
+//     110.5; a right-hand side or one step, whose CTAs would run several tiles, up to
+//     two tiles per SM (20,000 cells: 33 us / 35);
+//   FP64 scalar laws while one cluster holds them (200 cells 19.4 / 9.7, 3700 20.0 /
+//     12.4, 8000 22 / 23);
+//   FP32 Euler, a warp's tiles up to eight per SM (1600 cells 19.2 / 8.5, 24,000 22.4 /
+//     15.5, 34,000 22.4 / 17.9), then paired faces up to 2^20 cells (50,000 22.0 /
+//     18.7, 100,003 23.7 / 24.5, 300,000 45.7 / 41.2, 700,000 77.4 / 70.1, 1M 95.7 /
+//     90.9; with the stages of one kernel 2M took 159 / 157, 4M 281 / 298: there the
+//     tuned two-wave grid wins);
 //   FP32 scalar laws, a warp's tiles up to two per SM, then paired faces up to
-//     seven (Burgers 24,000 16.4 / 15.0, 50,000 16.1 / 16.1, 100,000 17.9 / 21.9);
-//   mixed Euler up to eight tiles per SM, scalar laws up to two.
+//     seven (Burgers 24,000 15.2 / 12.9, 50,000 (stage launches) 15.6, 100,000 17.9 / 21.9);
+//   mixed Euler up to eight tiles per SM (24,000 21.5 / 18.9), scalar laws up to two.
 // Advection's right-hand side needs no alpha pass, and one plain launch is the
 // cheaper one for the host (8.4 / 10.5).
 template <typename T, typename S, int SYS, int SCH>

@@ -623,10 +623,7 @@ __device__ __forceinline__ void cell2d_f32(const float U[4], float gm1, float al
     }
 }
 
-// One face along DIR: frame, per-field projection / cutoff / Delta / polynomial,
-// back-projection to the physical face flux fh[4].  pr(q, i), gp(c, i),
-// gm(c, i) read staged index i (face j+1/2 <-> cells j-3+t at index lane+t).
-// codes_p / codes_m receive the four fields' Delta codes (5 bits each).
+// Table co2 row 0 of two windows.
 __device__ __forceinline__ float2 poly_f0_pair(const float2 P[7]) {
     float2 v = __fmul2_rn(f2(-1.f / 140.f), P[0]);
     v = __ffma2_rn(f2(5.f / 84.f), P[1], v);
@@ -637,6 +634,10 @@ __device__ __forceinline__ float2 poly_f0_pair(const float2 P[7]) {
     return __ffma2_rn(f2(1.f / 105.f), P[6], v);
 }
 
+// One face along DIR: frame, per-field projection / cutoff / Delta / polynomial,
+// back-projection to the physical face flux fh[4].  pr(q, i), gp(c, i),
+// gm(c, i) read staged index i (face j+1/2 <-> cells j-3+t at index lane+t).
+// codes_p / codes_m receive the four fields' Delta codes (5 bits each).
 // VOTE: a warp whose windows all keep every stencil skips the exchange.  Not in the mixed
 // y sweep: its latency shows on small grids (60 x 50, 64 steps 6.22 ->
 // 5.96 ms; 200 x 170, 29 steps 2.89 -> 2.80) against 0.7% at 2048^2.
